@@ -349,7 +349,9 @@ int hotrg_isometry(hotrg_ctx* ctx, int leg, double* U, int64_t cap, int* rows,
  * lattice axis `leg` in the last step (Sec. 4.2.5); *n = chi_leg^2. */
 int hotrg_spectrum(hotrg_ctx* ctx, int leg, int prime, double* lam, int64_t cap, int* n);
 
-/* FP64 one-sided Jacobi sweeps used for lattice axis `leg` in the last step. */
+/* Iterations of the eigen-solver for lattice axis `leg` in the last step: FP64
+ * one-sided Jacobi sweeps (blocks of up to 20 rows), else one more than the most QR
+ * iterations an eigenvalue of a leaf of the divide and conquer took. */
 int hotrg_jacobi_sweeps(hotrg_ctx* ctx, int leg, int* sweeps);
 
 /* Discarded sums epsilon^(j), epsilon'^(j) of the last step (Sec. 2). */

@@ -180,10 +180,10 @@ struct hotrg_ctx {
   // buffers
   Buf Za, Zb, Zc, Zmap;   // Z2 blocks of the contraction operands, index maps
   Buf Zg;                 // Z2 index maps of the environment Grams and the eigen blocks
-  Buf Eb;                 // Z2 blocks of A, W, V for the eigen-solver
-  Buf T, T2, Xp, parts, S, Amat, W, V, lam, U64, U32, legres, Y, state, counters, sweeps;
+  Buf Eb;                 // the eigen-solver's batch: blocks of A, their eigenvectors and eigenvalues
+  Buf T, T2, Xp, parts, S, Amat, V, lam, U64, U32, legres, Y, state, counters, sweeps;
   Buf Ap, Bp, Cb, chA, chB;
-  Buf J32, Gns, Vtmp;   // eigen-solver warm start
+  Buf Ew, lraw, selw;   // eigen-solver workspace, its eigenvalues, scratch of the selection
   // d/d beta carried with T in forward mode (Ising runs; FP64 dense form while on):
   // dT in the slot layout of T, its trace bookkeeping in tstate
   int tangent = 0;
@@ -350,14 +350,6 @@ void* pinned_stage(hotrg_ctx* c, size_t bytes) {
   }
   return c->hpin;
 }
-
-// Jacobi grid-barrier counters: 3 per matrix of one launch (up to 4 (d - 1) parity
-// blocks), then 3 for the FP32 warm start
-constexpr int kCounters32 = 3 * 4 * kMaxD;
-// the FP64 eigen-solver's per-matrix largest squared column norm (16 x 64 bits) after
-// the rotation counters of both solvers
-constexpr int kColmaxOff = kCounters32 + 4;
-constexpr int kCounterInts = kColmaxOff + 2 * 16;
 
 int num_sms() { return sm_count(); }
 
@@ -671,10 +663,10 @@ int hotrg_set_allocator(hotrg_ctx* c, hotrg_alloc_fn alloc, hotrg_free_fn free_f
       return cuda_status(c);
   }
   int n = 0;
-  Buf* b[] = {&c->T,  &c->T2, &c->Xp,     &c->parts, &c->S,     &c->Amat,     &c->W,
+  Buf* b[] = {&c->T,  &c->T2, &c->Xp,     &c->parts, &c->S,     &c->Amat,
               &c->V,  &c->lam, &c->U64,   &c->U32,   &c->legres, &c->Y,       &c->state,
               &c->counters, &c->sweeps, &c->Ap, &c->Bp, &c->Cb, &c->chA, &c->chB,
-              &c->J32,  &c->Gns, &c->Vtmp, &c->Za, &c->Zb, &c->Zc, &c->Zmap, &c->Zg, &c->Eb,
+              &c->Ew, &c->lraw, &c->selw, &c->Za, &c->Zb, &c->Zc, &c->Zmap, &c->Zg, &c->Eb,
               &c->dT, &c->dT2, &c->dTb, &c->dXp, &c->dS, &c->dA, &c->dU64, &c->eG, &c->eZ, &c->eZt,
               &c->rank, &c->Yd, &c->tstate, &c->dchA, &c->dchB, &c->dchT, &c->dBp, &c->tBp, &c->dCb,
               &c->tCb, &c->dAp, &c->dB64, &c->dU32, &c->d2T, &c->d2T2, &c->d2Tb, &c->d2Tc, &c->d2Xp,
@@ -819,49 +811,15 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
   }
 
   // ---- environments (Sec. 3.2; Sec. 4.2.4), FP64
-  // legs grouped by n = chi_j^2 so that one Jacobi launch covers a group
   const int nlegs = d - 1;
-  int grp_of[kMaxD], grp_n[kMaxD], grp_first_mat[kMaxD], ngrp = 0, mat_of_leg[kMaxD];
-  {
-    int nmat_acc = 0;
-    for (int j = 1; j < d; ++j) {
-      int n = chij[j] * chij[j];
-      int g = -1;
-      for (int q = 0; q < ngrp; ++q)
-        if (grp_n[q] == n) g = q;
-      if (g < 0) {
-        g = ngrp++;
-        grp_n[g] = n;
-      }
-      grp_of[j] = g;
-    }
-    // matrices laid out group by group, two per leg (A, A')
-    for (int g = 0; g < ngrp; ++g) {
-      grp_first_mat[g] = nmat_acc;
-      for (int j = 1; j < d; ++j)
-        if (grp_of[j] == g) {
-          mat_of_leg[j] = nmat_acc;
-          nmat_acc += 2;
-        }
-    }
-  }
-  // matrix element offsets: group base + local index * n^2
+  // element offsets of A^(j), A'^(j) (and their eigenvectors): leg by leg
   long long mat_elem_off[2 * kMaxD];
   long long total_mat_elems = 0;
-  {
-    for (int g = 0; g < ngrp; ++g) {
-      int cnt = 0;
-      for (int j = 1; j < d; ++j)
-        if (grp_of[j] == g) cnt += 2;
-      for (int j = 1; j < d; ++j)
-        if (grp_of[j] == g) {
-          int local = mat_of_leg[j] - grp_first_mat[g];
-          mat_elem_off[2 * j] = total_mat_elems + (long long)local * grp_n[g] * grp_n[g];
-          mat_elem_off[2 * j + 1] = mat_elem_off[2 * j] + (long long)grp_n[g] * grp_n[g];
-        }
-      total_mat_elems += (long long)cnt * grp_n[g] * grp_n[g];
+  for (int j = 1; j < d; ++j)
+    for (int k = 0; k < 2; ++k) {
+      mat_elem_off[2 * j + k] = total_mat_elems;
+      total_mat_elems += (long long)chij[j] * chij[j] * chij[j] * chij[j];
     }
-  }
   long long mmax = 0, nmax = 0;
   for (int j = 1; j < d; ++j) {
     mmax = std::max<long long>(mmax, (long long)chij[j] * chi_c);
@@ -899,12 +857,8 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
   CHECK_ALLOC(dev_alloc(c, c->parts, sizeof(double) * nsplit_max * mmax * mmax));
   CHECK_ALLOC(dev_alloc(c, c->S, sizeof(double) * 4 * nlegs * mmax * mmax));
   CHECK_ALLOC(dev_alloc(c, c->Amat, sizeof(double) * total_mat_elems));
-  CHECK_ALLOC(dev_alloc(c, c->W, sizeof(double) * total_mat_elems));
   CHECK_ALLOC(dev_alloc(c, c->V, sizeof(double) * total_mat_elems));
-  CHECK_ALLOC(dev_alloc(c, c->J32, sizeof(float) * 2 * total_mat_elems));
-  CHECK_ALLOC(dev_alloc(c, c->Gns, sizeof(double) * total_mat_elems));
-  CHECK_ALLOC(dev_alloc(c, c->Vtmp, sizeof(double) * total_mat_elems));
-  CHECK_ALLOC(dev_alloc(c, c->counters, sizeof(int) * kCounterInts));
+  CHECK_ALLOC(dev_alloc(c, c->selw, sizeof(int) * 5 * nmax));
   CHECK_ALLOC(dev_alloc(c, c->sweeps, sizeof(int) * 6 * kMaxD));
 
   // Gram of leg j, kind: X = T with the free pair (n_j or n'_j, c' or c) first, rest after
@@ -1136,124 +1090,74 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
   }
 
   if (pending_error(c, "the environments") != HOTRG_OK) return HOTRG_ECUDA;
-  // ---- eigen-decomposition (Sec. 4.2.5), batched over matrices of equal size
-  auto eig_batch = [&](const double* Ag, double* Wg, double* Vg, int n, int cnt, int* sweeps_out) -> int {
-    const long long nn = (long long)n * n;
-    const double* Ainit = Ag;
-    if (n >= 32) {
-      Phase phw(c, 9);
-      // FP32 warm start, FP64 re-orthonormalisation of its vectors (two Newton-Schulz
-      // steps Q <- Q (3I - Q^T Q) / 2), W = A Q; the FP64 sweeps then start from (W, Q)
-      float* W32 = (float*)c->J32.p;
-      float* V32 = W32 + cnt * nn;
-      double* G = (double*)c->Gns.p;
-      double* Vt = (double*)c->Vtmp.p;
-      int ok32;
-      {
-        Phase ph32(c, 10);
-        // at most 15 FP32 sweeps: on 3D chi = 16 (steps 9-28) a cap of 15 against 30 leaves the
-        // FP64 sweeps nearly unchanged and saves ~1 ms per step; 10 or 6 cost more FP64 sweeps
-        ok32 = launch_jacobi32_block(Ag, W32, V32, n, cnt, 15, (int*)c->counters.p + kCounters32, s) == 0;
-        if (!ok32) cudaGetLastError();
-      }
-      if (ok32) {
-        launch_widen_f32(V32, Vg, cnt * nn, s);
-        for (int it = 0; it < 2; ++it) {
-          launch_gemm_nt_f64_batched(Vg, n, Vg, n, G, n, n, n, n, cnt, nn, nn, nn, s);
-          launch_ns_coeff(G, n, cnt, s);
-          launch_gemm_nn_f64(G, n, Vg, n, Vt, n, n, n, n, cnt, nn, nn, nn, s);
-          cudaMemcpyAsync(Vg, Vt, sizeof(double) * cnt * nn, cudaMemcpyDeviceToDevice, s);
-        }
-        launch_gemm_nt_f64_batched(Vg, n, Ag, n, Wg, n, n, n, n, cnt, nn, nn, nn, s);
-        Ainit = nullptr;
-      }
-    }
-    return launch_jacobi(Wg, Vg, Ainit, n, cnt, 60, (int*)c->counters.p,
-                         (unsigned long long*)((int*)c->counters.p + kColmaxOff), sweeps_out,
-                         (DevState*)c->state.p, s);
-  };
-  if (!env_phase) {
-    // PH_CONTRACT / PH_FINISH: the isometries were installed by PH_ISO
-  } else if (!z2g) {
-    for (int g = 0; g < ngrp; ++g) {
-      Phase ph(c, 2);
-      int cnt = 0;
-      long long base = -1;
-      for (int j = 1; j < d; ++j)
-        if (grp_of[j] == g) {
-          cnt += 2;
-          if (base < 0 || mat_elem_off[2 * j] < base) base = mat_elem_off[2 * j];
-        }
-      if (eig_batch((const double*)c->Amat.p + base, (double*)c->W.p + base, (double*)c->V.p + base,
-                    grp_n[g], cnt, (int*)c->sweeps.p + grp_first_mat[g]) != 0)
-        return launch_failed(c, "Jacobi", grp_n[g], cnt, 0);
-    }
-  } else {
-    // A^(j), A'^(j) are block diagonal in the parity of (hat, check): gather the blocks
-    // (both blocks of a leg zero-padded to the larger, so that one launch decomposes
-    // them), decompose each size group, scatter W and V back (zeros between parities)
-    Phase ph(c, 2);
-    const int* zi = (const int*)((const long long*)c->Zg.p + gz_n64);
-    long long boff[kMaxD][2][2];
-    int bidx[kMaxD][2][2], npad[kMaxD];
-    std::vector<int> sizes;
+  // ---- eigen-decomposition (Sec. 4.2.5): every matrix of the step in one batch.  With known
+  // parities A^(j), A'^(j) are block diagonal in the parity of (hat, check): their blocks are
+  // gathered and decomposed on their own, and V is scattered back (zeros between parities).
+  // PH_CONTRACT / PH_FINISH: the isometries were installed by PH_ISO
+  long long lraw_off[kMaxD], lraw_n = 0;
+  {
+    long long o = 0;
     for (int j = 1; j < d; ++j) {
-      npad[j] = std::max(eig_nb[j][0], eig_nb[j][1]);
-      if (std::find(sizes.begin(), sizes.end(), npad[j]) == sizes.end()) sizes.push_back(npad[j]);
+      lraw_off[j] = o;
+      o += 2LL * chij[j] * chij[j];
     }
-    long long eoff = 0;
-    int nblk = 0;
-    std::vector<std::pair<long long, int>> grp_first(sizes.size());   // element offset, block index
-    std::vector<int> grp_cnt(sizes.size(), 0);
-    for (size_t g = 0; g < sizes.size(); ++g) {
-      grp_first[g] = {eoff, nblk};
-      for (int j = 1; j < d; ++j)
-        for (int k = 0; k < 2; ++k)
-          for (int b = 0; b < 2; ++b)
-            if (eig_nb[j][b] > 0 && npad[j] == sizes[g]) {
-              boff[j][k][b] = eoff;
-              bidx[j][k][b] = nblk++;
-              eoff += (long long)sizes[g] * sizes[g];
-              ++grp_cnt[g];
-            }
-    }
-    CHECK_ALLOC(dev_alloc(c, c->Eb, sizeof(double) * 3 * std::max<long long>(eoff, 1)));
-    // the warm start's scratch holds one size group: padded blocks can outgrow the dense
-    // matrices (4 npad^2 > 2 n^2 when one parity holds more than 0.707 of a leg's states)
-    CHECK_ALLOC(dev_alloc(c, c->J32, sizeof(float) * 2 * std::max<long long>(eoff, 1)));
-    CHECK_ALLOC(dev_alloc(c, c->Gns, sizeof(double) * std::max<long long>(eoff, 1)));
-    CHECK_ALLOC(dev_alloc(c, c->Vtmp, sizeof(double) * std::max<long long>(eoff, 1)));
+    lraw_n = o;
+    CHECK_ALLOC(dev_alloc(c, c->lraw, (sizeof(double) + sizeof(int)) * o));
+  }
+  int* craw = (int*)((double*)c->lraw.p + lraw_n);   // the vectors' classes, after the eigenvalues
+  if (env_phase) {
+    Phase ph(c, 2);
+    const int* zi = z2g ? (const int*)((const long long*)c->Zg.p + gz_n64) : nullptr;
+    if (!z2g)
+      for (int j = 1; j < d; ++j) {
+        eig_nb[j][0] = chij[j] * chij[j];
+        eig_nb[j][1] = 0;
+      }
+    int ld = 1, nblk = 0, na[4 * kMaxD], keep[4 * kMaxD], bidx[kMaxD][2][2];
+    for (int j = 1; j < d; ++j)
+      for (int k = 0; k < 2; ++k)
+        for (int b = 0; b < 2; ++b) {
+          bidx[j][k][b] = -1;
+          if (eig_nb[j][b] == 0) continue;
+          bidx[j][k][b] = nblk;
+          keep[nblk] = nnew[j];
+          na[nblk++] = eig_nb[j][b];
+          ld = std::max(ld, eig_nb[j][b]);
+        }
+    const long long bb = (long long)ld * ld;
+    CHECK_ALLOC(dev_alloc(c, c->Eb, (sizeof(double) * (2 * bb + ld) + sizeof(int) * 2 * ld) * nblk));
+    CHECK_ALLOC(dev_alloc(c, c->Ew, eig_workspace_bytes(ld, nblk)));
     double* Ab = (double*)c->Eb.p;
-    double* Wb = Ab + eoff;
-    double* Vb = Wb + eoff;
+    double* Vb = Ab + bb * nblk;
+    double* lb = Vb + bb * nblk;
+    int* swp = (int*)(lb + (long long)ld * nblk);
+    int* cb = swp + (long long)ld * nblk;
+    int* swb = (int*)c->sweeps.p + 2 * kMaxD;
     for (int j = 1; j < d; ++j)
       for (int k = 0; k < 2; ++k)
         for (int b = 0; b < 2; ++b)
-          if (eig_nb[j][b] > 0)
-            launch_z2_gather_sym((const double*)c->Amat.p + mat_elem_off[2 * j + k], chij[j] * chij[j],
-                                 zi + gz_eig[j] + (b == 0 ? 0 : eig_nb[j][0]), eig_nb[j][b], npad[j],
-                                 Ab + boff[j][k][b], s);
-    int* swb = (int*)c->sweeps.p + 2 * kMaxD;
-    for (size_t g = 0; g < sizes.size(); ++g) {
-      const long long o = grp_first[g].first;
-      if (eig_batch(Ab + o, Wb + o, Vb + o, sizes[g], grp_cnt[g], swb + grp_first[g].second) != 0)
-        return launch_failed(c, "Jacobi (Z2 blocks)", sizes[g], grp_cnt[g], 0);
-    }
+          if (bidx[j][k][b] >= 0)
+            launch_z2_gather_sym((const double*)c->Amat.p + mat_elem_off[2 * j + k], chij[j],
+                                 z2g ? zi + gz_eig[j] + (b == 0 ? 0 : eig_nb[j][0]) : nullptr,
+                                 z2g ? zi + gz_eig[j] + 2 * chij[j] * chij[j] : nullptr, eig_nb[j][b], ld,
+                                 Ab + bb * bidx[j][k][b], swp + ld * bidx[j][k][b], s);
+    if (launch_eig(Ab, ld, nblk, na, keep, swp, c->Ew.p, Vb, lb, cb, swb, (DevState*)c->state.p, s) != 0)
+      return launch_failed(c, "eigen-solver", ld, nblk, 0);
     SweepMerge sm;
     sm.n = 2 * (d - 1);
     for (int j = 1; j < d; ++j) {
       const int n = chij[j] * chij[j];
-      const int* eb = zi + gz_eig[j] + n;
+      const int* eb = z2g ? zi + gz_eig[j] + n : nullptr;
       for (int k = 0; k < 2; ++k) {
-        const int mat = mat_of_leg[j] + k;
-        sm.a[mat] = eig_nb[j][0] > 0 ? bidx[j][k][0] : -1;
-        sm.b[mat] = eig_nb[j][1] > 0 ? bidx[j][k][1] : -1;
-        const double* w0 = eig_nb[j][0] > 0 ? Wb + boff[j][k][0] : nullptr;
-        const double* w1 = eig_nb[j][1] > 0 ? Wb + boff[j][k][1] : nullptr;
-        const double* v0 = eig_nb[j][0] > 0 ? Vb + boff[j][k][0] : nullptr;
-        const double* v1 = eig_nb[j][1] > 0 ? Vb + boff[j][k][1] : nullptr;
-        launch_z2_scatter_eig(w0, w1, npad[j], eb, eb + n, n, (double*)c->W.p + mat_elem_off[2 * j + k], s);
-        launch_z2_scatter_eig(v0, v1, npad[j], eb, eb + n, n, (double*)c->V.p + mat_elem_off[2 * j + k], s);
+        const int mat = 2 * (j - 1) + k, i0 = bidx[j][k][0], i1 = bidx[j][k][1];
+        sm.a[mat] = i0;
+        sm.b[mat] = i1;
+        launch_z2_scatter_eig(i0 >= 0 ? Vb + bb * i0 : nullptr, i1 >= 0 ? Vb + bb * i1 : nullptr,
+                              i0 >= 0 ? lb + (long long)ld * i0 : nullptr, i1 >= 0 ? lb + (long long)ld * i1 : nullptr,
+                              i0 >= 0 ? cb + (long long)ld * i0 : nullptr, i1 >= 0 ? cb + (long long)ld * i1 : nullptr,
+                              ld, eb, eb ? eb + n : nullptr, n, (double*)c->V.p + mat_elem_off[2 * j + k],
+                              (double*)c->lraw.p + lraw_off[j] + (long long)k * n, craw + lraw_off[j] + (long long)k * n,
+                              s);
       }
     }
     launch_z2_merge_sweeps(swb, sm, (int*)c->sweeps.p, s);
@@ -1278,15 +1182,14 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
     rank_off[j] = rank_total;
     rank_total += (long long)chij[j] * chij[j];
   }
-  if (tangent) CHECK_ALLOC(dev_alloc(c, c->rank, sizeof(int) * rank_total));
+  if (tangent) CHECK_ALLOC(dev_alloc(c, c->rank, sizeof(int) * 2 * rank_total));
   for (int j = 1; j < d && env_phase; ++j) {
     Phase ph(c, 3);
-    int n = chij[j] * chij[j];
-    // select_kernel addresses matrices 2*leg_index, 2*leg_index+1 from a base
-    launch_select((const double*)c->W.p + mat_elem_off[2 * j], (const double*)c->V.p + mat_elem_off[2 * j],
-                  n, 0, nnew[j], (double*)c->lam.p + lam_off[j], (double*)c->U64.p + u_off[j],
-                  (float*)c->U32.p + u_off[j], (LegResult*)c->legres.p + j,
-                  (int*)c->sweeps.p + mat_of_leg[j], s, tangent ? (int*)c->rank.p + rank_off[j] : nullptr);
+    launch_select((const double*)c->lraw.p + lraw_off[j], (const double*)c->V.p + mat_elem_off[2 * j],
+                  chij[j] * chij[j], nnew[j], (double*)c->lam.p + lam_off[j], (double*)c->U64.p + u_off[j],
+                  (float*)c->U32.p + u_off[j], (LegResult*)c->legres.p + j, (int*)c->sweeps.p + 2 * (j - 1),
+                  (int*)c->selw.p, s, craw + lraw_off[j], tangent ? (int*)c->rank.p + rank_off[j] : nullptr,
+                  tangent ? (int*)c->rank.p + rank_total + rank_off[j] : nullptr);
   }
 
   if (pending_error(c, "the selection") != HOTRG_OK) return HOTRG_ECUDA;
@@ -1445,7 +1348,8 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
       launch_gemm_nn_f64(dAs, n, (const double*)c->U64.p + u_off[j], nn, G, nn, n, nn, n, 1, 0, 0, 0, s);
       launch_gemm_nn_f64(Vs, n, G, nn, (double*)c->eZ.p, nn, n, nn, n, 1, 0, 0, 0, s);    // v_i . dA u_k
       launch_eig_dscale((const double*)c->eZ.p, (const double*)c->lam.p + lam_off[j] + (long long)side * n,
-                        (const int*)c->rank.p + rank_off[j], n, nn, fp64 ? 1e-12 : 1e-8, (double*)c->eZt.p,
+                        (const int*)c->rank.p + rank_off[j], (const int*)c->rank.p + rank_total + rank_off[j], n, nn,
+                        fp64 ? 1e-12 : 1e-8, (double*)c->eZt.p,
                         tst, s);
       launch_gemm_nn_f64((const double*)c->eZt.p, n, Vs, n, G, n, nn, n, n, 1, 0, 0, 0, s);   // dU^T
       launch_transpose(G, nn, n, (double*)c->dU64.p + u_off[j], s);
@@ -1463,7 +1367,8 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
         launch_gemm_nn_f64(Vs, n, G, nn, (double*)c->eZ2.p, nn, n, nn, n, 1, 0, 0, 0, s);    // v_i . d2A u_k
         launch_eig_d2((const double*)c->eG1.p, (const double*)c->eZ.p, (const double*)c->eZ2.p,
                       (const double*)c->lam.p + lam_off[j] + (long long)side * n,
-                      (const int*)c->rank.p + rank_off[j], n, nn, 1e-12, (double*)c->eZ2t.p, s);
+                      (const int*)c->rank.p + rank_off[j], (const int*)c->rank.p + rank_total + rank_off[j], n, nn, 1e-12,
+                      (double*)c->eZ2t.p, s);
         launch_gemm_nn_f64((const double*)c->eZ2t.p, n, Vs, n, G, n, nn, n, n, 1, 0, 0, 0, s);   // d2U^T
         launch_transpose(G, nn, n, (double*)c->d2U64.p + u_off[j], s);
       }
@@ -2611,7 +2516,7 @@ int hotrg_set_parity(hotrg_ctx* c, const int* parity) {
     sl.mask[k] = 0;
     for (int v = 0; v < c->chis[ax]; ++v) sl.mask[k] |= (unsigned)par[ax][v] << v;
   }
-  CHECK_ALLOC(dev_alloc(c, c->counters, sizeof(int) * kCounterInts));
+  CHECK_ALLOC(dev_alloc(c, c->counters, sizeof(int)));
   int* cnt = (int*)c->counters.p;
   int bad = 0;
   cudaMemsetAsync(cnt, 0, sizeof(int), c->stream);
@@ -2797,10 +2702,10 @@ void hotrg_free(hotrg_ctx* c) {
   if (!c) return;
   cudaStreamSynchronize(c->stream);
   cudaGetLastError();
-  Buf* b[] = {&c->T,  &c->T2, &c->Xp,     &c->parts, &c->S,     &c->Amat,     &c->W,
+  Buf* b[] = {&c->T,  &c->T2, &c->Xp,     &c->parts, &c->S,     &c->Amat,
               &c->V,  &c->lam, &c->U64,   &c->U32,   &c->legres, &c->Y,       &c->state,
               &c->counters, &c->sweeps, &c->Ap, &c->Bp, &c->Cb, &c->chA, &c->chB,
-              &c->J32,  &c->Gns, &c->Vtmp, &c->Za, &c->Zb, &c->Zc, &c->Zmap, &c->Zg, &c->Eb,
+              &c->Ew, &c->lraw, &c->selw, &c->Za, &c->Zb, &c->Zc, &c->Zmap, &c->Zg, &c->Eb,
               &c->dT, &c->dT2, &c->dTb, &c->dXp, &c->dS, &c->dA, &c->dU64, &c->eG, &c->eZ, &c->eZt,
               &c->rank, &c->Yd, &c->tstate, &c->dchA, &c->dchB, &c->dchT, &c->dBp, &c->tBp, &c->dCb,
               &c->tCb, &c->dAp, &c->dB64, &c->dU32, &c->d2T, &c->d2T2, &c->d2Tb, &c->d2Tc, &c->d2Xp,

@@ -45,7 +45,7 @@ struct LegResult {
   double lam1[2];
   double gap;
   int chose_prime;
-  int sweeps[2];
+  int sweeps[2];       // iterations of the eigen-solver
 };
 
 // Generic strided description of a tensor-times-isometry stage: every
@@ -166,23 +166,21 @@ void launch_assemble_a(const double* s_hat, const double* s_chk, int chi_j, int 
                        double* A, cudaStream_t s);
 
 // ---- kernels_eig.cu
-// colmax: nmat (<= 16) words of scratch
-int launch_jacobi(double* W, double* V, const double* A, int n, int nmat, int max_sweeps,
-                  int* counters, unsigned long long* colmax, int* sweeps_out, DevState* st,
-                  cudaStream_t s);
-int launch_jacobi32_block(const double* A, float* W32, float* V32, int n, int nmat,
-                          int max_sweeps, int* counters, cudaStream_t s);
-void launch_widen_f32(const float* in, double* out, long long n, cudaStream_t s);
-void launch_ns_coeff(double* G, int n, int nmat, cudaStream_t s);
+// Eigen-decomposition of nmat (<= 16) symmetric matrices of orders na[] <= n <= 1024, leading
+// dimension n: eigenvectors in the rows of V, eigenvalues in lam, an iteration count per matrix;
+// keep[]: the leading eigenvectors that may be kept; swp [nmat][n]: the partner of every index
+// under the exchange of hat and check; cls [nmat][n]: vectors that are even and odd under it have
+// opposite nonzero values
+size_t eig_workspace_bytes(int n, int nmat);
+int launch_eig(const double* A, int n, int nmat, const int* na, const int* keep, const int* swp, void* work, double* V,
+               double* lam, int* cls, int* iters, DevState* st, cudaStream_t s);
 void launch_gemm_nn_f64(const double* A, long long lda, const double* B, long long ldb, double* C,
                         long long ldc, int M, int N, int K, int batch, long long bsa,
                         long long bsb, long long bsc, cudaStream_t s);
-void launch_gemm_nt_f64_batched(const double* A, long long lda, const double* B, long long ldb,
-                                double* C, long long ldc, int M, int N, int K, int batch,
-                                long long bsa, long long bsb, long long bsc, cudaStream_t s);
-void launch_select(const double* W, const double* V, int n, int leg_index, int nnew,
-                   double* lam_sorted, double* U64, float* U32, LegResult* res,
-                   const int* sweeps, cudaStream_t s, int* rank_out = nullptr);
+// lam, V: the matrices A^(j), A'^(j) of one leg, contiguous; scratch: 5 n words
+void launch_select(const double* lam, const double* V, int n, int nnew, double* lam_sorted, double* U64, float* U32,
+                   LegResult* res, const int* sweeps, int* scratch, cudaStream_t s, const int* cls = nullptr,
+                   int* rank_out = nullptr, int* cls_out = nullptr);
 
 // ---- kernels_chain.cu
 void launch_chain_f32(const ChainDesc& d, const void* in, int in_is_f64, const float* U,
@@ -247,10 +245,11 @@ struct SweepMerge {
   int n;
   int a[2 * kMaxD], b[2 * kMaxD];
 };
-void launch_z2_gather_sym(const double* A, int n, const int* rows, int nb, int npad, double* Ab,
-                          cudaStream_t s);
-void launch_z2_scatter_eig(const double* m0, const double* m1, int ld, const int* blk, const int* pos,
-                           int n, double* M, cudaStream_t s);
+void launch_z2_gather_sym(const double* A, int chi, const int* rows, const int* pos, int nb, int npad, double* Ab,
+                          int* swp, cudaStream_t s);
+void launch_z2_scatter_eig(const double* m0, const double* m1, const double* l0, const double* l1,
+                           const int* c0, const int* c1, int ld, const int* blk, const int* pos, int n, double* M,
+                           double* lam, int* cls, cudaStream_t s);
 void launch_z2_merge_sweeps(const int* src, const SweepMerge& m, int* dst, cudaStream_t s);
 void launch_z2_gather_rc(const double* T, const long long* roff, int m, const long long* koff,
                          long long K, double* X, cudaStream_t s);
@@ -295,7 +294,7 @@ void launch_init_ising_dbeta(double* dT, int d, double beta, double h, cudaStrea
 void launch_sym_sum(const double* parts, int nsplit, int m, double* dS, cudaStream_t s);
 void launch_assemble_dot(const double* sh, const double* dsh, const double* sc, const double* dsc, int chi_j,
                          int chi_c, double* dA, cudaStream_t s);
-void launch_eig_dscale(const double* Z, const double* lam_sorted, const int* rank, int n, int nnew,
+void launch_eig_dscale(const double* Z, const double* lam_sorted, const int* rank, const int* cls, int n, int nnew,
                        double rel_tol, double* Zt, TanState* tst, cudaStream_t s);
 void launch_transpose(const double* in, int rows, int cols, double* out, cudaStream_t s);
 void launch_axpby(double a, const double* x, double b, double* y, long long n, cudaStream_t s);
@@ -310,7 +309,7 @@ void launch_init_ising_d2beta(double* d2T, int d, double beta, double h, cudaStr
 void launch_assemble_ddot(const double* sh, const double* dsh, const double* d2sh, const double* sc,
                           const double* dsc, const double* d2sc, int chi_j, int chi_c, double* d2A, cudaStream_t s);
 void launch_eig_d2(const double* G1, const double* Gs, const double* G2s, const double* lam_sorted, const int* rank,
-                   int n, int nnew, double rel_tol, double* Z2t, cudaStream_t s);
+                   const int* cls, int n, int nnew, double rel_tol, double* Z2t, cudaStream_t s);
 void launch_finish_tangent2(const double* Yd2, int chi_c, const DevState* st, TanState* tst, int p, int first,
                             cudaStream_t s);
 void launch_tangent2_scale(const double* d2T, const double* dT, const double* dThat, const double* That, double* out,

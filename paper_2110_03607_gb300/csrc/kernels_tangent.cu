@@ -106,9 +106,11 @@ void launch_assemble_dot(const double* sh, const double* dsh, const double* sc, 
 // opposite Z2 parity, couples with Z = 0).  rel_tol is 1e-12 with an FP64 contraction
 // and 1e-8 with the split-BF16 one, whose rounding (not symmetric under the lattice
 // symmetries) splits exactly degenerate pairs by about that much.
+__device__ __forceinline__ bool odd_pair(int a, int b) { return a != 0 && a == -b; }
+
 __global__ void eig_dscale_kernel(const double* __restrict__ Z, const double* __restrict__ lam_sorted,
-                                  const int* __restrict__ rank, int n, int nnew, double rel_tol,
-                                  double* __restrict__ Zt, TanState* tst) {
+                                  const int* __restrict__ rank, const int* __restrict__ cls, int n, int nnew,
+                                  double rel_tol, double* __restrict__ Zt, TanState* tst) {
   const double tol = rel_tol * lam_sorted[0];
   const int total = n * nnew;
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
@@ -117,7 +119,9 @@ __global__ void eig_dscale_kernel(const double* __restrict__ Z, const double* __
     double v = 0.0;
     if (ri >= nnew) {
       const double den = lam_sorted[k] - lam_sorted[ri];
-      const double z = Z[(long long)i * nnew + k];
+      // an even and an odd vector under the exchange of hat and check (cls by rank): dA has A's
+      // symmetry, so their coupling is zero, and what was computed is rounding
+      const double z = odd_pair(cls[k], cls[ri]) ? 0.0 : Z[(long long)i * nnew + k];
       if (fabs(den) > tol) v = z / den;
       else if (fabs(z) > 1e-9 * lam_sorted[0]) atomicAdd(&tst->degenerate, 1);
     }
@@ -125,9 +129,10 @@ __global__ void eig_dscale_kernel(const double* __restrict__ Z, const double* __
   }
 }
 
-void launch_eig_dscale(const double* Z, const double* lam_sorted, const int* rank, int n, int nnew,
+void launch_eig_dscale(const double* Z, const double* lam_sorted, const int* rank, const int* cls, int n, int nnew,
                        double rel_tol, double* Zt, TanState* tst, cudaStream_t s) {
-  eig_dscale_kernel<<<tgrid((long long)n * nnew), 256, 0, s>>>(Z, lam_sorted, rank, n, nnew, rel_tol, Zt, tst);
+  eig_dscale_kernel<<<tgrid((long long)n * nnew), 256, 0, s>>>(Z, lam_sorted, rank, cls, n, nnew, rel_tol, Zt,
+                                                                 tst);
   ++g_launches;
 }
 
@@ -306,7 +311,8 @@ void launch_assemble_ddot(const double* sh, const double* dsh, const double* d2s
 // A term whose kept-discarded gap is within rel_tol lam_1 is left out (no derivative there).
 __global__ void eig_d2_kernel(const double* __restrict__ G1, const double* __restrict__ Gs,
                               const double* __restrict__ G2s, const double* __restrict__ lam_sorted,
-                              const int* __restrict__ rank, int n, int nnew, double rel_tol, double* __restrict__ Z2t) {
+                              const int* __restrict__ rank, const int* __restrict__ cls, int n, int nnew,
+                              double rel_tol, double* __restrict__ Z2t) {
   const double tol = rel_tol * lam_sorted[0];
   const int total = n * nnew;
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
@@ -316,11 +322,12 @@ __global__ void eig_d2_kernel(const double* __restrict__ G1, const double* __res
     const bool ka = ra < nnew;
     const double la = lam_sorted[ra];
     double acc = 0.0;
-    if (!ka && fabs(lc - la) > tol) acc = G2s[(long long)a * nnew + k] / (lc - la);
+    if (!ka && fabs(lc - la) > tol && !odd_pair(cls[k], cls[ra])) acc = G2s[(long long)a * nnew + k] / (lc - la);
     for (int b = 0; b < n; ++b) {
       const int rb = rank[b];
       const bool kb = rb < nnew;
       if (ka && kb) continue;
+      if (odd_pair(cls[ra], cls[rb]) || odd_pair(cls[rb], cls[k])) continue;   // zero couplings
       const double lb = lam_sorted[rb];
       double w;
       if (ka) {   // a kept, b discarded
@@ -343,8 +350,8 @@ __global__ void eig_d2_kernel(const double* __restrict__ G1, const double* __res
 }
 
 void launch_eig_d2(const double* G1, const double* Gs, const double* G2s, const double* lam_sorted, const int* rank,
-                   int n, int nnew, double rel_tol, double* Z2t, cudaStream_t s) {
-  eig_d2_kernel<<<tgrid((long long)n * nnew), 256, 0, s>>>(G1, Gs, G2s, lam_sorted, rank, n, nnew, rel_tol, Z2t);
+                   const int* cls, int n, int nnew, double rel_tol, double* Z2t, cudaStream_t s) {
+  eig_d2_kernel<<<tgrid((long long)n * nnew), 256, 0, s>>>(G1, Gs, G2s, lam_sorted, rank, cls, n, nnew, rel_tol, Z2t);
   ++g_launches;
 }
 

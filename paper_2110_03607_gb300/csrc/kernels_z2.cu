@@ -277,42 +277,65 @@ void launch_z2_reduce_sum_t(const double* p0, int ns0, int m0, const double* p1,
 
 // Eigen-decomposition in parity blocks (Sec. 4.2.5): A^(j) is block diagonal in the
 // parity of its composite index (hat, check), so each block is decomposed on its own.
-// Ab[p][q] = A[rows[p]][rows[q]] for p, q < nb, zero-padded to npad x npad (a zero row and
-// column of A adds an exact zero column to W = A V that no rotation ever touches)
-__global__ void z2_gather_sym_kernel(const double* __restrict__ A, int n, const int* __restrict__ rows,
-                                     int nb, int npad, double* __restrict__ Ab) {
-  const int total = npad * npad;
+// Ab[p][q] = A[rows[p]][rows[q]] (no rows: A in order) for p, q < nb, zero up to npad x npad;
+// swp[p]: the place of the exchanged composite index, hat + check chi -> check + hat chi, which
+// has the same parity
+__global__ void z2_gather_sym_kernel(const double* __restrict__ A, int chi, const int* __restrict__ rows,
+                                     const int* __restrict__ pos, int nb, int npad, double* __restrict__ Ab,
+                                     int* __restrict__ swp) {
+  const int total = npad * npad, n = chi * chi;
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
     const int p = e / npad, q = e - p * npad;
-    Ab[e] = (p < nb && q < nb) ? A[(long long)rows[p] * n + rows[q]] : 0.0;
+    Ab[e] = (p < nb && q < nb) ? A[(long long)(rows ? rows[p] : p) * n + (rows ? rows[q] : q)] : 0.0;
+    if (e < npad) {
+      const int r = e < nb ? (rows ? rows[e] : e) : 0, x = (r % chi) * chi + r / chi;
+      swp[e] = e < nb ? (pos ? pos[x] : x) : e;
+    }
   }
 }
 
-void launch_z2_gather_sym(const double* A, int n, const int* rows, int nb, int npad, double* Ab,
-                          cudaStream_t s) {
-  z2_gather_sym_kernel<<<grid_for((long long)npad * npad), 256, 0, s>>>(A, n, rows, nb, npad, Ab);
+void launch_z2_gather_sym(const double* A, int chi, const int* rows, const int* pos, int nb, int npad, double* Ab,
+                          int* swp, cudaStream_t s) {
+  z2_gather_sym_kernel<<<grid_for((long long)npad * npad), 256, 0, s>>>(A, chi, rows, pos, nb, npad, Ab, swp);
   ++g_launches;
 }
 
 // Column-major n x n M from the blocks (leading dimension ld): M[r + c n] =
 // M_b[pos[r] + pos[c] ld] if rows r and c are both of parity b, else 0 (column c of M is
-// column pos[c] of block blk[c]; the padding columns of the blocks are dropped)
+// column pos[c] of block blk[c]; the padding columns of the blocks are dropped), and the
+// eigenvalue and the class of every column.  No blk: one block, in order.
 __global__ void z2_scatter_eig_kernel(const double* __restrict__ m0, const double* __restrict__ m1,
-                                      int ld, const int* __restrict__ blk, const int* __restrict__ pos,
-                                      int n, double* __restrict__ M) {
+                                      const double* __restrict__ l0, const double* __restrict__ l1,
+                                      const int* __restrict__ c0, const int* __restrict__ c1, int ld,
+                                      const int* __restrict__ blk, const int* __restrict__ pos, int n,
+                                      double* __restrict__ M, double* __restrict__ lam, int* __restrict__ cls) {
   const int total = n * n;
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
     const int cidx = e / n, r = e - cidx * n;
+    if (!blk) {
+      M[e] = m0[r + (long long)cidx * ld];
+      if (e < n) {
+        lam[e] = l0[e];
+        cls[e] = c0[e];
+      }
+      continue;
+    }
     const int b = blk[r];
     double v = 0.0;
     if (b == blk[cidx]) v = (b == 0 ? m0 : m1)[pos[r] + (long long)pos[cidx] * ld];
     M[e] = v;
+    if (e < n) {
+      lam[e] = (blk[e] == 0 ? l0 : l1)[pos[e]];
+      cls[e] = (blk[e] == 0 ? c0 : c1)[pos[e]];
+    }
   }
 }
 
-void launch_z2_scatter_eig(const double* m0, const double* m1, int ld, const int* blk, const int* pos,
-                           int n, double* M, cudaStream_t s) {
-  z2_scatter_eig_kernel<<<grid_for((long long)n * n), 256, 0, s>>>(m0, m1, ld, blk, pos, n, M);
+void launch_z2_scatter_eig(const double* m0, const double* m1, const double* l0, const double* l1,
+                           const int* c0, const int* c1, int ld, const int* blk, const int* pos, int n, double* M,
+                           double* lam, int* cls, cudaStream_t s) {
+  z2_scatter_eig_kernel<<<grid_for((long long)n * n), 256, 0, s>>>(m0, m1, l0, l1, c0, c1, ld, blk, pos, n, M, lam,
+                                                                   cls);
   ++g_launches;
 }
 
