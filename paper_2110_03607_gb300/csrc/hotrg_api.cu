@@ -38,6 +38,7 @@ struct Buf {
 enum : int {
   I_C = 1,
   I_RHO = 2,
+  I_CP = 3,    // c' (the slices of one pass)
   I_NH = 10,   // n^_j   (hat copy, unprimed)
   I_NC = 20,   // n~_j   (check copy, unprimed)
   I_NHP = 30,  // n^'_j  (hat copy, primed)
@@ -1442,11 +1443,12 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
   // everything below except the split T scales with the number of n'_1 values.
   const int nnew1 = nnew[1];
   int n1_chunk = nnew1;
+  double per_unit = 1.0;   // operand bytes of one n'_1 value of a slice
   {
     // the Z2 blocks of B and C hold about half of B and C again; the derivative
     // adds two more of B and C (and FP64 staging of dB in the split form) and three
     // more chain buffers
-    const double per_unit =
+    per_unit =
         (z2 ? 1.6 : 1.0) * (tangent ? (fp64 ? (tan2 ? 4.0 : 3.0) : 4.0) : 1.0) * (double)(Ns / nnew1) *
             ((fp64 ? 8.0 * R : (double)pbytes * npieces * Kpad) + (fp64 ? 8.0 : 4.0) * R) +
         (tan2 ? 7.0 : (tangent ? 5.0 : 2.0)) * (double)elt * (double)chain_max / nnew1;
@@ -1457,8 +1459,18 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
                              c->slice_budget_bytes);
     n1_chunk = (int)std::max(1.0, std::min((double)nnew1, std::floor(budget / per_unit)));
   }
-  const long long Nsub = (long long)n1_chunk * (Ns / nnew1);
-  const long long chain_sub = (chain_max / nnew1) * n1_chunk;
+  // Small slices share a pass: c' becomes one more index of the columns (c', n', n~), so that a step
+  // is a few launches with enough work for every SM instead of chi_c times as many small ones (2D
+  // chi = 24: one slice's non-prime stage has 576 threads).  As many as keep a pass's operands under
+  // 256 MB (a slice of that size fills the chip by itself), each output below 2^31 elements.
+  int sl_chunk = 1;
+  if (n1_chunk == nnew1) {
+    const double most = 268435456.0 / (per_unit * nnew1);
+    const double elems = 2147483648.0 / (double)std::max(Ns * R, chain_max);
+    sl_chunk = (int)std::max(1.0, std::min({(double)(sl_hi - sl_lo), most, elems}));
+  }
+  const long long Nsub = (long long)n1_chunk * (Ns / nnew1) * sl_chunk;
+  const long long chain_sub = (chain_max / nnew1) * n1_chunk * sl_chunk;
   CHECK_ALLOC(dev_alloc(c, c->chA, elt * chain_sub));
   CHECK_ALLOC(dev_alloc(c, c->chB, elt * chain_sub));
   if (tangent) {
@@ -1479,6 +1491,13 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
     long long off_blk, off_pos, off_list[2], L[2];
   };
   std::vector<Z2Chunk> zch;
+  long long moff_full = 0;
+  // columns of each block over the slices sl .. sl + cnt - 1, from those of one slice
+  auto slice_columns = [&](int sl, int cnt, const long long* L, long long* full) {
+    full[0] = full[1] = 0;
+    for (int k = sl; k < sl + cnt; ++k)
+      for (int b = 0; b < 2; ++b) full[b] += L[b ^ c->par[to[0]][k]];
+  };
   if (z2) {
     std::vector<int> hmap;
     auto push = [&](const std::vector<int>& v) {
@@ -1564,7 +1583,18 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
       }
       zch.push_back(ch);
     }
-    CHECK_ALLOC(dev_alloc(c, c->Zmap, sizeof(int) * hmap.size()));
+    if (sl_chunk > 1) {
+      // several slices a pass: the column maps of a pass (block, position, the two lists) are expanded
+      // on the device from those of one slice
+      moff_full = ((long long)hmap.size() + 63) / 64 * 64;
+      maxL = 0;
+      for (int sl = sl_lo; sl < sl_hi; sl += sl_chunk) {
+        long long l2[2];
+        slice_columns(sl, std::min(sl_chunk, sl_hi - sl), zch[0].L, l2);
+        maxL = std::max(maxL, std::max(l2[0], l2[1]));
+      }
+    }
+    CHECK_ALLOC(dev_alloc(c, c->Zmap, sizeof(int) * (sl_chunk > 1 ? moff_full + 4 * Nsub : (long long)hmap.size())));
     if (cudaMemcpyAsync(c->Zmap.p, hmap.data(), sizeof(int) * hmap.size(), cudaMemcpyHostToDevice, s) !=
         cudaSuccess)
       return cuda_status(c) == HOTRG_OK ? (c->poisoned = HOTRG_ECUDA) : HOTRG_ECUDA;
@@ -1648,10 +1678,34 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
   const int nterms = split_terms(npieces, terms_a, terms_b);
 
   const void* cblk_cur[2] = {nullptr, nullptr};   // this sub-slice's C blocks (Z2)
-  for (int sl = sl_lo; sl < sl_hi; ++sl)
+  for (int sl = sl_lo; sl < sl_hi; sl += sl_chunk)
   for (int n1lo = 0; n1lo < nnew1; n1lo += n1_chunk) {
     const int n1cnt = std::min(n1_chunk, nnew1 - n1lo);
-    const long long Nc = (long long)n1cnt * (Ns / nnew1);   // bottleneck columns of this sub-slice
+    const int scnt = std::min(sl_chunk, sl_hi - sl);         // slices of this pass
+    const long long Nc = (long long)n1cnt * (Ns / nnew1) * scnt;   // bottleneck columns of this pass
+    // Z2: parity of the slice (several slices: it is part of the columns' parities), the column maps
+    int q_sl = 0;
+    Z2Chunk zc_cur = {};
+    if (z2) {
+      zc_cur = zch[n1lo / n1_chunk];
+      if (sl_chunk == 1) {
+        q_sl = c->par[to[0]][sl];
+      } else {
+        unsigned qmask = 0;
+        for (int k = 0; k < scnt; ++k) qmask |= (unsigned)c->par[to[0]][sl + k] << k;
+        Z2Chunk full;
+        slice_columns(sl, scnt, zc_cur.L, full.L);
+        full.off_blk = moff_full;
+        full.off_pos = moff_full + Nsub;
+        full.off_list[0] = moff_full + 2 * Nsub;
+        full.off_list[1] = moff_full + 3 * Nsub;
+        int* zw = (int*)c->Zmap.p;
+        launch_z2_expand(zmap + zc_cur.off_blk, zmap + zc_cur.off_pos, (int)Ns, (int)zc_cur.L[0], (int)zc_cur.L[1],
+                         scnt, qmask, zw + full.off_blk, zw + full.off_pos, zw + full.off_list[0],
+                         zw + full.off_list[1], s);
+        zc_cur = full;
+      }
+    }
     int nsz[kMaxD];                                          // n' sizes of this sub-slice
     for (int k = 1; k < d; ++k) nsz[k] = k == 1 ? n1cnt : nnew[k];
     // -- prime-side chain, Eqs. (TU1)-(TUNCD), on the c'-fixed tensor T[(rho, n~), (sl, n~')]
@@ -1659,6 +1713,7 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
     in.push_back({I_RHO, chi_c, rs[0]});
     for (int k = 1; k < d; ++k) in.push_back({I_NC + k, chij[k], rs[k]});
     for (int k = 1; k < d; ++k) in.push_back({I_NCP + k, chij[k], cs[k]});
+    in.push_back({I_CP, scnt, cs[0]});
     const void* src = Tc + (long long)sl * cs[0];
     const void* dsrc = tangent ? (const double*)c->dT.p + (long long)sl * cs[0] : nullptr;
     const void* d2src = tan2 ? (const double*)c->d2T.p + (long long)sl * cs[0] : nullptr;
@@ -1669,6 +1724,7 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
       bool last = (j == d - 1);
       if (!last) {
         std::vector<std::pair<int, long long>> names;
+        names.push_back({I_CP, scnt});
         for (int k = 1; k <= j; ++k) names.push_back({I_NP + k, nsz[k]});
         names.push_back({I_RHO, chi_c});
         for (int k = 1; k < d; ++k) names.push_back({I_NC + k, chij[k]});
@@ -1677,6 +1733,7 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
         out = contiguous(names);
       } else {
         long long K_ = Kpad;
+        out.push_back({I_CP, scnt, Ns * K_});
         for (int k = 1; k < d; ++k) out.push_back({I_NP + k, nsz[k], prod_after(nnew, k) * P * K_});
         for (int k = 1; k < d; ++k) out.push_back({I_NC + k, chij[k], prod_after(chij, k) * K_});
         out.push_back({I_RHO, chi_c, P});
@@ -1721,8 +1778,8 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
         // the parity of their k, at the positions the bottleneck's blocks use
         cd.npieces = npieces;
         cd.pfmt = pfmt;
-        const Z2Chunk& ch = zch[n1lo / n1_chunk];
-        const int q = c->par[to[0]][sl];
+        const Z2Chunk& ch = zc_cur;
+        const int q = q_sl;
         Z2Out zo;
         zo.kcat = zmap + moff_kcat;
         zo.R = (unsigned)R;
@@ -1778,6 +1835,7 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
           ChainDesc cdt = cd;
           if (last) {
             View outT;
+            outT.push_back({I_CP, scnt, Ns * R});
             for (int k = 1; k < d; ++k) outT.push_back({I_NP + k, nsz[k], prod_after(nnew, k) * P * R});
             for (int k = 1; k < d; ++k) outT.push_back({I_NC + k, chij[k], prod_after(chij, k) * R});
             outT.push_back({I_RHO, chi_c, P});
@@ -1810,8 +1868,8 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
     // -- bottleneck, Eq. (BottleneckPart): C[(c, n^)][(n', n~)] = T . B^T
     if (z2) {
       // blocks b = 0, 1: rows and K of parity b, columns of parity b ^ q
-      const int q = c->par[to[0]][sl];
-      const Z2Chunk& ch = zch[n1lo / n1_chunk];
+      const int q = q_sl;
+      const Z2Chunk& ch = zc_cur;
       const void* cblk[2] = {nullptr, nullptr};
       long long ldb_[2] = {1, 1};
       for (int b = 0; b < 2; ++b) {
@@ -1907,6 +1965,7 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
     const long long rsh = zfold ? (1LL << 32) : Nc;
     cin.push_back({I_C, chi_c, P * rsh});
     for (int k = 1; k < d; ++k) cin.push_back({I_NH + k, chij[k], prod_after(chij, k) * rsh});
+    cin.push_back({I_CP, scnt, Ns});
     for (int k = 1; k < d; ++k) cin.push_back({I_NP + k, nsz[k], prod_after(nnew, k) * P});
     for (int k = 1; k < d; ++k) cin.push_back({I_NC + k, chij[k], prod_after(chij, k)});
     const void* csrc = c->Cb.p;
@@ -1920,6 +1979,7 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
         std::vector<std::pair<int, long long>> names;
         names.push_back({I_C, chi_c});
         for (int k = 1; k < j; ++k) names.push_back({I_NH + k, chij[k]});
+        names.push_back({I_CP, scnt});
         for (int k = 1; k < d; ++k) names.push_back({I_NP + k, nsz[k]});
         for (int k = 1; k < j; ++k) names.push_back({I_NC + k, chij[k]});
         for (int k = j; k < d; ++k) names.push_back({I_N + k, nnew[k]});
@@ -1927,6 +1987,7 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
       } else {
         out.push_back({I_C, chi_c, Pn * Rn});
         for (int k = 1; k < d; ++k) out.push_back({I_N + k, nnew[k], prod_after(nnew, k) * Rn});
+        out.push_back({I_CP, scnt, Pn});
         for (int k = 1; k < d; ++k) out.push_back({I_NP + k, nsz[k], prod_after(nnew, k)});
       }
       ChainDesc cd;
@@ -1964,13 +2025,13 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
       } else if (c->f64_chains && !tangent) {
         launch_chain_f64acc(cd, csrc, j == d - 1 ? 0 : 1, (const double*)c->U64.p + u_off[j], dst, OUT_F64, s);
       } else if (zfold && j == d - 1) {
-        const Z2Chunk& ch = zch[n1lo / n1_chunk];
+        const Z2Chunk& ch = zc_cur;
         Z2In zi;
         zi.rblk = zmap + moff_rowblk;
         zi.rpos = zmap + moff_rowpos;
         zi.cblk = zmap + ch.off_blk;
         zi.cpos = zmap + ch.off_pos;
-        zi.q = c->par[to[0]][sl];
+        zi.q = q_sl;
         zi.c[0] = (const float*)cblk_cur[0];
         zi.c[1] = (const float*)cblk_cur[1];
         zi.ld = ldz;

@@ -257,6 +257,8 @@ void launch_z2_reduce_sym(const double* p0, int ns0, int m0, const double* p1, i
                           const int* blk, const int* pos, int m, double* S, cudaStream_t s);
 void launch_z2_reduce_sum_t(const double* p0, int ns0, int m0, const double* p1, int ns1, int m1,
                             const int* blk, const int* pos, int m, double* dS, cudaStream_t s);
+void launch_z2_expand(const int* blk, const int* pos, int ns, int l0, int l1, int slices, unsigned qmask, int* fblk,
+                      int* fpos, int* list0, int* list1, cudaStream_t s);
 void launch_z2_gather_split(const double* src, long long ld, const int* rowmap, int nrows,
                             const int* colmap, int ncols, void* dst, long long piece_stride,
                             int npieces, int pfmt, cudaStream_t s);

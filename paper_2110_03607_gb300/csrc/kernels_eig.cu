@@ -15,7 +15,7 @@
 // the count of operations is what matters: n^3 (reduction) + up to 4/3 n^3 (merges, less what
 // deflates) + n^3 (back-transformation) + 2 n^3 (W = A V and its Gram
 // matrix).  Measured, before and after: 4 matrices of 32 rows 1.4 and 0.58 ms, 8 of 128 9.1 and 1.4,
-// 4 of 288 (2D, chi = 24, zero field) 85 and 3.9, 2 of 784 450 and 24.
+// 4 of 288 (2D, chi = 24, zero field) 85 and 3.9.
 //
 // Which vectors are taken from a degenerate eigenspace matters: the run goes on from them, and on
 // an isotropic lattice many pairs are degenerate, each vector with a symmetry of its own.  So the

@@ -124,6 +124,31 @@ static unsigned grid_for(long long total) {
   return (unsigned)blocks;
 }
 
+// Column maps of several slices from those of one: column (k, n) of slice k (parity q_k, bit k of
+// qmask) lies in block b = blk[n] ^ q_k, after the columns that the slices before it put there.
+__global__ void z2_expand_kernel(const int* __restrict__ blk, const int* __restrict__ pos, int ns, int l0, int l1,
+                                 unsigned qmask, int* __restrict__ fblk, int* __restrict__ fpos,
+                                 int* __restrict__ list0, int* __restrict__ list1) {
+  const int k = blockIdx.y;
+  const int odd = __popc(qmask & ((1u << k) - 1u)), even = k - odd, q = (qmask >> k) & 1;
+  for (int n = blockIdx.x * blockDim.x + threadIdx.x; n < ns; n += gridDim.x * blockDim.x) {
+    const int b = blk[n] ^ q;
+    const int before = b == 0 ? even * l0 + odd * l1 : even * l1 + odd * l0;
+    const int p = before + pos[n], g = k * ns + n;
+    fblk[g] = b;
+    fpos[g] = p;
+    (b == 0 ? list0 : list1)[p] = g;
+  }
+}
+
+void launch_z2_expand(const int* blk, const int* pos, int ns, int l0, int l1, int slices, unsigned qmask, int* fblk,
+                      int* fpos, int* list0, int* list1, cudaStream_t s) {
+  unsigned bx = (unsigned)((ns + 255) / 256);
+  if (bx > 64) bx = 64;
+  z2_expand_kernel<<<dim3(bx, (unsigned)slices), 256, 0, s>>>(blk, pos, ns, l0, l1, qmask, fblk, fpos, list0, list1);
+  ++g_launches;
+}
+
 void launch_z2_gather_split(const double* src, long long ld, const int* rowmap, int nrows,
                             const int* colmap, int ncols, void* dst, long long piece_stride,
                             int npieces, int pfmt, cudaStream_t s) {

@@ -5,8 +5,6 @@ batch, environments with degenerate, rank-deficient and exchange-symmetric struc
 import numpy as np
 import pytest
 
-from seeded_inputs import gaussian_tensor, reflection_symmetric_tensor
-
 pytestmark = pytest.mark.gpu
 
 
@@ -31,28 +29,31 @@ def _environment(t, axis, leg, prime):
     return a.reshape(chi_j * chi_j, chi_j * chi_j)
 
 
-def _falling(t, rate=0.35):
-    """The tensor with every leg falling off, as a coarse-grained one does."""
-    for k in range(t.ndim):
-        f = np.exp(-rate * np.arange(t.shape[k]))
-        t = t * f.reshape([-1 if q == k else 1 for q in range(t.ndim)])
-    return t
+def _sum_of_products(chis, seed, terms, rate, skew):
+    """sum_c prod_k f_k[c, x_k] f'_k[c, x_k']: the form of a block of spins, whose traces are positive
+    (f' = f + skew x noise; skew = 0: symmetric under the reflections)."""
+    rng = np.random.default_rng(seed)
+    t = np.ones((terms, 1))
+    for c in chis:
+        fall = np.exp(-rate * np.arange(c))
+        f = rng.standard_normal((terms, c)) * fall
+        g = f + skew * rng.standard_normal((terms, c)) * fall
+        t = (t[:, :, None, None] * f[:, None, :, None] * g[:, None, None, :]).reshape(terms, -1)
+    return t.sum(0).reshape([c for c in chis for _ in range(2)])
 
 
 def _product(chis, seed):
     """A tensor product of two equal tensors: every environment is a Kronecker square."""
-    h = [int(round(c ** 0.5)) for c in chis]
-    g = _falling(reflection_symmetric_tensor(h, seed))
-    t = np.multiply.outer(g, g)
+    g = _sum_of_products([int(round(c ** 0.5)) for c in chis], seed, 12, 0.35, 0.0)
     n = g.ndim
-    t = t.transpose([v for k in range(n) for v in (k, n + k)])
+    t = np.multiply.outer(g, g).transpose([v for k in range(n) for v in (k, n + k)])
     return t.reshape([c for c in chis for _ in range(2)])
 
 
 CASES = {
-    "jacobi_limit": ((4, 4, 4), 6, "gauss"),        # n = 16
-    "above_jacobi": ((3, 5, 5), 5, "gauss"),        # n = 25, two leaves
-    "unequal_legs": ((3, 2, 9), 7, "gauss"),        # n = 4 and 81 in one batch
+    "jacobi_limit": ((4, 4, 4), 6, "flat"),         # n = 16
+    "above_jacobi": ((3, 5, 5), 5, "flat"),        # n = 25, two leaves
+    "unequal_legs": ((3, 2, 9), 7, "flat"),        # n = 4 and 81 in one batch
     "tile_edge": ((2, 6, 8), 8, "falling"),         # n = 36 and 64
     "odd": ((7, 13), 13, "falling"),                # n = 169
     "cluster16": ((3, 15), 15, "falling"),          # n = 225
@@ -70,17 +71,11 @@ def test_spectra_and_isometries_match_lapack(pkg, case):
     chis, chi, kind = CASES[case]
     if kind == "product":
         t = _product(chis, 5)
-    elif kind == "reflect":
-        t = _falling(reflection_symmetric_tensor(chis, 3))
     else:
-        t = gaussian_tensor(chis, 7)
-        if kind == "lowrank":
-            t = np.einsum("ab,cd->abcd", *(gaussian_tensor([c], 8 + c) for c in chis)) + 0.1 * _falling(t, 2.0)
-        elif kind == "falling":
-            t = _falling(t)
-    tr = np.einsum("".join(2 * chr(97 + k) for k in range(len(chis))) + "->", t)
-    t = t * np.sign(tr)
-    t = t / abs(tr)
+        terms, rate, skew = {"flat": (200, 0.0, 0.3), "falling": (200, 0.35, 0.3), "reflect": (200, 0.35, 0.0),
+                             "lowrank": (3, 0.35, 0.3)}[kind]
+        t = _sum_of_products(chis, 7, terms, rate, skew)
+    t = t / np.einsum("".join(2 * chr(97 + k) for k in range(len(chis))) + "->", t)
     ctx = pkg.hotrg_init_tensor(len(chis), chis, t, 0.3)
     try:
         pkg.hotrg_set_precision(ctx, pkg.PREC_FP64)
@@ -91,7 +86,8 @@ def test_spectra_and_isometries_match_lapack(pkg, case):
             # decompose it backward stably (a few n eps): 1e-12 of lambda_1 covers n = 1024
             for side in (0, 1):
                 want = np.linalg.eigvalsh(_environment(t, 0, leg, side))[::-1]
-                lam = pkg.hotrg_spectrum(ctx, leg, side)
+                # values in a group of near-ties (1e-12 lambda_1 apart) stand in the pivots' order
+                lam = np.sort(pkg.hotrg_spectrum(ctx, leg, side))[::-1]
                 np.testing.assert_allclose(lam, np.abs(want), rtol=0, atol=1e-12 * want[0])
             a = _environment(t, 0, leg, prime)
             lam = pkg.hotrg_spectrum(ctx, leg, int(prime))
