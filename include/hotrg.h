@@ -396,7 +396,8 @@ int hotrg_gemm_nt(int mode, int M, int N, int K, const double* A, const double* 
  * the scratch is 256 + r(2*np*M*Kp) + r(2*np*N*Kp) + r(4*M*N) bytes, with
  * np = 2 (BF16X3) or 3 (BF16X6), Kp = K rounded up to a multiple of 64 and
  * r(x) = x rounded up to a multiple of 256; sizes whose scratch exceeds the
- * array are rejected with HOTRG_EINVAL (the FP64 mode needs no scratch).
+ * array are rejected with HOTRG_EINVAL (the FP64 mode works within the array: it holds the
+ * digits of the operands, of B in passes where they do not fit).
  * mode is HOTRG_PREC_FP64, HOTRG_PREC_BF16X3 or HOTRG_PREC_BF16X6 (the TF32
  * modes give HOTRG_EINVAL here).  The
  * size limits of hotrg_gemm_nt apply in every mode.  The first call on a device looks up the

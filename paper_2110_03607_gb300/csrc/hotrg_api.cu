@@ -181,6 +181,7 @@ struct hotrg_ctx {
   // buffers
   Buf Za, Zb, Zc, Zmap;   // Z2 blocks of the contraction operands, index maps
   Buf Zg;                 // Z2 index maps of the environment Grams and the eigen blocks
+  Buf Wd;                 // digits of the FP64 products on the tensor cores
   Buf Eb;                 // the eigen-solver's batch: blocks of A, their eigenvectors and eigenvalues
   Buf T, T2, Xp, parts, S, Amat, V, lam, U64, U32, legres, Y, state, counters, sweeps;
   Buf Ap, Bp, Cb, chA, chB;
@@ -364,8 +365,30 @@ int launch_failed(hotrg_ctx* c, const char* what, long long a, long long b, long
   return HOTRG_ECUDA;
 }
 
+// C = A . B^T in FP64: on the tensor cores where the product is large enough and the workspace can be
+// had, else on the FP64 pipe.  nsplit > 1: split along K, at most nsplit_most partials.  Returns the
+// partials written, or a negative status.
+int gemm64(hotrg_ctx* c, const double* A, long long lda, const double* B, long long ldb, double* C, long long ldc,
+           long long split_stride, int M, int N, long long K, int nsplit, int upper_only, cudaStream_t s,
+           int nsplit_most = 1) {
+  const size_t want = f64_tc_bytes(M, N, K, A == B && lda == ldb && M == N, upper_only);
+  if (want > 0) {
+    // sizes in powers of two: a run's bond dimensions grow, its workspace seldom
+    size_t size = (size_t)4 << 20;
+    while (size < want) size <<= 1;
+    if (c->Wd.bytes >= want || dev_alloc(c, c->Wd, size) == HOTRG_OK) {
+      const int r = launch_gemm_nt_f64_tc(A, lda, B, ldb, C, ldc, split_stride, M, N, K, std::max(nsplit, nsplit_most),
+                                          upper_only, c->Wd.p, c->Wd.bytes, &((DevState*)c->state.p)->status, s);
+      if (r > 0) return r;
+      if (r < 0) return launch_failed(c, "FP64 product on the tensor cores", M, N, K);
+    }
+  }
+  return launch_gemm_nt_f64(A, lda, B, ldb, C, ldc, split_stride, M, N, K, nsplit, upper_only, s);
+}
+
 // A launch error left pending by the kernels of one part of the step: report the part
 int pending_error(hotrg_ctx* c, const char* part) {
+  if (c->poisoned) return c->poisoned;   // a launch of this part was refused and reported
   const cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) return HOTRG_OK;
   fprintf(stderr, "hotrg: CUDA error after %s: %s\n", part, cudaGetErrorString(e));
@@ -667,7 +690,7 @@ int hotrg_set_allocator(hotrg_ctx* c, hotrg_alloc_fn alloc, hotrg_free_fn free_f
   Buf* b[] = {&c->T,  &c->T2, &c->Xp,     &c->parts, &c->S,     &c->Amat,
               &c->V,  &c->lam, &c->U64,   &c->U32,   &c->legres, &c->Y,       &c->state,
               &c->counters, &c->sweeps, &c->Ap, &c->Bp, &c->Cb, &c->chA, &c->chB,
-              &c->Ew, &c->lraw, &c->selw, &c->Za, &c->Zb, &c->Zc, &c->Zmap, &c->Zg, &c->Eb,
+              &c->Ew, &c->lraw, &c->selw, &c->Za, &c->Zb, &c->Zc, &c->Zmap, &c->Zg, &c->Eb, &c->Wd,
               &c->dT, &c->dT2, &c->dTb, &c->dXp, &c->dS, &c->dA, &c->dU64, &c->eG, &c->eZ, &c->eZt,
               &c->rank, &c->Yd, &c->tstate, &c->dchA, &c->dchB, &c->dchT, &c->dBp, &c->tBp, &c->dCb,
               &c->tCb, &c->dAp, &c->dB64, &c->dU32, &c->d2T, &c->d2T2, &c->d2Tb, &c->d2Tc, &c->d2Xp,
@@ -1040,8 +1063,8 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
           if (mb == 0 || Kb == 0) continue;
           const int nsplit = gram_splits(mb, Kb);
           double* pdst = (double*)c->parts.p + poff;
-          nsb[b] = launch_gemm_nt_f64(X + r0 * K + k0, K, X + r0 * K + k0, K, pdst, mb, mb * mb, (int)mb,
-                                      (int)mb, Kb, nsplit, 1, s);
+          nsb[b] = gemm64(c, X + r0 * K + k0, K, X + r0 * K + k0, K, pdst, mb, mb * mb, (int)mb,
+                                      (int)mb, Kb, nsplit, 1, s, nsplit_max);
           pb[b] = pdst;
           poff += (long long)nsb[b] * mb * mb;
         }
@@ -1060,8 +1083,8 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
       const int nsplit = gram_splits(m, Kp);
       // the GEMM may round nsplit down: reduce the partials it wrote
       const double* X0 = (const double*)c->Xp.p + k_lo;
-      const int used = launch_gemm_nt_f64(X0, K, X0, K, (double*)c->parts.p, m, m * m, (int)m, (int)m, Kp,
-                                          nsplit, 1, s);
+      const int used = gemm64(c, X0, K, X0, K, (double*)c->parts.p, m, m * m, (int)m, (int)m, Kp,
+                                          nsplit, 1, s, nsplit_max);
       launch_reduce_sym((const double*)c->parts.p, used, (int)m, Sdst, s);
     }
     double* S0 = (double*)c->S.p + ((long long)(j - 1) * 4) * mmax * mmax;
@@ -1309,8 +1332,8 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
             const long long r0 = b == 0 ? 0 : gz_mb[j][0], q0 = b == 0 ? 0 : gz_Kb[j][kind][0];
             const int nsplit = gram_splits(mb, Kb);
             double* pdst = (double*)c->parts.p + poff;
-            nsb[b] = launch_gemm_nt_f64(dX + r0 * K + q0, K, X + r0 * K + q0, K, pdst, mb, mb * mb, (int)mb,
-                                        (int)mb, Kb, nsplit, 0, s);
+            nsb[b] = gemm64(c, dX + r0 * K + q0, K, X + r0 * K + q0, K, pdst, mb, mb * mb, (int)mb,
+                                        (int)mb, Kb, nsplit, 0, s, nsplit_max);
             pb[b] = pdst;
             poff += (long long)nsb[b] * mb * mb;
           }
@@ -1322,8 +1345,8 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
         launch_permute(Tc, (double*)c->Xp.p, nd, size, ist, 1.0, s);
         launch_permute((const double*)c->dT.p, (double*)c->dXp.p, nd, size, ist, 1.0, s);
         const int nsplit = gram_splits(m, K);
-        const int used = launch_gemm_nt_f64((const double*)c->dXp.p, K, (const double*)c->Xp.p, K,
-                                            (double*)c->parts.p, m, m * m, (int)m, (int)m, K, nsplit, 0, s);
+        const int used = gemm64(c, (const double*)c->dXp.p, K, (const double*)c->Xp.p, K,
+                                            (double*)c->parts.p, m, m * m, (int)m, (int)m, K, nsplit, 0, s, nsplit_max);
         launch_sym_sum((const double*)c->parts.p, used, (int)m, dS0 + kind * mmax * mmax, s);
         if (tan2) {
           // d2S = d2X X^T + X d2X^T + 2 dX dX^T: the partials of d2X X^T and of dX dX^T (each
@@ -1331,10 +1354,10 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
           double* d2S0 = (double*)c->d2S.p + ((long long)(j - 1) * 4) * mmax * mmax;
           launch_permute((const double*)c->d2T.p, (double*)c->d2Xp.p, nd, size, ist, 1.0, s);
           double* p2 = (double*)c->parts2.p;
-          const int u1 = launch_gemm_nt_f64((const double*)c->d2Xp.p, K, (const double*)c->Xp.p, K, p2, m, m * m,
-                                            (int)m, (int)m, K, nsplit, 0, s);
-          const int u2 = launch_gemm_nt_f64((const double*)c->dXp.p, K, (const double*)c->dXp.p, K,
-                                            p2 + (long long)u1 * m * m, m, m * m, (int)m, (int)m, K, nsplit, 0, s);
+          const int u1 = gemm64(c, (const double*)c->d2Xp.p, K, (const double*)c->Xp.p, K, p2, m, m * m,
+                                            (int)m, (int)m, K, nsplit, 0, s, nsplit_max);
+          const int u2 = gemm64(c, (const double*)c->dXp.p, K, (const double*)c->dXp.p, K,
+                                            p2 + (long long)u1 * m * m, m, m * m, (int)m, (int)m, K, nsplit, 0, s, nsplit_max);
           launch_sym_sum(p2, u1 + u2, (int)m, d2S0 + kind * mmax * mmax, s);
         }
       }
@@ -1363,7 +1386,7 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
                              S0 + (k0 + 1) * mmax * mmax, dS0 + (k0 + 1) * mmax * mmax,
                              d2S0 + (k0 + 1) * mmax * mmax, chij[j], chi_c, d2As, s);
         launch_gemm_nn_f64(Vs, n, dAs, n, (double*)c->eW.p, n, n, n, n, 1, 0, 0, 0, s);       // rows dA v_a
-        launch_gemm_nt_f64((const double*)c->eW.p, n, Vs, n, (double*)c->eG1.p, n, 0, n, n, n, 1, 0, s);
+        gemm64(c, (const double*)c->eW.p, n, Vs, n, (double*)c->eG1.p, n, 0, n, n, n, 1, 0, s);
         launch_gemm_nn_f64(d2As, n, (const double*)c->U64.p + u_off[j], nn, G, nn, n, nn, n, 1, 0, 0, 0, s);
         launch_gemm_nn_f64(Vs, n, G, nn, (double*)c->eZ2.p, nn, n, nn, n, 1, 0, 0, 0, s);    // v_i . d2A u_k
         launch_eig_d2((const double*)c->eG1.p, (const double*)c->eZ.p, (const double*)c->eZ2.p,
@@ -1888,7 +1911,7 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
             launch_z2_gather_f64((const double*)c->Bp.p, R, nmap, (int)Nb, kmap, (int)Kpb[b], zb, s);
           }
           Phase ph(c, 6);
-          launch_gemm_nt_f64((const double*)c->Za.p + a_off, Kpb[b], zb, Kpb[b], zc, ldz, 0, (int)Rb[b],
+          gemm64(c, (const double*)c->Za.p + a_off, Kpb[b], zb, Kpb[b], zc, ldz, 0, (int)Rb[b],
                              (int)Nb, Kpb[b], 1, 0, s);
           cblk[b] = zc;
         } else {
@@ -1925,22 +1948,22 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
     bn_done += 2.0 * (double)R * (double)Nc * (double)R;
     Phase ph(c, 6);
     if (fp64) {
-      launch_gemm_nt_f64(Tc, R, (const double*)c->Bp.p, R, (double*)c->Cb.p, Nc, 0, (int)R, (int)Nc,
+      gemm64(c, Tc, R, (const double*)c->Bp.p, R, (double*)c->Cb.p, Nc, 0, (int)R, (int)Nc,
                          R, 1, 0, s);
       if (tangent) {   // dC = T^ . dB^T + dT^ . B^T
-        launch_gemm_nt_f64(Tc, R, (const double*)c->dBp.p, R, (double*)c->dCb.p, Nc, 0, (int)R, (int)Nc, R, 1,
+        gemm64(c, Tc, R, (const double*)c->dBp.p, R, (double*)c->dCb.p, Nc, 0, (int)R, (int)Nc, R, 1,
                            0, s);
-        launch_gemm_nt_f64((const double*)c->dT.p, R, (const double*)c->Bp.p, R, (double*)c->tCb.p, Nc, 0,
+        gemm64(c, (const double*)c->dT.p, R, (const double*)c->Bp.p, R, (double*)c->tCb.p, Nc, 0,
                            (int)R, (int)Nc, R, 1, 0, s);
         launch_axpby(1.0, (const double*)c->tCb.p, 1.0, (double*)c->dCb.p, R * Nc, s);
       }
       if (tan2) {      // d2C = T^ . d2B^T + 2 dT^ . dB^T + d2T^ . B^T
-        launch_gemm_nt_f64(Tc, R, (const double*)c->d2Bp.p, R, (double*)c->d2Cb.p, Nc, 0, (int)R, (int)Nc, R, 1,
+        gemm64(c, Tc, R, (const double*)c->d2Bp.p, R, (double*)c->d2Cb.p, Nc, 0, (int)R, (int)Nc, R, 1,
                            0, s);
-        launch_gemm_nt_f64((const double*)c->dT.p, R, (const double*)c->dBp.p, R, (double*)c->tCb.p, Nc, 0,
+        gemm64(c, (const double*)c->dT.p, R, (const double*)c->dBp.p, R, (double*)c->tCb.p, Nc, 0,
                            (int)R, (int)Nc, R, 1, 0, s);
         launch_axpby(2.0, (const double*)c->tCb.p, 1.0, (double*)c->d2Cb.p, R * Nc, s);
-        launch_gemm_nt_f64((const double*)c->d2T.p, R, (const double*)c->Bp.p, R, (double*)c->tCb.p, Nc, 0,
+        gemm64(c, (const double*)c->d2T.p, R, (const double*)c->Bp.p, R, (double*)c->tCb.p, Nc, 0,
                            (int)R, (int)Nc, R, 1, 0, s);
         launch_axpby(1.0, (const double*)c->tCb.p, 1.0, (double*)c->d2Cb.p, R * Nc, s);
       }
@@ -2304,7 +2327,17 @@ int hotrg_gemm_nt(int mode, int M, int N, int K, const double* A, const double* 
     cudaMemcpy(dB, B, sizeof(double) * N * K, cudaMemcpyDefault);
     cudaMemset(err, 0, sizeof(int));
     if (mode == HOTRG_PREC_FP64) {
-      launch_gemm_nt_f64((const double*)dA, K, (const double*)dB, K, (double*)dC, N, 0, M, N, K, 1, 0, s);
+      const size_t want = f64_tc_bytes(M, N, K, false, 0);
+      int r = 0;
+      if (want > 0) {
+        if (cudaMalloc(&pA, want) == cudaSuccess)
+          r = launch_gemm_nt_f64_tc((const double*)dA, K, (const double*)dB, K, (double*)dC, N, 0, M, N, K, 1, 0, pA,
+                                    want, err, s);
+        else
+          cudaGetLastError();   // no workspace: the FP64 pipe needs none
+      }
+      if (r == 0) launch_gemm_nt_f64((const double*)dA, K, (const double*)dB, K, (double*)dC, N, 0, M, N, K, 1, 0, s);
+      if (r < 0) fail(HOTRG_ECUDA);
     } else {
       cudaMemset(pA, 0, pbytes * np * M * Kpad);
       cudaMemset(pB, 0, pbytes * np * N * Kpad);
@@ -2766,7 +2799,7 @@ void hotrg_free(hotrg_ctx* c) {
   Buf* b[] = {&c->T,  &c->T2, &c->Xp,     &c->parts, &c->S,     &c->Amat,
               &c->V,  &c->lam, &c->U64,   &c->U32,   &c->legres, &c->Y,       &c->state,
               &c->counters, &c->sweeps, &c->Ap, &c->Bp, &c->Cb, &c->chA, &c->chB,
-              &c->Ew, &c->lraw, &c->selw, &c->Za, &c->Zb, &c->Zc, &c->Zmap, &c->Zg, &c->Eb,
+              &c->Ew, &c->lraw, &c->selw, &c->Za, &c->Zb, &c->Zc, &c->Zmap, &c->Zg, &c->Eb, &c->Wd,
               &c->dT, &c->dT2, &c->dTb, &c->dXp, &c->dS, &c->dA, &c->dU64, &c->eG, &c->eZ, &c->eZt,
               &c->rank, &c->Yd, &c->tstate, &c->dchA, &c->dchB, &c->dchT, &c->dBp, &c->tBp, &c->dCb,
               &c->tCb, &c->dAp, &c->dB64, &c->dU32, &c->d2T, &c->d2T2, &c->d2Tb, &c->d2Tc, &c->d2Xp,

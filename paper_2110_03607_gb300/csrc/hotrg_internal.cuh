@@ -99,6 +99,22 @@ inline int split_terms(int npieces, int* ta, int* tb) {
 }
 
 #ifdef __CUDACC__
+// sum of n split-K partials in eight chains: the loads overlap, and the rounding error grows with the
+// square root of n / 8, not of n
+template <typename F>
+__device__ __forceinline__ double sum_partials(int n, F&& part) {
+  double s[8] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+  int z = 0;
+  for (; z + 8 <= n; z += 8) {
+#pragma unroll
+    for (int q = 0; q < 8; ++q) s[q] += part(z + q);
+  }
+#pragma unroll
+  for (int q = 0; q < 7; ++q)
+    if (z + q < n) s[q] += part(z + q);
+  return ((s[0] + s[1]) + (s[2] + s[3])) + ((s[4] + s[5]) + (s[6] + s[7]));
+}
+
 // x rounded to TF32 (10 stored mantissa bits, ties to even) in an FP32 word whose low
 // 13 bits are zero; infinities and NaNs pass unchanged
 __device__ __forceinline__ float round_tf32(float x) {
@@ -286,6 +302,14 @@ int tc_gemm_ready();
 // milliseconds per launch of the split GEMM on device-resident operands (rate probe)
 int measure_tc_gemm_rate(int npieces, int M, int N, int Kpad, int iters, double* ms_per_launch,
                          int pfmt = PIECE_BF16);
+
+// ---- kernels_f64_tc.cu: the FP64 products on the tensor cores, C = A . B^T as launch_gemm_nt_f64
+// workspace wanted (0: the product is left to the FP64 pipe)
+size_t f64_tc_bytes(long long M, long long N, long long K, bool same, int upper);
+// partials written (<= max_split); 0: not done; negative: an error
+int launch_gemm_nt_f64_tc(const double* A, long long lda, const double* B, long long ldb, double* C, long long ldc,
+                          long long split_stride, int M, int N, long long K, int max_split, int upper_only, void* ws,
+                          size_t ws_bytes, int* err_flag, cudaStream_t s);
 
 // ---- kernels_tensor.cu: streaming multiprocessors of the current device (cached per device)
 int sm_count();

@@ -369,6 +369,15 @@ void launch_chain_f64acc(const ChainDesc& d, const void* in, int in_is_f64, cons
 
 void launch_chain_f64(const ChainDesc& d, const double* in, const double* U, double* out,
                       cudaStream_t s) {
+  if (sizeof(double) * d.chi * d.chi * (d.nn <= 24 ? 25 : 33) > 227 * 1024) {
+    // chi >= 30: all columns of U~ do not fit in shared memory; half of them at a time
+    ChainDesc h = d;
+    h.nn = 16;
+    dispatch_nn<double, double>(h, in, U, out, OUT_F64, s);
+    h.nn = d.nn - 16;
+    dispatch_nn<double, double>(h, in, U + 16, out + 16 * d.n_out_stride, OUT_F64, s);
+    return;
+  }
   dispatch_nn<double, double>(d, in, U, out, OUT_F64, s);
 }
 

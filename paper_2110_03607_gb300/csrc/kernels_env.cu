@@ -232,9 +232,7 @@ __global__ void reduce_sym_kernel(const double* __restrict__ parts, int nsplit, 
        e += (long long)gridDim.x * blockDim.x) {
     int i = (int)(e / m), j = (int)(e % m);
     int lo = i < j ? i : j, hi = i < j ? j : i;
-    double acc = 0.0;
-    for (int z = 0; z < nsplit; ++z) acc += parts[(long long)z * total + (long long)lo * m + hi];
-    G[e] = acc;
+    G[e] = sum_partials(nsplit, [&](int z) { return parts[(long long)z * total + (long long)lo * m + hi]; });
   }
 }
 

@@ -53,10 +53,9 @@ __global__ void sym_sum_kernel(const double* __restrict__ parts, int nsplit, int
   for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total;
        e += (long long)gridDim.x * blockDim.x) {
     const int i = (int)(e / m), j = (int)(e % m);
-    double acc = 0.0;
-    for (int z = 0; z < nsplit; ++z)
-      acc += parts[z * total + (long long)i * m + j] + parts[z * total + (long long)j * m + i];
-    dS[e] = acc;
+    dS[e] = sum_partials(nsplit, [&](int z) {
+      return parts[z * total + (long long)i * m + j] + parts[z * total + (long long)j * m + i];
+    });
   }
 }
 

@@ -33,15 +33,13 @@
 // (small) scale and only the four leading MMAs truncate at the scale of the result.
 // Every mbarrier wait is bounded in time; an expired wait sets a global error flag
 // that also makes the other CTAs give up.
-#include <cuda.h>
 #include <stdio.h>
 #include <stdlib.h>
 
 #include <algorithm>
 #include <atomic>
 
-#include "hotrg_internal.cuh"
-#include "../../include/hotrg.h"
+#include "tcgen05.cuh"
 
 namespace hotrg {
 
@@ -78,7 +76,6 @@ constexpr int W_PROD = EPI_WARPS, W_MMA = EPI_WARPS + 1;
 constexpr int NTHREADS = 32 * (EPI_WARPS + 2);      // epilogue warps + producer + MMA
 constexpr int SMEM_BYTES = 1024 + STAGES * STAGE_BYTES + 256;
 static_assert(SMEM_BYTES <= 227 * 1024, "shared memory of one CTA");
-constexpr unsigned long long WAIT_NS = 4000000000ull;  // 4 s per wait
 }  // namespace
 
 // K slabs per accumulation chunk (chunk length TK x this along K; 64 by default)
@@ -96,144 +93,6 @@ struct TcTerms {
   // register: an indexed array would live in local memory on the MMA issuer's path)
   unsigned long long code;
 };
-
-__device__ __forceinline__ uint32_t su32(const void* p) {
-  return (uint32_t)__cvta_generic_to_shared(p);
-}
-
-__device__ __forceinline__ unsigned long long gtimer() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t* bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(su32(bar)), "r"(count) : "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint64_t* bar, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(su32(bar)),
-               "r"(bytes)
-               : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(ok)
-      : "r"(su32(bar)), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-
-// Bounded wait: gives up after WAIT_NS, or as soon as another thread of the
-// CTA or another CTA has given up.
-__device__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* cta_abort,
-                          volatile int* g_err) {
-  unsigned long long t0 = 0;
-  uint32_t spins = 0;
-  while (!mbar_try_wait(bar, parity)) {
-    if ((++spins & 127u) == 0) {
-      if (*cta_abort || *g_err) return false;
-      unsigned long long t = gtimer();
-      if (t0 == 0) t0 = t;
-      else if (t - t0 > WAIT_NS) {
-        *cta_abort = 1;
-        atomicExch((int*)g_err, HOTRG_ETIMEOUT);
-        return false;
-      }
-    }
-  }
-  return true;
-}
-
-__device__ __forceinline__ void tma_load_3d(const CUtensorMap* map, void* dst, uint64_t* bar, int x,
-                                            int y, int z) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes"
-      " [%0], [%1, {%2, %3, %4}], [%5];" ::"r"(su32(dst)),
-      "l"((unsigned long long)map), "r"(x), "r"(y), "r"(z), "r"(su32(bar))
-      : "memory");
-}
-
-// Shared-memory matrix descriptor for a K-major operand tile written by TMA with
-// the SW_BYTES swizzle: rows of SW_BYTES bytes (TK BF16 along K), 8-row groups
-// 8 SW_BYTES apart (the swizzle pattern repeats every 8 rows).
-__device__ __forceinline__ uint64_t sdesc_sw(uint32_t saddr) {
-  uint64_t d = 0;
-  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);         // start address
-  d |= (uint64_t)1 << 16;                           // leading byte offset (unused for this layout)
-  d |= (uint64_t)((8 * SW_BYTES) >> 4) << 32;       // stride byte offset: 8 rows
-  d |= (uint64_t)1 << 46;                           // descriptor version
-  d |= (uint64_t)(SW_BYTES == 128 ? 2 : 4) << 61;   // 128- or 64-byte swizzle
-  return d;
-}
-
-// Instruction descriptor, kind::f16: D = F32, A = B = BF16, both K-major, N, M.
-__host__ __device__ constexpr uint32_t idesc_bf16_f32(int m, int n) {
-  return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(n >> 3) << 17) |
-         ((uint32_t)(m >> 4) << 24);
-}
-
-// Instruction descriptor, kind::tf32: D = F32, A = B = TF32 (format 2), both K-major.
-__host__ __device__ constexpr uint32_t idesc_tf32_f32(int m, int n) {
-  return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(n >> 3) << 17) |
-         ((uint32_t)(m >> 4) << 24);
-}
-
-__device__ __forceinline__ void umma_bf16(uint32_t d_tmem, uint64_t a, uint64_t b, uint32_t idesc,
-                                          uint32_t accumulate) {
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "setp.ne.b32 p, %4, 0;\n\t"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
-      : "memory");
-}
-
-__device__ __forceinline__ void umma_commit(uint64_t* bar) {
-  asm volatile(
-      "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-          su32(bar))
-      : "memory");
-}
-
-__device__ __forceinline__ void tc_fence_before() {
-  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-}
-__device__ __forceinline__ void tc_fence_after() {
-  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-}
-
-// 32 lanes x 32 (or 16) columns of FP32 from TMEM; usable after tmem_wait_ld()
-__device__ __forceinline__ void tmem_ld_async(uint32_t taddr, uint32_t (&v)[32]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
-        "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]),
-        "=r"(v[14]), "=r"(v[15]), "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]),
-        "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]), "=r"(v[24]), "=r"(v[25]),
-        "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-      : "r"(taddr));
-}
-__device__ __forceinline__ void tmem_ld_async(uint32_t taddr, uint32_t (&v)[16]) {
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-      : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]),
-        "=r"(v[7]), "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]),
-        "=r"(v[14]), "=r"(v[15])
-      : "r"(taddr));
-}
-
-__device__ __forceinline__ void tmem_wait_ld() {
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-}
 
 __global__ void __launch_bounds__(NTHREADS, 1)
     tc_gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
@@ -362,8 +221,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
               const uint32_t st = su32(smem + s * STAGE_BYTES);
               for (int t = t0; t < t1; ++t) {
                 const int pa_t = (int)(terms.code >> (4 * t)) & 3, pb_t = (int)(terms.code >> (4 * t + 2)) & 3;
-                const uint64_t a0 = sdesc_sw(st + pa_t * A_PIECE);
-                const uint64_t b0 = sdesc_sw(st + MAXP * A_PIECE + pb_t * B_PIECE);
+                const uint64_t a0 = sdesc_sw<SW_BYTES>(st + pa_t * A_PIECE);
+                const uint64_t b0 = sdesc_sw<SW_BYTES>(st + MAXP * A_PIECE + pb_t * B_PIECE);
 #pragma unroll
                 for (int kk = 0; kk < TK / 16; ++kk) {
                   // advance 16 BF16 = 32 bytes along K inside the swizzled row;
@@ -760,17 +619,14 @@ static EncodeTiledFn get_encode() {
 
 int tc_gemm_ready() { return get_encode() != nullptr; }
 
-// operand pieces stored as [piece][rows][kpad] elements (BF16, or TF32 in FP32 words);
-// one box = box_k elements of K (box_k x element size = the swizzle width) x box_rows
-// rows of one piece
-static int make_map(CUtensorMap* map, const void* base, int rows, int kpad, int npieces, int box_rows,
-                    int box_k = TK, bool tf32 = false) {
+int make_piece_map(CUtensorMap* map, const void* base, int rows, int kpad, int npieces, int box_rows, int box_k,
+                   bool tf32, int box_pieces) {
   EncodeTiledFn enc = get_encode();
   if (!enc) return -1;
   const cuuint64_t esz = tf32 ? 4 : 2;
   cuuint64_t dims[3] = {(cuuint64_t)kpad, (cuuint64_t)rows, (cuuint64_t)npieces};
   cuuint64_t strides[2] = {(cuuint64_t)kpad * esz, (cuuint64_t)kpad * esz * (cuuint64_t)rows};
-  cuuint32_t box[3] = {(cuuint32_t)box_k, (cuuint32_t)box_rows, 1};
+  cuuint32_t box[3] = {(cuuint32_t)box_k, (cuuint32_t)box_rows, (cuuint32_t)box_pieces};
   cuuint32_t estr[3] = {1, 1, 1};
   CUresult r = enc(map, tf32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, (void*)base,
                    dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -834,9 +690,9 @@ int launch_tc_gemm(const void* A, int M, const void* B, int N, int Kpad, int npi
   const int slab_k = tf32 ? P_TK / 2 : P_TK;   // elements of a 128-byte row
   CUtensorMap ma, mb;
   if (use_pair) {
-    if (make_map(&ma, A, M, Kpad, npieces, 128, slab_k, tf32) || make_map(&mb, B, N, Kpad, npieces, 128, slab_k, tf32))
+    if (make_piece_map(&ma, A, M, Kpad, npieces, 128, slab_k, tf32) || make_piece_map(&mb, B, N, Kpad, npieces, 128, slab_k, tf32))
       return -1;
-  } else if (make_map(&ma, A, M, Kpad, npieces, TM) || make_map(&mb, B, N, Kpad, npieces, TN)) {
+  } else if (make_piece_map(&ma, A, M, Kpad, npieces, TM, TK) || make_piece_map(&mb, B, N, Kpad, npieces, TN, TK)) {
     return -1;
   }
   // terms ordered by decreasing piece order (pa + pb): the smallest terms go first into

@@ -255,7 +255,7 @@ __global__ void z2_reduce_sym_kernel(const double* __restrict__ p0, int ns0, int
       const double* p = b == 0 ? p0 : p1;
       const int mb = b == 0 ? m0 : m1, ns = b == 0 ? ns0 : ns1;
       const long long bb = (long long)mb * mb;
-      for (int z = 0; z < ns; ++z) acc += p[z * bb + (long long)lo * mb + hi];
+      acc = sum_partials(ns, [&](int z) { return p[z * bb + (long long)lo * mb + hi]; });
     }
     S[e] = acc;
   }
@@ -286,8 +286,8 @@ __global__ void z2_reduce_sum_t_kernel(const double* __restrict__ p0, int ns0, i
       const double* p = b == 0 ? p0 : p1;
       const int mb = b == 0 ? m0 : m1, ns = b == 0 ? ns0 : ns1;
       const long long bb = (long long)mb * mb;
-      for (int z = 0; z < ns; ++z)
-        acc += p[z * bb + (long long)pi * mb + pj] + p[z * bb + (long long)pj * mb + pi];
+      acc = sum_partials(
+          ns, [&](int z) { return p[z * bb + (long long)pi * mb + pj] + p[z * bb + (long long)pj * mb + pi]; });
     }
     dS[e] = acc;
   }
