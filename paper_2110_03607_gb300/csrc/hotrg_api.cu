@@ -1628,6 +1628,16 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
   // directly (no dense C)
   const bool zfold = z2 && !fp64 && !c->f64_chains;
   const long long ldz = (maxL + 3) / 4 * 4;   // row pitch of the C blocks
+  // the last leg's isometry and parities, for the two large stages of the Z2 form
+  Z2Chain last_leg = {};
+  if (zfold) {
+    last_leg.U = (const float*)c->U32.p + u_off[d - 1];
+    last_leg.ldu = nnew[d - 1];
+    last_leg.chi = chij[d - 1];
+    last_leg.nn = nnew[d - 1];
+    for (int i = 0; i < std::min(32, chij[d - 1]); ++i) last_leg.mask_b |= (unsigned)c->par[to[d - 1]][i] << i;
+    for (int i = 0; i < nnew[d - 1]; ++i) last_leg.mask_n |= (unsigned)newpar[d - 1][i] << i;
+  }
   if (fp64) {
     CHECK_ALLOC(dev_alloc(c, c->Bp, sizeof(double) * Nsub * R));
     CHECK_ALLOC(dev_alloc(c, c->Cb, sizeof(double) * R * Nsub));
@@ -1845,7 +1855,16 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
           zo.r_shift = l;
           zo.r_magic = (unsigned)((((1ULL << l) - (unsigned long long)R) << 32) / (unsigned long long)R + 1);
         }
-        tuned_chain(c, cd, 1, [&] { launch_chain_f32_z2out(cd, src, src_f64, (const float*)c->U32.p + u_off[j] + ucol, zo, s); });
+        tuned_chain(c, cd, 1, [&] {
+          if (d >= 3 && chij[j] <= 32 && !src_f64) {
+            Z2Blocks zb = {zo.cblk, zo.cpos, zo.q, {zo.blk[0], zo.blk[1]}, {zo.ld[0], zo.ld[1]},
+                           {zo.pstride[0], zo.pstride[1]}, npieces};
+            if (launch_z2_prime(last_leg, (const float*)src, (int)(P / chij[j]), chi_c, (int)P, Nc / nsz[j], zo.kcat,
+                                (int)Rb[0], (int)R, zb, pfmt, cd.ctas_per_sm, s))
+              return;
+          }
+          launch_chain_f32_z2out(cd, src, src_f64, (const float*)c->U32.p + u_off[j] + ucol, zo, s);
+        });
       } else {
         cd.npieces = npieces;
         cd.pfmt = pfmt;
@@ -2058,7 +2077,12 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
         zi.c[0] = (const float*)cblk_cur[0];
         zi.c[1] = (const float*)cblk_cur[1];
         zi.ld = ldz;
-        tuned_chain(c, cd, 2, [&] { launch_chain_f32_z2in(cd, zi, (const float*)c->U32.p + u_off[j], dst, last ? OUT_F64 : OUT_F32, s); });
+        tuned_chain(c, cd, 2, [&] {
+          if (d >= 3 && chij[j] <= 32 &&
+              launch_z2_nonprime(last_leg, zi, R / chij[j], Nc / chij[j], (float*)dst, cd.ctas_per_sm, s))
+            return;
+          launch_chain_f32_z2in(cd, zi, (const float*)c->U32.p + u_off[j], dst, last ? OUT_F64 : OUT_F32, s);
+        });
       } else {
         launch_chain_f32(cd, csrc, 0, (const float*)c->U32.p + u_off[j], dst, last ? OUT_F64 : OUT_F32, s);
         if (tangent) {   // the same in FP32 (FP64 output of the last stage)

@@ -250,6 +250,29 @@ void launch_chain_f32_z2in(const ChainDesc& d, const Z2In& zi, const float* U, v
 void launch_chain_f32_z2out(const ChainDesc& d, const void* in, int in_is_f64, const float* U, const Z2Out& zo,
                             cudaStream_t s);
 
+// ---- kernels_z2chain.cu: the two large chain stages of the Z2 form (d >= 3) without their zero terms
+struct Z2Chain {
+  const float* U;      // U~ of the last leg, row (a + b chi), pitch ldu
+  int ldu;
+  int chi, nn;         // hat / check and new indices of the last leg (both at most 32)
+  unsigned mask_b;     // bit i: parity of hat / check index i
+  unsigned mask_n;     // bit i: parity of new index i
+};
+struct Z2Blocks {
+  const int* cblk;        // as in Z2Out
+  const int* cpos;
+  int q;
+  void* blk[2];
+  long long ld[2];
+  long long pstride[2];
+  int npieces;
+};
+// false: not launched (U~ does not fit in shared memory)
+bool launch_z2_prime(const Z2Chain& p, const float* in, int H, int chi_c, int P, long long groups, const int* kcat,
+                     int rb0, int R, const Z2Blocks& zo, int pfmt, int ctas_per_sm, cudaStream_t s);
+bool launch_z2_nonprime(const Z2Chain& p, const Z2In& zi, long long rrs, long long ccs, float* out, int ctas_per_sm,
+                        cudaStream_t s);
+
 // ---- kernels_z2.cu
 struct Z2Slots {
   int d;
