@@ -914,21 +914,37 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
   long long gz_mb[kMaxD][2], gz_Kb[kMaxD][4][2], gz_n64 = 0, gz_eig[kMaxD];
   int eig_nb[kMaxD][2];
   if (z2g && env_phase) {
+    // uploaded: the row offsets, the int maps, and for every summed index k = (hi, lo), each half d - 1
+    // legs, two tables of about sqrt(K) entries, from which the device writes the K offsets
     long long n64 = 0, n32 = 0;
+    Z2SumDesc sd = {};
     for (int j = 1; j < d; ++j) {
       const long long m = (long long)chij[j] * chi_c;
       for (int kind = 0; kind < 4; ++kind) {
         gz_roff[j][kind] = n64;
-        gz_koff[j][kind] = n64 + m;
-        n64 += m + RR / m;
+        n64 += m;
+        long long size[kMaxDims], ist[kMaxDims];
+        int pslot[kMaxDims];
+        gram_dims(j, kind, size, ist, pslot);
+        Z2Sum& z = sd.sum[sd.n++];
+        z.nhi = z.nlo = 1;
+        for (int q = 2; q < 2 * d; ++q) (q <= d ? z.nhi : z.nlo) *= (int)size[q];
+        z.off_hi = n64;
+        z.off_lo = n64 + z.nhi;
+        n64 += z.nhi + z.nlo;
+        z.rank_hi = (int)n32;
+        z.rank_lo = (int)n32 + z.nhi;
+        n32 += z.nhi + z.nlo;
       }
       gz_rowmap[j] = n32;
       n32 += 2 * m;
       gz_eig[j] = n32;                       // rows by parity, block, position (n = chi_j^2)
       n32 += 3LL * chij[j] * chij[j];
     }
-    gz_n64 = n64;   // the int maps follow the offsets
+    gz_n64 = n64;   // the int maps follow the offsets, the K offsets the int maps
+    n32 += n32 & 1;
     const size_t bytes = sizeof(long long) * n64 + sizeof(int) * n32;
+    long long kout = n64 + n32 / 2;
     long long* h64 = (long long*)pinned_stage(c, bytes);
     std::vector<long long> h64v;
     if (!h64) {
@@ -936,8 +952,7 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
       h64 = h64v.data();
     }
     int* h32 = (int*)(h64 + n64);
-    std::vector<long long> offs;
-    std::vector<unsigned char> pk;
+    int at = 0;
     for (int j = 1; j < d; ++j) {
       const std::vector<unsigned char>& pf = c->par[to[j]];
       const std::vector<unsigned char>& pc = c->par[to[0]];
@@ -972,51 +987,55 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
       for (int kind = 0; kind < 4; ++kind) {
         long long size[kMaxDims], ist[kMaxDims];
         int pslot[kMaxDims];
-        const int nd = gram_dims(j, kind, size, ist, pslot);
+        gram_dims(j, kind, size, ist, pslot);
         long long* ro = h64 + gz_roff[j][kind];
         long long w[2] = {0, cnt[0]};
         for (int f = 0; f < chij[j]; ++f)
           for (int cu = 0; cu < chi_c; ++cu) ro[w[pf[f] ^ pc[cu]]++] = f * ist[0] + cu * ist[1];
-        // the summed index, row-major over dims 2 .. nd-1, by an odometer
-        const long long K = RR / ((long long)chij[j] * chi_c);
-        offs.resize(K);
-        pk.resize(K);
-        long long idx[kMaxDims] = {0};
-        long long off = 0;
-        int par_ = 0;
-        for (int q = 2; q < nd; ++q) par_ ^= c->par[to[pslot[q]]][0];
-        long long kc[2] = {0, 0};
-        for (long long k = 0; k < K; ++k) {
-          offs[k] = off;
-          pk[k] = (unsigned char)par_;
-          ++kc[par_];
-          for (int q = nd - 1; q >= 2; --q) {
-            const std::vector<unsigned char>& pq = c->par[to[pslot[q]]];
-            par_ ^= pq[idx[q]];
-            off -= idx[q] * ist[q];
-            if (++idx[q] < size[q]) {
-              par_ ^= pq[idx[q]];
-              off += idx[q] * ist[q];
-              break;
+        // one half of the summed index: offset, and (even ones before << 1 | parity) for hi or
+        // (ones of the same parity before << 1 | parity) for lo
+        Z2Sum& z = sd.sum[at++];
+        int even_hi = 0, lo_cnt[2] = {0, 0};
+        for (int half = 0; half < 2; ++half) {
+          const int q0 = half == 0 ? 2 : d + 1, q1 = half == 0 ? d : 2 * d - 1;
+          const int nh = half == 0 ? z.nhi : z.nlo;
+          for (int x = 0; x < nh; ++x) {
+            long long off = 0;
+            int par = 0, rest = x;
+            for (int q = q1; q >= q0; --q) {
+              const int v = rest % (int)size[q];
+              rest /= (int)size[q];
+              off += v * ist[q];
+              par ^= c->par[to[pslot[q]]][v];
             }
-            idx[q] = 0;
-            par_ ^= pq[0];
+            h64[(half == 0 ? z.off_hi : z.off_lo) + x] = off;
+            if (half == 0) {
+              h32[z.rank_hi + x] = even_hi << 1 | par;
+              even_hi += par ^ 1;
+            } else {
+              h32[z.rank_lo + x] = lo_cnt[par]++ << 1 | par;
+            }
           }
         }
-        long long* ko = h64 + gz_koff[j][kind];
-        long long wk[2] = {0, kc[0]};
-        for (long long k = 0; k < K; ++k) ko[wk[pk[k]]++] = offs[k];
-        gz_Kb[j][kind][0] = kc[0];
-        gz_Kb[j][kind][1] = kc[1];
+        z.even_lo = lo_cnt[0];
+        const long long K = RR / ((long long)chij[j] * chi_c);
+        const long long k0 = (long long)even_hi * lo_cnt[0] + (long long)(z.nhi - even_hi) * lo_cnt[1];
+        gz_Kb[j][kind][0] = k0;
+        gz_Kb[j][kind][1] = K - k0;
+        z.even_all = k0;
+        gz_koff[j][kind] = kout;
+        z.out = kout;
+        kout += K;
       }
     }
-    CHECK_ALLOC(dev_alloc(c, c->Zg, bytes));
+    CHECK_ALLOC(dev_alloc(c, c->Zg, sizeof(long long) * kout));
     if (cudaMemcpyAsync(c->Zg.p, h64, bytes, cudaMemcpyHostToDevice, s) != cudaSuccess)
       return cuda_status(c) == HOTRG_OK ? (c->poisoned = HOTRG_ECUDA) : HOTRG_ECUDA;
     if (h64v.empty()) {
       cudaEventRecord(c->hpin_ev, s);
       c->hpin_pending = 1;
     }
+    launch_z2_sum_offsets((long long*)c->Zg.p, gz_n64, sd, s);
   }
   // the shard's layout of the Grams: legs j = 1 .. d-1, kinds 0 .. 3, each m_j x m_j
   // row-major (m_j = chi_j chi_c), concatenated
@@ -1511,10 +1530,10 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
   long long Rb[2] = {0, 0}, Kpb[2] = {0, 0}, maxL = 0;
   long long moff_rowblk = 0, moff_rowpos = 0, moff_kcat = 0, moff_k[2] = {0, 0};
   struct Z2Chunk {
-    long long off_blk, off_pos, off_list[2], L[2];
+    long long x0, off_blk, off_pos, off_list[2], L[2];
   };
   std::vector<Z2Chunk> zch;
-  long long moff_full = 0;
+  long long moff_full = 0, moff_rx = 0, moff_ry = 0, map_upload = 0;
   // columns of each block over the slices sl .. sl + cnt - 1, from those of one slice
   auto slice_columns = [&](int sl, int cnt, const long long* L, long long* full) {
     full[0] = full[1] = 0;
@@ -1584,32 +1603,41 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
       }
       ptl[x] = (unsigned char)p_;
     }
-    const long long per_n1 = Ns / nnew1;
+    // columns n = x P + y: the device writes each chunk's maps (block, position, the two lists) from the
+    // parities and ranks of x = n' and y = n~
+    std::vector<int> rx((size_t)Pn + 1), ry((size_t)P);
+    for (long long x = 0, even = 0; x <= Pn; ++x) {
+      const int p_ = x < Pn ? pnp[x] : 0;
+      rx[x] = (int)(even << 1) | p_;
+      even += p_ ^ 1;
+    }
+    int ycnt[2] = {0, 0};
+    for (long long y = 0; y < P; ++y) {
+      const int p_ = ptl[y];
+      ry[y] = ycnt[p_]++ << 1 | p_;
+    }
+    moff_rx = push(rx);
+    moff_ry = push(ry);
+    map_upload = (long long)hmap.size();
+    moff_full = (map_upload + 63) / 64 * 64;
     for (int n1lo = 0; n1lo < nnew1; n1lo += n1_chunk) {
-      const long long Nc = (long long)std::min(n1_chunk, nnew1 - n1lo) * per_n1;
-      const long long base = (long long)n1lo * per_n1;
-      std::vector<int> colblk(Nc), colpos(Nc), lst[2];
-      for (long long n = 0; n < Nc; ++n) {
-        const long long g = base + n;
-        const int p_ = pnp[g / P] ^ ptl[g % P];
-        colblk[n] = p_;
-        colpos[n] = (int)lst[p_].size();
-        lst[p_].push_back((int)n);
-      }
+      const long long x0 = (long long)n1lo * (Pn / nnew1), nx = (long long)std::min(n1_chunk, nnew1 - n1lo) * (Pn / nnew1);
+      const long long even = (rx[x0 + nx] >> 1) - (rx[x0] >> 1), Nc = nx * P;
       Z2Chunk ch;
-      ch.off_blk = push(colblk);
-      ch.off_pos = push(colpos);
-      for (int b = 0; b < 2; ++b) {
-        ch.off_list[b] = push(lst[b]);
-        ch.L[b] = (long long)lst[b].size();
-        maxL = std::max(maxL, ch.L[b]);
-      }
+      ch.x0 = x0;
+      ch.L[0] = even * ycnt[0] + (nx - even) * ycnt[1];
+      ch.L[1] = Nc - ch.L[0];
+      ch.off_blk = moff_full;
+      ch.off_pos = ch.off_blk + Nc;
+      ch.off_list[0] = ch.off_pos + Nc;
+      ch.off_list[1] = ch.off_list[0] + ch.L[0];
+      moff_full = (ch.off_list[1] + ch.L[1] + 63) / 64 * 64;
+      maxL = std::max(maxL, std::max(ch.L[0], ch.L[1]));
       zch.push_back(ch);
     }
     if (sl_chunk > 1) {
       // several slices a pass: the column maps of a pass (block, position, the two lists) are expanded
       // on the device from those of one slice
-      moff_full = ((long long)hmap.size() + 63) / 64 * 64;
       maxL = 0;
       for (int sl = sl_lo; sl < sl_hi; sl += sl_chunk) {
         long long l2[2];
@@ -1617,10 +1645,12 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
         maxL = std::max(maxL, std::max(l2[0], l2[1]));
       }
     }
-    CHECK_ALLOC(dev_alloc(c, c->Zmap, sizeof(int) * (sl_chunk > 1 ? moff_full + 4 * Nsub : (long long)hmap.size())));
-    if (cudaMemcpyAsync(c->Zmap.p, hmap.data(), sizeof(int) * hmap.size(), cudaMemcpyHostToDevice, s) !=
-        cudaSuccess)
+    CHECK_ALLOC(dev_alloc(c, c->Zmap, sizeof(int) * (sl_chunk > 1 ? moff_full + 4 * Nsub : moff_full)));
+    if (cudaMemcpyAsync(c->Zmap.p, hmap.data(), sizeof(int) * map_upload, cudaMemcpyHostToDevice, s) != cudaSuccess)
       return cuda_status(c) == HOTRG_OK ? (c->poisoned = HOTRG_ECUDA) : HOTRG_ECUDA;
+    for (const Z2Chunk& ch : zch)
+      launch_z2_columns((int*)c->Zmap.p, moff_rx + ch.x0, moff_ry, (int)((ch.L[0] + ch.L[1]) / P), (int)P, ycnt[0],
+                        ch.off_blk, ch.off_pos, ch.off_list[0], ch.off_list[1], s);
   }
   const int* zmap = (const int*)c->Zmap.p;
   // split form with Z2 blocks: the last prime stage writes the B blocks directly (no

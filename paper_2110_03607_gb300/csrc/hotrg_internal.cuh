@@ -296,6 +296,21 @@ void launch_z2_reduce_sym(const double* p0, int ns0, int m0, const double* p1, i
                           const int* blk, const int* pos, int m, double* S, cudaStream_t s);
 void launch_z2_reduce_sum_t(const double* p0, int ns0, int m0, const double* p1, int ns1, int m1,
                             const int* blk, const int* pos, int m, double* dS, cudaStream_t s);
+struct Z2Sum {
+  int nhi, nlo;             // the two halves of the summed index
+  int even_lo;              // lo values of even parity
+  int rank_hi, rank_lo;     // tables among the ints: even ones before << 1 | parity, same ones before << 1 | parity
+  long long even_all;       // k of even parity
+  long long off_hi, off_lo; // tables of element offsets
+  long long out;            // the K offsets written
+};
+struct Z2SumDesc {
+  int n;
+  Z2Sum sum[4 * (kMaxD - 1)];
+};
+void launch_z2_sum_offsets(long long* base, long long n64, const Z2SumDesc& d, cudaStream_t s);
+void launch_z2_columns(int* map, long long rx, long long ry, int nx, int P, int even_y, long long blk, long long pos,
+                       long long list0, long long list1, cudaStream_t s);
 void launch_z2_expand(const int* blk, const int* pos, int ns, int l0, int l1, int slices, unsigned qmask, int* fblk,
                       int* fpos, int* list0, int* list1, cudaStream_t s);
 void launch_z2_gather_split(const double* src, long long ld, const int* rowmap, int nrows,

@@ -141,6 +141,58 @@ __global__ void z2_expand_kernel(const int* __restrict__ blk, const int* __restr
   }
 }
 
+// Z2Sum: the element offsets of a Gram's summed index k = hi nlo + lo, even parity first, each parity in
+// the order of k.  Before hi stand E even and hi - E odd halves, each with even_lo or nlo - even_lo
+// elements of a parity, so the place of k needs no scan.
+__global__ void z2_sum_offsets_kernel(long long* base, long long n64, Z2SumDesc d) {
+  const Z2Sum& z = d.sum[blockIdx.y];
+  const int* h32 = (const int*)(base + n64);
+  const long long K = (long long)z.nhi * z.nlo;
+  for (long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x; k < K; k += (long long)gridDim.x * blockDim.x) {
+    const int hi = (int)(k / z.nlo), lo = (int)(k - (long long)hi * z.nlo);
+    const int rh = h32[z.rank_hi + hi], rl = h32[z.rank_lo + lo];
+    const int par = (rh ^ rl) & 1;
+    const long long even = rh >> 1, odd = hi - even;
+    const long long c0 = par ? z.nlo - z.even_lo : z.even_lo, c1 = z.nlo - c0;   // per even, per odd half
+    base[z.out + (par ? z.even_all : 0) + even * c0 + odd * c1 + (rl >> 1)] = base[z.off_hi + hi] + base[z.off_lo + lo];
+  }
+}
+
+void launch_z2_sum_offsets(long long* base, long long n64, const Z2SumDesc& d, cudaStream_t s) {
+  long long most = 1;
+  for (int i = 0; i < d.n; ++i) most = d.sum[i].nhi * (long long)d.sum[i].nlo > most ? d.sum[i].nhi * (long long)d.sum[i].nlo : most;
+  long long bx = (most + 255) / 256;
+  if (bx > 256) bx = 256;
+  z2_sum_offsets_kernel<<<dim3((unsigned)bx, (unsigned)d.n), 256, 0, s>>>(base, n64, d);
+  ++g_launches;
+}
+
+// the maps of nx P bottleneck columns n = x P + y from the ranks of x and y, as above
+__global__ void z2_columns_kernel(int* map, long long rx, long long ry, int nx, int P, int even_y, long long blk,
+                                  long long pos, long long list0, long long list1) {
+  const int e0 = map[rx] >> 1;
+  const long long total = (long long)nx * P;
+  for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < total;
+       n += (long long)gridDim.x * blockDim.x) {
+    const int x = (int)(n / P), y = (int)(n - (long long)x * P);
+    const int a = map[rx + x], b = map[ry + y];
+    const int par = (a ^ b) & 1, even = (a >> 1) - e0, odd = x - even;
+    const int c0 = par ? P - even_y : even_y;
+    const int p = even * c0 + odd * (P - c0) + (b >> 1);
+    map[blk + n] = par;
+    map[pos + n] = p;
+    map[(par ? list1 : list0) + p] = (int)n;
+  }
+}
+
+void launch_z2_columns(int* map, long long rx, long long ry, int nx, int P, int even_y, long long blk, long long pos,
+                       long long list0, long long list1, cudaStream_t s) {
+  long long bx = ((long long)nx * P + 255) / 256;
+  if (bx > 1024) bx = 1024;
+  z2_columns_kernel<<<(unsigned)bx, 256, 0, s>>>(map, rx, ry, nx, P, even_y, blk, pos, list0, list1);
+  ++g_launches;
+}
+
 void launch_z2_expand(const int* blk, const int* pos, int ns, int l0, int l1, int slices, unsigned qmask, int* fblk,
                       int* fpos, int* list0, int* list1, cudaStream_t s) {
   unsigned bx = (unsigned)((ns + 255) / 256);
