@@ -311,6 +311,7 @@ struct Z2SumDesc {
 void launch_z2_sum_offsets(long long* base, long long n64, const Z2SumDesc& d, cudaStream_t s);
 void launch_z2_columns(int* map, long long rx, long long ry, int nx, int P, int even_y, long long blk, long long pos,
                        long long list0, long long list1, cudaStream_t s);
+void launch_z2_one_block(int* blk, int* pos, int* kcat, int* kpad, int n, int np, int last, cudaStream_t s);
 void launch_z2_expand(const int* blk, const int* pos, int ns, int l0, int l1, int slices, unsigned qmask, int* fblk,
                       int* fpos, int* list0, int* list1, cudaStream_t s);
 void launch_z2_gather_split(const double* src, long long ld, const int* rowmap, int nrows,

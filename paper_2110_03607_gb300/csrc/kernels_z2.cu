@@ -193,6 +193,29 @@ void launch_z2_columns(int* map, long long rx, long long ry, int nx, int P, int 
   ++g_launches;
 }
 
+// Maps of the dense form as one block: list position o holds index (o % rest) last + o / rest (rest = n /
+// last: the fastest index goes slowest); blk and pos per index, list (twice: kcat, and kpad padded with
+// -1) per position.  last = 1 and no lists: the identity.
+__global__ void z2_one_block_kernel(int* blk, int* pos, int* kcat, int* kpad, int n, int np, int last) {
+  const int rest = n / last;
+  for (int o = blockIdx.x * blockDim.x + threadIdx.x; o < n || o < np; o += gridDim.x * blockDim.x) {
+    if (o < n) {
+      const int r = (o % rest) * last + o / rest;
+      blk[r] = 0;
+      pos[r] = o;
+      if (kcat) kcat[o] = r;
+    }
+    if (o < np) kpad[o] = o < n ? (o % rest) * last + o / rest : -1;
+  }
+}
+
+void launch_z2_one_block(int* blk, int* pos, int* kcat, int* kpad, int n, int np, int last, cudaStream_t s) {
+  int bx = ((n > np ? n : np) + 255) / 256;
+  if (bx > 1024) bx = 1024;
+  z2_one_block_kernel<<<bx, 256, 0, s>>>(blk, pos, kcat, kpad, n, np, last);
+  ++g_launches;
+}
+
 void launch_z2_expand(const int* blk, const int* pos, int ns, int l0, int l1, int slices, unsigned qmask, int* fblk,
                       int* fpos, int* list0, int* list1, cudaStream_t s) {
   unsigned bx = (unsigned)((ns + 255) / 256);

@@ -8,9 +8,12 @@
 // multiply-adds and half of the loads of the dense stage.  The terms that remain are summed in the order
 // of the dense stage, and those left out are exact zeros: the results are the same bit for bit.
 //
-// The prime stage is bound by instruction issue (splitting into pieces and storing them is half of it)
-// and close to the rate at which HBM takes its output; the non-prime stage by its shared-memory reads of
-// U~ (one 16-byte read for 4 multiply-adds) and the reads of C.
+// The dense form runs through the same kernels as one block with one parity.
+//
+// 3D chi = 16, one c'-slice (0.8 GB of B written, 0.54 GB of C read): prime 0.85 -> 0.30 ms, bound by
+// instruction issue (67 % of the slots: forming, packing and storing the pieces is half of it), 2.7 TB/s
+// written; non-prime 0.57 -> 0.22 ms, bound by the L1 pipe (reads of U~, then of C), 2.4 TB/s read.  Per step
+// at chi = 20: 108 -> 47 and 119 -> 32 ms.
 #include "hotrg_internal.cuh"
 
 namespace hotrg {
@@ -90,10 +93,11 @@ __device__ void load_u(const Z2Chain& p, float* us, Lists* l) {
   __syncthreads();
 }
 
-template <int PF>
-__device__ __forceinline__ void store_pair(char* o, long long pbytes, int npieces, float v0, float v1) {
+template <int PF, int NP>
+__device__ __forceinline__ void store_pair(char* o, long long pbytes, float v0, float v1) {
   if (PF == PIECE_TF32) {
-    for (int q = 0; q < npieces; ++q) {
+#pragma unroll
+    for (int q = 0; q < NP; ++q) {
       const float w0 = round_tf32(v0), w1 = round_tf32(v1);
       *reinterpret_cast<float2*>(o) = make_float2(w0, w1);
       v0 -= w0;
@@ -101,7 +105,8 @@ __device__ __forceinline__ void store_pair(char* o, long long pbytes, int npiece
       o += pbytes;
     }
   } else {
-    for (int q = 0; q < npieces; ++q) {
+#pragma unroll
+    for (int q = 0; q < NP; ++q) {
       const __nv_bfloat162 w = __floats2bfloat162_rn(v0, v1);
       *reinterpret_cast<__nv_bfloat162*>(o) = w;
       v0 -= __low2float(w);
@@ -118,7 +123,7 @@ __device__ __forceinline__ void store_pair(char* o, long long pbytes, int npiece
 // (g1, n, nc), column k = (rho, h, a) at its position in the list of k's parity.
 // A warp takes 64 positions of one block's K list, two neighbours a lane (so that pieces are stored in
 // pairs), and goes through GPER row groups (g1, nc) with them: the positions are decoded once.
-template <int PF, int NH>
+template <int PF, int NP, int NH>
 __global__ void __launch_bounds__(256, NH <= 8 ? 3 : (NH <= 16 ? 2 : 1)) z2_prime_kernel(Z2Chain p, const float* __restrict__ in, int H, int chi_c, int P,
                                                        int groups, int gper, const int* __restrict__ kcat, int rb0,
                                                        int R, Z2Blocks zo) {
@@ -133,7 +138,10 @@ __global__ void __launch_bounds__(256, NH <= 8 ? 3 : (NH <= 16 ? 2 : 1)) z2_prim
   const int pn0 = (int)(p.mask_n & 1u);
   const long long tasks = (long long)chunks * ((groups + gper - 1) / gper);
   const int hp = hat_pitch<NH>(p.chi);
-  constexpr int UB = NH <= 8 ? 8 : 4;
+  constexpr int UB = 4;
+  __shared__ int bo[64];   // offset of the i-th check index of a parity
+  if (threadIdx.x < 64) bo[threadIdx.x] = (threadIdx.x & 31) < (threadIdx.x < 32 ? nb0 : nb1) ? l.b[threadIdx.x >> 5][threadIdx.x & 31] * H : 0;
+  __syncthreads();
   for (long long t = (long long)blockIdx.x * 8 + (threadIdx.x >> 5); t < tasks; t += (long long)gridDim.x * 8) {
     const int chunk = (int)(t % chunks);
     const int g_lo = (int)(t / chunks) * gper, g_hi = min(groups, g_lo + gper);
@@ -190,16 +198,17 @@ __global__ void __launch_bounds__(256, NH <= 8 ? 3 : (NH <= 16 ? 2 : 1)) z2_prim
       if (shared_a) {
         const int pb = sig ^ pa0, m = pb ? nb1 : nb0;
         const float* row = us + a0 * hp + (pb ? nb0 : 0) * NH;
-        const int* bl = l.b[pb];
+        const int* bl = bo + pb * 32;
+        const float *xa = x + o0, *xb = x + o1;
         for (int i = 0; i < m; i += UB) {
           float x0[UB], x1[UB];
 #pragma unroll
-          for (int u = 0; u < UB; ++u) {
-            const bool in_list = i + u < m;
-            const long long ofs = in_list ? (long long)bl[i + u] * H : 0;
-            x0[u] = in_list ? x[o0 + ofs] : 0.0f;
-            x1[u] = in_list ? x[o1 + ofs] : 0.0f;
-          }
+          for (int u = 0; u < UB; ++u)
+            if (i + u < m) {
+              const int ofs = bl[i + u];
+              x0[u] = xa[ofs];
+              x1[u] = xb[ofs];
+            }
 #pragma unroll
           for (int u = 0; u < UB; ++u) {
             if (i + u >= m) break;
@@ -230,116 +239,154 @@ __global__ void __launch_bounds__(256, NH <= 8 ? 3 : (NH <= 16 ? 2 : 1)) z2_prim
         if (n >= ncols) break;
         const int z = __shfl_sync(0xffffffffu, pos, n);
         // past the end of the list stands the K padding, which reads as zero
-        if (ok0) store_pair<PF>(ob + z * ldb, psb, zo.npieces, v0, ok1 ? v1 : 0.0f);
+        if (ok0) store_pair<PF, NP>(ob + z * ldb, psb, v0, ok1 ? v1 : 0.0f);
         if (n + 1 >= ncols) break;
         const int z1 = __shfl_sync(0xffffffffu, pos, n + 1);
-        if (ok0) store_pair<PF>(ob + z1 * ldb, psb, zo.npieces, w0, ok1 ? w1 : 0.0f);
+        if (ok0) store_pair<PF, NP>(ob + z1 * ldb, psb, w0, ok1 ? w1 : 0.0f);
       }
     }
   }
 }
 
 // First non-prime stage.  C rows (rr, a), columns (cc, b); output [rr][cc][n], FP32, zero where the
-// parities forbid it.  A warp takes 32 neighbouring cc of one rr.  In a block's row the check indices of
-// one cc stand next to each other (VEC: class sizes and so their starts are multiples of VEC), so a
-// lane's terms for one hat index are one or two vector loads and a warp reads a contiguous stretch.
+// parities forbid it.  A warp takes 128 neighbouring cc of one rr and goes through those of either parity
+// by themselves, two a lane: the rows of U~ are then the same for all its lanes and serve two outputs a
+// read (with both parities together and one output a lane these reads took 92 % of the L1 pipe).  In a
+// block's row the check indices of one cc stand next to each other (VEC: class sizes, and so their
+// starts, are multiples of VEC), so that a lane's terms for one hat index are one or two vector loads of
+// whole sectors.
+constexpr int kCcs = 128;
 template <int NH, int VEC>
-__global__ void __launch_bounds__(256, NH <= 8 ? 4 : (NH <= 12 ? 3 : 2)) z2_nonprime_kernel(Z2Chain p, Z2In zi, long long rrs, long long ccs,
+__global__ void __launch_bounds__(256, NH <= 8 ? 3 : (NH <= 16 ? 2 : 1)) z2_nonprime_kernel(Z2Chain p, Z2In zi, long long rrs, long long ccs,
                                                           float* __restrict__ out) {
   extern __shared__ __align__(16) unsigned char smem_u[];
   __shared__ Lists l;
+  __shared__ unsigned char s_list[8][kCcs];
   float* us = reinterpret_cast<float*>(smem_u);
   const int hp = hat_pitch<NH>(p.chi);
   load_u<NH>(p, us, &l);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float* tile = us + p.chi * hp + warp * 32 * (p.nn + 1);
-  // class sizes (selects, not arrays: an indexed array would live in local memory)
+  float* tile = us + p.chi * hp + warp * 64 * (p.nn + 1);
+  unsigned char* list = s_list[warp];   // even ones from the front, odd ones from the back
   const int nb1 = __popc(p.mask_b), nb0 = p.chi - nb1, nc1 = __popc(p.mask_n), nc0 = p.nn - nc1;
   const int pb0 = (int)(p.mask_b & 1u);
   constexpr int MB = NH <= 16 ? NH : 8;
-  const long long chunks = (ccs + 31) / 32, tasks = rrs * chunks;
+  const long long chunks = (ccs + kCcs - 1) / kCcs, tasks = rrs * chunks;
   for (long long t = (long long)blockIdx.x * 8 + warp; t < tasks; t += (long long)gridDim.x * 8) {
-    const long long rr = t / chunks, cc0 = (t - rr * chunks) * 32;
-    const int live = (int)min(32LL, ccs - cc0);
-    const long long cc = cc0 + min(lane, live - 1);
+    const long long rr = t / chunks, c0 = (t - rr * chunks) * kCcs;
+    const int live = (int)min((long long)kCcs, ccs - c0);
     // rows: lane a holds the position and block of (rr, a)
     unsigned zr = 0u;
     if (lane < p.chi) zr = (unsigned)zi.rpos[rr * p.chi + lane] | ((unsigned)zi.rblk[rr * p.chi + lane] << 31);
-    // columns: the block of (cc, b) is blk0 ^ par(b); the first of each parity
-    const int cpar = zi.cblk[cc * p.chi] ^ pb0 ^ zi.q;
-    const int s0 = nb0 ? zi.cpos[cc * p.chi + l.b[0][0]] : 0, s1 = nb1 ? zi.cpos[cc * p.chi + l.b[1][0]] : 0;
-    u64 acc[NH / 2];
+    // the block of column (cc, b) is cpar ^ par(b)
+    int count[2] = {0, 0};
 #pragma unroll
-    for (int n = 0; n < NH / 2; ++n) acc[n] = 0ULL;
-    int sig = 0;   // the parity of the new indices with a nonzero result: that of (rr, cc)
-    // the terms of one hat index: their count, their rows of U~ and (up to MB of them) their values; the
-    // next hat index is read while one is summed
-    auto fetch = [&](int a, int& m, const float*& ur, const float*& x, float (&v)[MB]) {
-      const unsigned z = __shfl_sync(0xffffffffu, zr, a);
-      const int rb = (int)(z >> 31), pb = rb ^ cpar;
-      if (a == 0) sig = pb ^ (int)(p.mask_b & 1u);
-      const float* cr = rb ? zi.c[1] : zi.c[0];
-      m = cr ? (pb ? nb1 : nb0) : 0;
-      ur = us + a * hp + (pb ? nb0 : 0) * NH;
-      x = cr + (long long)(z & 0x7fffffffu) * zi.ld + (pb ? s1 : s0);
-      if (VEC == 4) {
-#pragma unroll
-        for (int i = 0; i + 3 < MB; i += 4)
-          if (i < m) *reinterpret_cast<float4*>(v + i) = *reinterpret_cast<const float4*>(x + i);
-      } else if (VEC == 2) {
-#pragma unroll
-        for (int i = 0; i + 1 < MB; i += 2)
-          if (i < m) *reinterpret_cast<float2*>(v + i) = *reinterpret_cast<const float2*>(x + i);
-      } else {
-#pragma unroll
-        for (int i = 0; i < MB; ++i)
-          if (i < m) v[i] = x[i];
-      }
-    };
-    int m;
-    const float *ur, *x;
-    alignas(16) float v[MB];
-    fetch(0, m, ur, x, v);
-    for (int a = 0; a < p.chi; ++a) {
-      int m1 = 0;
-      const float *ur1 = ur, *x1 = x;
-      alignas(16) float v1[MB];
-      if (a + 1 < p.chi) fetch(a + 1, m1, ur1, x1, v1);
-      u64 part[NH / 2];
-#pragma unroll
-      for (int n = 0; n < NH / 2; ++n) part[n] = 0ULL;
-#pragma unroll
-      for (int i = 0; i < MB; ++i)
-        if (i < m) fma_row2<NH>(v[i], ur + i * NH, part);
-      for (int i = MB; i < m; ++i) fma_row2<NH>(x[i], ur + i * NH, part);
-#pragma unroll
-      for (int n = 0; n < NH / 2; ++n) acc[n] = add2(acc[n], part[n]);
-      m = m1;
-      ur = ur1;
-      x = x1;
-#pragma unroll
-      for (int i = 0; i < MB; ++i) v[i] = v1[i];
+    for (int q = 0; q < kCcs / 32; ++q) {
+      const int i = q * 32 + lane;
+      const bool ok = i < live;
+      const int cpar = ok ? zi.cblk[(c0 + i) * p.chi] ^ pb0 ^ zi.q : 0;
+      const unsigned odd = __ballot_sync(0xffffffffu, ok && cpar), even = __ballot_sync(0xffffffffu, ok && !cpar);
+      const unsigned below = (1u << lane) - 1u;
+      if (ok) list[cpar ? kCcs - 1 - count[1] - __popc(odd & below) : count[0] + __popc(even & below)] = (unsigned char)i;
+      count[0] += __popc(even);
+      count[1] += __popc(odd);
     }
-    // through shared memory, so that the warp's outputs leave in one contiguous stretch
-    const int ncols = sig ? nc1 : nc0;
-    float* mine = tile + lane * (p.nn + 1);
-#pragma unroll
-    for (int n = 0; n < NH; n += 2) {
-      float v, w;
-      unpack2(acc[n / 2], v, w);
-      if (n < ncols) mine[l.n[sig][n]] = v;
-      if (n + 1 < ncols) mine[l.n[sig][n + 1]] = w;
-    }
-    for (int n = 0; n < p.nn - ncols; ++n) mine[l.n[sig ^ 1][n]] = 0.0f;
     __syncwarp();
-    float* o = out + (rr * ccs + cc0) * p.nn;
-    int i = lane / p.nn, n = lane - i * p.nn;
-    for (int e = lane; e < live * p.nn; e += 32) {
-      o[e] = tile[i * (p.nn + 1) + n];
-      n += 32;
-      while (n >= p.nn) {
-        n -= p.nn;
-        ++i;
+#pragma unroll 1
+    for (int cpar = 0; cpar < 2; ++cpar) {
+      const int cnt = cpar ? count[1] : count[0];
+#pragma unroll 1
+      for (int base = 0; base < cnt; base += 64) {
+        const int e0 = min(base + lane, cnt - 1), e1 = min(base + lane + 32, cnt - 1);
+        const long long k0 = (c0 + list[cpar ? kCcs - 1 - e0 : e0]) * p.chi, k1 = (c0 + list[cpar ? kCcs - 1 - e1 : e1]) * p.chi;
+        // the first column of either class of check indices
+        const int s00 = nb0 ? zi.cpos[k0 + l.b[0][0]] : 0, s01 = nb1 ? zi.cpos[k0 + l.b[1][0]] : 0;
+        const int s10 = nb0 ? zi.cpos[k1 + l.b[0][0]] : 0, s11 = nb1 ? zi.cpos[k1 + l.b[1][0]] : 0;
+        u64 acc0[NH / 2], acc1[NH / 2];
+#pragma unroll
+        for (int n = 0; n < NH / 2; ++n) acc0[n] = acc1[n] = 0ULL;
+        int sig = 0;   // the parity of the new indices with a nonzero result: that of (rr, cc)
+#pragma unroll 1
+        for (int a = 0; a < p.chi; ++a) {
+          const unsigned z = __shfl_sync(0xffffffffu, zr, a);
+          const int rb = (int)(z >> 31), pb = rb ^ cpar, m = pb ? nb1 : nb0;
+          if (a == 0) sig = pb ^ pb0;
+          const float* cr = rb ? zi.c[1] : zi.c[0];
+          if (!cr) continue;
+          cr += (long long)(z & 0x7fffffffu) * zi.ld;
+          const float *x0 = cr + (pb ? s01 : s00), *x1 = cr + (pb ? s11 : s10);
+          const float* ur = us + a * hp + (pb ? nb0 : 0) * NH;
+          u64 part0[NH / 2], part1[NH / 2];
+#pragma unroll
+          for (int n = 0; n < NH / 2; ++n) part0[n] = part1[n] = 0ULL;
+          for (int i0 = 0; i0 < m; i0 += MB) {
+            alignas(16) float v0[MB], v1[MB];
+#pragma unroll
+            for (int i = 0; i < MB; i += VEC)
+              if (i0 + i < m) {
+                if constexpr (VEC == 4) {
+                  *reinterpret_cast<float4*>(v0 + i) = *reinterpret_cast<const float4*>(x0 + i0 + i);
+                  *reinterpret_cast<float4*>(v1 + i) = *reinterpret_cast<const float4*>(x1 + i0 + i);
+                } else if constexpr (VEC == 2) {
+                  *reinterpret_cast<float2*>(v0 + i) = *reinterpret_cast<const float2*>(x0 + i0 + i);
+                  *reinterpret_cast<float2*>(v1 + i) = *reinterpret_cast<const float2*>(x1 + i0 + i);
+                } else {
+                  v0[i] = x0[i0 + i];
+                  v1[i] = x1[i0 + i];
+                }
+              }
+#pragma unroll
+            for (int i = 0; i < MB; ++i) {
+              if (i0 + i >= m) break;
+              const float* row = ur + (i0 + i) * NH;
+              const u64 xx0 = pack2(v0[i], v0[i]), xx1 = pack2(v1[i], v1[i]);
+#pragma unroll
+              for (int n = 0; n < NH; n += 4) {
+                const ulonglong2 u = *reinterpret_cast<const ulonglong2*>(row + n);
+                part0[n / 2] = fma2(xx0, u.x, part0[n / 2]);
+                part0[n / 2 + 1] = fma2(xx0, u.y, part0[n / 2 + 1]);
+                part1[n / 2] = fma2(xx1, u.x, part1[n / 2]);
+                part1[n / 2 + 1] = fma2(xx1, u.y, part1[n / 2 + 1]);
+              }
+            }
+          }
+#pragma unroll
+          for (int n = 0; n < NH / 2; ++n) {
+            acc0[n] = add2(acc0[n], part0[n]);
+            acc1[n] = add2(acc1[n], part1[n]);
+          }
+        }
+        // through shared memory, so that the outputs of a cc leave together
+        const int ncols = sig ? nc1 : nc0;
+        float *mine0 = tile + lane * (p.nn + 1), *mine1 = mine0 + 32 * (p.nn + 1);
+#pragma unroll
+        for (int n = 0; n < NH; n += 2) {
+          float v, w, v1, w1;
+          unpack2(acc0[n / 2], v, w);
+          unpack2(acc1[n / 2], v1, w1);
+          if (n < ncols) {
+            mine0[l.n[sig][n]] = v;
+            mine1[l.n[sig][n]] = v1;
+          }
+          if (n + 1 < ncols) {
+            mine0[l.n[sig][n + 1]] = w;
+            mine1[l.n[sig][n + 1]] = w1;
+          }
+        }
+        for (int n = 0; n < p.nn - ncols; ++n) mine0[l.n[sig ^ 1][n]] = mine1[l.n[sig ^ 1][n]] = 0.0f;
+        __syncwarp();
+        const int rows = min(64, cnt - base);
+        int i = lane / p.nn, n = lane - i * p.nn;
+        for (int e = lane; e < rows * p.nn; e += 32) {
+          const int k = base + i;
+          out[(rr * ccs + c0 + list[cpar ? kCcs - 1 - k : k]) * p.nn + n] = tile[i * (p.nn + 1) + n];
+          n += 32;
+          while (n >= p.nn) {
+            n -= p.nn;
+            ++i;
+          }
+        }
+        __syncwarp();
       }
     }
     __syncwarp();
@@ -361,11 +408,11 @@ bool room(K kernel, size_t smem) {
          cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess;
 }
 
-template <int PF, int NH>
+template <int PF, int NP, int NH>
 bool prime_nh(const Z2Chain& p, const float* in, int H, int chi_c, int P, int groups, const int* kcat, int rb0, int R,
               const Z2Blocks& zo, int ctas_per_sm, cudaStream_t s) {
   const size_t smem = sizeof(float) * p.chi * (p.chi * NH + 4);
-  auto kernel = z2_prime_kernel<PF, NH>;
+  auto kernel = z2_prime_kernel<PF, NP, NH>;
   if (!room(kernel, smem)) return false;
   const long long chunks = (rb0 + 63) / 64 + (R - rb0 + 63) / 64;
   const long long warps = 8LL * ctas_per_sm * sm_count();
@@ -379,23 +426,25 @@ bool prime_nh(const Z2Chain& p, const float* in, int H, int chi_c, int P, int gr
   return true;
 }
 
-template <int PF>
+template <int PF, int NP>
 bool prime_pf(const Z2Chain& p, const float* in, int H, int chi_c, int P, int groups, const int* kcat, int rb0, int R,
               const Z2Blocks& zo, int cps, cudaStream_t s) {
   const int w = half_width(p);
-  if (w <= 4) return prime_nh<PF, 4>(p, in, H, chi_c, P, groups, kcat, rb0, R, zo, cps, s);
-  if (w <= 8) return prime_nh<PF, 8>(p, in, H, chi_c, P, groups, kcat, rb0, R, zo, cps, s);
-  if (w <= 12) return prime_nh<PF, 12>(p, in, H, chi_c, P, groups, kcat, rb0, R, zo, cps, s);
-  if (w <= 16) return prime_nh<PF, 16>(p, in, H, chi_c, P, groups, kcat, rb0, R, zo, cps, s);
-  return prime_nh<PF, 32>(p, in, H, chi_c, P, groups, kcat, rb0, R, zo, cps, s);
+  if (w <= 4) return prime_nh<PF, NP, 4>(p, in, H, chi_c, P, groups, kcat, rb0, R, zo, cps, s);
+  if (w <= 8) return prime_nh<PF, NP, 8>(p, in, H, chi_c, P, groups, kcat, rb0, R, zo, cps, s);
+  if (w <= 12) return prime_nh<PF, NP, 12>(p, in, H, chi_c, P, groups, kcat, rb0, R, zo, cps, s);
+  if (w <= 16) return prime_nh<PF, NP, 16>(p, in, H, chi_c, P, groups, kcat, rb0, R, zo, cps, s);
+  if (w <= 20) return prime_nh<PF, NP, 20>(p, in, H, chi_c, P, groups, kcat, rb0, R, zo, cps, s);
+  if (w <= 24) return prime_nh<PF, NP, 24>(p, in, H, chi_c, P, groups, kcat, rb0, R, zo, cps, s);
+  return prime_nh<PF, NP, 32>(p, in, H, chi_c, P, groups, kcat, rb0, R, zo, cps, s);
 }
 
 template <int NH, int VEC>
 bool nonprime_one(const Z2Chain& p, const Z2In& zi, long long rrs, long long ccs, float* out, int cps, cudaStream_t s) {
-  const size_t smem = sizeof(float) * (p.chi * (p.chi * NH + 4) + 8 * 32 * (p.nn + 1));
+  const size_t smem = sizeof(float) * (p.chi * (p.chi * NH + 4) + 8 * 64 * (p.nn + 1));
   auto kernel = z2_nonprime_kernel<NH, VEC>;
   if (!room(kernel, smem)) return false;
-  long long blocks = (rrs * ((ccs + 31) / 32) + 7) / 8;
+  long long blocks = (rrs * ((ccs + kCcs - 1) / kCcs) + 7) / 8;
   if (blocks > (long long)cps * sm_count()) blocks = (long long)cps * sm_count();
   kernel<<<(unsigned)blocks, 256, smem, s>>>(p, zi, rrs, ccs, out);
   ++g_launches;
@@ -414,10 +463,15 @@ bool nonprime_nh(const Z2Chain& p, const Z2In& zi, long long rrs, long long ccs,
 
 bool launch_z2_prime(const Z2Chain& p, const float* in, int H, int chi_c, int P, long long groups, const int* kcat,
                      int rb0, int R, const Z2Blocks& zo, int pfmt, int ctas_per_sm, cudaStream_t s) {
-  if (groups < 1 || groups >= (1LL << 31)) return false;
-  return pfmt == PIECE_TF32
-             ? prime_pf<PIECE_TF32>(p, in, H, chi_c, P, (int)groups, kcat, rb0, R, zo, ctas_per_sm, s)
-             : prime_pf<PIECE_BF16>(p, in, H, chi_c, P, (int)groups, kcat, rb0, R, zo, ctas_per_sm, s);
+  if (groups < 1 || groups >= (1LL << 31) || zo.npieces < (pfmt == PIECE_TF32 ? 1 : 2) ||
+      zo.npieces > (pfmt == PIECE_TF32 ? 2 : 3))
+    return false;
+  const int n = zo.npieces;
+  if (pfmt == PIECE_TF32)
+    return n == 1 ? prime_pf<PIECE_TF32, 1>(p, in, H, chi_c, P, (int)groups, kcat, rb0, R, zo, ctas_per_sm, s)
+                  : prime_pf<PIECE_TF32, 2>(p, in, H, chi_c, P, (int)groups, kcat, rb0, R, zo, ctas_per_sm, s);
+  return n == 2 ? prime_pf<PIECE_BF16, 2>(p, in, H, chi_c, P, (int)groups, kcat, rb0, R, zo, ctas_per_sm, s)
+                : prime_pf<PIECE_BF16, 3>(p, in, H, chi_c, P, (int)groups, kcat, rb0, R, zo, ctas_per_sm, s);
 }
 
 bool launch_z2_nonprime(const Z2Chain& p, const Z2In& zi, long long rrs, long long ccs, float* out, int ctas_per_sm,
@@ -427,6 +481,8 @@ bool launch_z2_nonprime(const Z2Chain& p, const Z2In& zi, long long rrs, long lo
   if (w <= 8) return nonprime_nh<8>(p, zi, rrs, ccs, out, ctas_per_sm, s);
   if (w <= 12) return nonprime_nh<12>(p, zi, rrs, ccs, out, ctas_per_sm, s);
   if (w <= 16) return nonprime_nh<16>(p, zi, rrs, ccs, out, ctas_per_sm, s);
+  if (w <= 20) return nonprime_nh<20>(p, zi, rrs, ccs, out, ctas_per_sm, s);
+  if (w <= 24) return nonprime_nh<24>(p, zi, rrs, ccs, out, ctas_per_sm, s);
   return nonprime_nh<32>(p, zi, rrs, ccs, out, ctas_per_sm, s);
 }
 
