@@ -1750,11 +1750,9 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
                              za + pbytes * npieces * Rb[0] * Kpb[0], Rb[1] * Kpb[1], npieces, pfmt, s);
     } else {
       CHECK_ALLOC(dev_alloc(c, c->Ap, pbytes * npieces * R * Kpad));
-      if (Kpad != R) cudaMemsetAsync(c->Ap.p, 0, pbytes * npieces * R * Kpad, s);
       launch_split(Tc, R, R, R, c->Ap.p, Kpad, R * Kpad, npieces, pfmt, s);
       if (tangent) {
         CHECK_ALLOC(dev_alloc(c, c->dAp, pbytes * npieces * R * Kpad));
-        if (Kpad != R) cudaMemsetAsync(c->dAp.p, 0, pbytes * npieces * R * Kpad, s);
         launch_split((const double*)c->dT.p, R, R, R, c->dAp.p, Kpad, R * Kpad, npieces, pfmt, s);
       }
     }
@@ -2427,8 +2425,6 @@ int hotrg_gemm_nt(int mode, int M, int N, int K, const double* A, const double* 
       if (r == 0) launch_gemm_nt_f64((const double*)dA, K, (const double*)dB, K, (double*)dC, N, 0, M, N, K, 1, 0, s);
       if (r < 0) fail(HOTRG_ECUDA);
     } else {
-      cudaMemset(pA, 0, pbytes * np * M * Kpad);
-      cudaMemset(pB, 0, pbytes * np * N * Kpad);
       launch_split((const double*)dA, M, K, K, pA, Kpad, M * Kpad, np, pfmt, s);
       launch_split((const double*)dB, N, K, K, pB, Kpad, N * Kpad, np, pfmt, s);
       int ta[6], tb[6];

@@ -125,24 +125,56 @@ __device__ __forceinline__ float round_tf32(float x) {
 }
 
 __device__ __forceinline__ __nv_bfloat16 bf16_rn(float x) { return __float2bfloat16_rn(x); }
-__device__ __forceinline__ __nv_bfloat16 bf16_rn(double x) { return __double2bfloat16(x); }
 
 // x as npieces pieces of format PF: piece p at element off + p * pstride of o
-template <int PF, typename T>
-__device__ __forceinline__ void store_pieces_as(void* o, long long off, long long pstride, int npieces, T x) {
+template <int PF>
+__device__ __forceinline__ void store_pieces_as(void* o, long long off, long long pstride, int npieces, float x) {
   if (PF == PIECE_TF32) {
     float* of = (float*)o + off;
     for (int p = 0; p < npieces; ++p) {
-      const float v = round_tf32((float)x);
+      const float v = round_tf32(x);
       of[p * pstride] = v;
-      x -= (T)v;
+      x -= v;
     }
   } else {
     __nv_bfloat16* ob = (__nv_bfloat16*)o + off;
     for (int p = 0; p < npieces; ++p) {
       const __nv_bfloat16 v = bf16_rn(x);
       ob[p * pstride] = v;
-      x -= (T)__bfloat162float(v);
+      x -= __bfloat162float(v);
+    }
+  }
+}
+// x as the sum of two FP32 numbers, x to 2^-47: the 24 leading bits, cut, and the rest.  In integer
+// arithmetic where the exponents allow it: the FP64 pipe converts and subtracts two a clock and SM.
+__device__ __forceinline__ void split_f32(double x, float& hi, float& lo) {
+  const unsigned top = (unsigned)__double2hiint(x), low = (unsigned)__double2loint(x);
+  const int e = (int)((top >> 20) & 0x7ff) - 1023;
+  if (e >= -100 && e < 127) {
+    const unsigned sign = top & 0x80000000u;
+    hi = __uint_as_float(sign | (unsigned)(e + 127) << 23 | (top & 0xfffffu) << 3 | low >> 29);
+    // 29 bits below, in units of 2^(e - 52)
+    lo = __uint2float_rn(low & 0x1fffffffu) * 1.862645149230957e-9f * __uint_as_float(sign | (unsigned)(e - 23 + 127) << 23);
+  } else {
+    hi = (float)x;
+    lo = (float)(x - (double)hi);
+  }
+}
+// FP64 input: the remainder after a piece is exact in FP32, the low part joins the last piece
+template <int PF>
+__device__ __forceinline__ void store_pieces_as(void* o, long long off, long long pstride, int npieces, double x) {
+  float r, lo;
+  split_f32(x, r, lo);
+  for (int p = 0; p < npieces; ++p) {
+    if (p == npieces - 1) r += lo;
+    if (PF == PIECE_TF32) {
+      const float v = round_tf32(r);
+      ((float*)o)[off + p * pstride] = v;
+      r -= v;
+    } else {
+      const __nv_bfloat16 v = bf16_rn(r);
+      ((__nv_bfloat16*)o)[off + p * pstride] = v;
+      r -= __bfloat162float(v);
     }
   }
 }
@@ -160,7 +192,8 @@ __device__ __forceinline__ void store_pieces(void* o, long long off, long long p
 void launch_init_ising(double* T, int d, double beta, double h, cudaStream_t s);
 void launch_permute(const double* in, double* out, int ndim, const long long* out_size,
                     const long long* in_stride, double scale, cudaStream_t s);
-// FP64 (in, + in2 when given) -> npieces pieces of format pfmt
+// FP64 (in, + in2 when given) -> npieces pieces of format pfmt, rows of ld_out elements (a multiple of 4)
+// with zeros behind cols
 void launch_split(const double* in, long long rows, long long cols, long long ld_in, void* out,
                   long long ld_out, long long piece_stride, int npieces, int pfmt, cudaStream_t s,
                   const double* in2 = nullptr);

@@ -92,11 +92,6 @@ extern "C" int hotrg_gemm_nt_noalloc(int mode, int M, int N, int K, const double
     __nv_bfloat16* pa = (__nv_bfloat16*)(base + off_a);
     __nv_bfloat16* pb = (__nv_bfloat16*)(base + off_b);
     float* c32 = (float*)(base + off_c);
-    // the pieces keep the previous call's contents: the K padding must read as zero
-    if (Kpad != K) {
-      if (cudaMemsetAsync(pa, 0, bytes_a, s) != cudaSuccess || cudaMemsetAsync(pb, 0, bytes_b, s) != cudaSuccess)
-        status = HOTRG_ECUDA;
-    }
     if (status == HOTRG_OK) {
       launch_split(A, M, K, K, pa, Kpad, (long long)M * Kpad, np, PIECE_BF16, s);
       launch_split(B, N, K, K, pb, Kpad, (long long)N * Kpad, np, PIECE_BF16, s);
