@@ -8,8 +8,8 @@
 // Two persistent kernels; launch_tc_gemm uses the CTA-pair one (HOTRG_TC_USE_PAIR).
 //
 // tc_gemm_pair_kernel (cta_group::2): a cluster of two CTAs on two SMs computes a
-// 256 x 256 tile of C; CTA 0 issues tcgen05.mma with M = 256, N = 256, K = 16.  CTA r
-// holds rows 128 r .. of the A tile and rows 128 r .. of the B tile, so each SM
+// 256 x 256 (or 256 x 128) tile of C; CTA 0 issues tcgen05.mma with M = 256, N = 256 (128), K = 16.  CTA r
+// holds rows 128 r .. of the A tile and its half of the rows of the B tile, so each SM
 // receives only half of the B tile: the per-SM copy rate, not the tensor pipe or the
 // L2, is what bounds the one-CTA form below.  K slabs of 128-byte rows (64 BF16 or 32
 // TF32, 128-byte swizzle), every piece of a slab in one ring stage (6 / npieces stages
@@ -332,11 +332,12 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 namespace {
 constexpr int P_TK = 64, P_UNITS = 6, P_MAXST = 6;
 constexpr int P_A_PIECE = 128 * P_TK * 2;                    // 16 KiB: this CTA's A rows
-constexpr int P_B_PIECE = 128 * P_TK * 2;                    // 16 KiB: this CTA's B rows
-constexpr int P_UNIT = P_A_PIECE + P_B_PIECE;                // one piece of each operand
-constexpr int P_SMEM = 1024 + P_UNITS * P_UNIT + 256;
+// tile width 256 or 128: this CTA's B rows are half of it (16 or 8 KiB a piece)
+__host__ __device__ constexpr int p_b_piece(int pn) { return pn / 2 * P_TK * 2; }
+__host__ __device__ constexpr int p_unit(int pn) { return P_A_PIECE + p_b_piece(pn); }   // one piece of each operand
+__host__ __device__ constexpr int p_smem(int pn) { return 1024 + P_UNITS * p_unit(pn) + 256; }
 constexpr int P_NTHREADS = 320;                              // 8 epilogue warps + producer + MMA/relay
-static_assert(P_SMEM <= 227 * 1024, "shared memory of one CTA");
+static_assert(p_smem(256) <= 227 * 1024, "shared memory of one CTA");
 }  // namespace
 
 __device__ __forceinline__ uint32_t cluster_ctarank() {
@@ -395,11 +396,12 @@ __device__ __forceinline__ void umma_commit_pair(uint64_t* bar, uint16_t cta_mas
       : "memory");
 }
 
-template <bool TF32>
+template <bool TF32, int PN>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_NTHREADS, 1)
     tc_gemm_pair_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                         float* __restrict__ C, int M, int N, long long ldc, int kslabs, TcTerms terms,
                         int* g_err) {
+  constexpr int P_UNIT = p_unit(PN), P_B_PIECE = p_b_piece(PN), EC = PN / 2;
   extern __shared__ uint8_t smem_raw[];
   volatile int* gerr = g_err;
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -415,7 +417,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_NTHREADS, 1)
   const uint32_t rank = cluster_ctarank();
   const bool leader = rank == 0;
   const int mgroups = (M + 255) / 256;
-  const long long ngroups = (long long)mgroups * ((N + 255) / 256);
+  const long long ngroups = (long long)mgroups * ((N + PN - 1) / PN);
   const long long cid = blockIdx.x >> 1, ncl = gridDim.x >> 1;
   const long long tiles_here = ngroups > cid ? (ngroups - 1 - cid) / ncl + 1 : 0;
   auto grp = [&](long long i) { return cid + i * ncl; };
@@ -441,7 +443,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_NTHREADS, 1)
   if (warp == 9) {
     // one warp of each CTA of the pair allocates, collectively, the TMEM of both
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(su32(tmem_slot)),
-                 "r"(512)
+                 "r"(2 * PN)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
   }
@@ -468,7 +470,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_NTHREADS, 1)
         const long long gg = grp(g / kslabs);
         const int kb = (int)(g % kslabs);
         const int m0 = (int)(gg % mgroups) * 256 + (int)rank * 128;
-        const int nb0 = (int)(gg / mgroups) * 256 + (int)rank * 128;
+        const int nb0 = (int)(gg / mgroups) * PN + (int)rank * (PN / 2);
         const int k0 = kb * (TF32 ? P_TK / 2 : P_TK);   // elements of a 128-byte row
         uint8_t* st = smem + s * stage_bytes;
         mbar_expect_tx(full + s, (uint32_t)stage_bytes);
@@ -497,9 +499,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_NTHREADS, 1)
         mbar_arrive_rank(full + s, 0);
       }
     } else if (lane == 0) {
-      // ---------------- MMA issuer (CTA 0): M = 256, N = 256, K = 32 bytes of a row;
+      // ---------------- MMA issuer (CTA 0): M = 256, N = PN, K = 32 bytes of a row;
       // one chunk per slab, its small terms first
-      constexpr uint32_t idesc = TF32 ? idesc_tf32_f32(256, 256) : idesc_bf16_f32(256, 256);
+      constexpr uint32_t idesc = TF32 ? idesc_tf32_f32(256, PN) : idesc_bf16_f32(256, PN);
       bool ok = true;
       for (long long g = 0; g < total && ok; ++g) {
         const int b = (int)(g & 1);
@@ -511,7 +513,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_NTHREADS, 1)
           break;
         }
         tc_fence_after();
-        const uint32_t dst = tmem + (uint32_t)(b * 256);
+        const uint32_t dst = tmem + (uint32_t)(b * PN);
         const uint32_t st = su32(smem + s * stage_bytes);
         for (int t = 0; t < terms.nterms; ++t) {
           const int pa_t = (int)(terms.code >> (4 * t)) & 3, pb_t = (int)(terms.code >> (4 * t + 2)) & 3;
@@ -538,13 +540,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_NTHREADS, 1)
   } else {
     // ---------------- epilogue warps (both CTAs): this CTA's 128 rows of the tile
     const int quarter = warp & 3, part = warp >> 2;
-    const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(part * 128);
+    const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(part * EC);
     bool ok = true;
     long long g = 0;
     for (long long i = 0; i < my_tiles && ok; ++i) {
-      float acc[128];
+      float acc[EC];
 #pragma unroll
-      for (int j = 0; j < 128; ++j) acc[j] = 0.0f;
+      for (int j = 0; j < EC; ++j) acc[j] = 0.0f;
       for (int kb = 0; kb < kslabs; ++kb, ++g) {
         const int b = (int)(g & 1);
         if (!mbar_wait(tfull + b, (uint32_t)(g >> 1) & 1u, cta_abort, gerr)) {
@@ -553,10 +555,10 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_NTHREADS, 1)
         }
         tc_fence_after();
 #pragma unroll
-        for (int q = 0; q < 128; q += 64) {
+        for (int q = 0; q < EC; q += 64) {
           uint32_t v0[32], v1[32];
-          tmem_ld_async(lane_base + (uint32_t)(b * 256 + q), v0);
-          tmem_ld_async(lane_base + (uint32_t)(b * 256 + q + 32), v1);
+          tmem_ld_async(lane_base + (uint32_t)(b * PN + q), v0);
+          tmem_ld_async(lane_base + (uint32_t)(b * PN + q + 32), v1);
           tmem_wait_ld();
 #pragma unroll
           for (int j = 0; j < 32; ++j) acc[q + j] += __uint_as_float(v0[j]);
@@ -570,17 +572,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_NTHREADS, 1)
       if (!ok || *cta_abort) break;
       const long long gg = grp(i);
       const int row = (int)(gg % mgroups) * 256 + (int)rank * 128 + quarter * 32 + lane;
-      const int col0 = (int)(gg / mgroups) * 256 + part * 128;
+      const int col0 = (int)(gg / mgroups) * PN + part * EC;
       if (row < M) {
         float* dst = C + (long long)row * ldc + col0;
-        const bool vec = ((ldc & 3) == 0) && ((((uintptr_t)C) & 15) == 0) && (col0 + 128 <= N);
+        const bool vec = ((ldc & 3) == 0) && ((((uintptr_t)C) & 15) == 0) && (col0 + EC <= N);
         if (vec) {
 #pragma unroll
-          for (int j = 0; j < 128; j += 4)
+          for (int j = 0; j < EC; j += 4)
             *reinterpret_cast<float4*>(dst + j) = make_float4(acc[j], acc[j + 1], acc[j + 2], acc[j + 3]);
         } else {
 #pragma unroll
-          for (int j = 0; j < 128; ++j)
+          for (int j = 0; j < EC; ++j)
             if (col0 + j < N) dst[j] = acc[j];
         }
       }
@@ -591,7 +593,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(P_NTHREADS, 1)
   cluster_sync_all();   // no CTA leaves while its peer may still use its TMEM or barriers
   if (warp == 9) {
     tc_fence_after();
-    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512)
+    asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * PN)
                  : "memory");
   }
 }
@@ -658,10 +660,11 @@ static bool pair_smem_attr_set() {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return false;
   if (dev >= 0 && dev < kMaxDevices && done[dev].load(std::memory_order_acquire)) return true;
-  if (cudaFuncSetAttribute(tc_gemm_pair_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, P_SMEM) !=
-          cudaSuccess ||
-      cudaFuncSetAttribute(tc_gemm_pair_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, P_SMEM) !=
-          cudaSuccess)
+  const cudaFuncAttribute at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  if (cudaFuncSetAttribute(tc_gemm_pair_kernel<false, 256>, at, p_smem(256)) != cudaSuccess ||
+      cudaFuncSetAttribute(tc_gemm_pair_kernel<true, 256>, at, p_smem(256)) != cudaSuccess ||
+      cudaFuncSetAttribute(tc_gemm_pair_kernel<false, 128>, at, p_smem(128)) != cudaSuccess ||
+      cudaFuncSetAttribute(tc_gemm_pair_kernel<true, 128>, at, p_smem(128)) != cudaSuccess)
     return false;
   if (dev >= 0 && dev < kMaxDevices) done[dev].store(1, std::memory_order_release);
   return true;
@@ -688,9 +691,16 @@ int launch_tc_gemm(const void* A, int M, const void* B, int N, int Kpad, int npi
   }
   const bool use_pair = tf32 || (HOTRG_TC_USE_PAIR != 0 && Kpad % P_TK == 0);
   const int slab_k = tf32 ? P_TK / 2 : P_TK;   // elements of a 128-byte row
+  // Tile width of the pair form: 256, or 128 where that ends sooner.  A slab costs 24 MMAs of 128 clocks
+  // (three BF16 pieces) at 256 columns; at 128 it has half the MMAs and three quarters of the copied rows,
+  // counted here as 0.7.  The tiles run in rounds over the pairs of SMs: a product with fewer tiles than
+  // pairs takes the narrow one.  1001 x 1500 x 1333, BF16X6: 48 tiles instead of 24, the whole call 146 -> 129 us
+  const long long pairs = std::max(1, sm_count() / 2), mg = (M + 255) / 256;
+  const long long wide = (mg * ((N + 255) / 256) + pairs - 1) / pairs, narrow = (mg * ((N + 127) / 128) + pairs - 1) / pairs;
+  const int pn = narrow * 70 < wide * 100 ? 128 : 256;
   CUtensorMap ma, mb;
   if (use_pair) {
-    if (make_piece_map(&ma, A, M, Kpad, npieces, 128, slab_k, tf32) || make_piece_map(&mb, B, N, Kpad, npieces, 128, slab_k, tf32))
+    if (make_piece_map(&ma, A, M, Kpad, npieces, 128, slab_k, tf32) || make_piece_map(&mb, B, N, Kpad, npieces, pn / 2, slab_k, tf32))
       return -1;
   } else if (make_piece_map(&ma, A, M, Kpad, npieces, TM, TK) || make_piece_map(&mb, B, N, Kpad, npieces, TN, TK)) {
     return -1;
@@ -720,8 +730,8 @@ int launch_tc_gemm(const void* A, int M, const void* B, int N, int Kpad, int npi
     return -1;
   }
   const long long ntiles = (long long)((M + TM - 1) / TM) * ((N + TN - 1) / TN);
-  const long long ngroups = (long long)((M + 255) / 256) * ((N + 255) / 256);
-  const int grid = use_pair ? 2 * (int)std::min<long long>(ngroups, std::max(1, sm_count() / 2))
+  const long long ngroups = mg * ((N + pn - 1) / pn);
+  const int grid = use_pair ? 2 * (int)std::min<long long>(ngroups, pairs)
                             : (int)std::min<long long>(ntiles, sm_count());
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (ms_out) {
@@ -729,11 +739,11 @@ int launch_tc_gemm(const void* A, int M, const void* B, int N, int Kpad, int npi
     cudaEventCreate(&e1);
     cudaEventRecord(e0, s);
   }
-  if (use_pair && tf32)
-    tc_gemm_pair_kernel<true><<<grid, P_NTHREADS, P_SMEM, s>>>(ma, mb, C, M, N, ldc, Kpad / slab_k, terms, err_flag);
-  else if (use_pair)
-    tc_gemm_pair_kernel<false><<<grid, P_NTHREADS, P_SMEM, s>>>(ma, mb, C, M, N, ldc, Kpad / slab_k, terms, err_flag);
-  else
+  if (use_pair) {
+    auto kernel = pn == 128 ? (tf32 ? tc_gemm_pair_kernel<true, 128> : tc_gemm_pair_kernel<false, 128>)
+                            : (tf32 ? tc_gemm_pair_kernel<true, 256> : tc_gemm_pair_kernel<false, 256>);
+    kernel<<<grid, P_NTHREADS, p_smem(pn), s>>>(ma, mb, C, M, N, ldc, Kpad / slab_k, terms, err_flag);
+  } else
     tc_gemm_kernel<<<grid, NTHREADS, SMEM_BYTES, s>>>(ma, mb, C, M, N, ldc, Kpad / TK, terms, err_flag);
   ++g_launches;
   if (ms_out) {
