@@ -23,6 +23,7 @@
 #include <vector>
 
 #include "hotrg_internal.cuh"
+#include "partials.h"
 #include "../../include/hotrg.h"
 
 using namespace hotrg;
@@ -367,7 +368,7 @@ int launch_failed(hotrg_ctx* c, const char* what, long long a, long long b, long
 
 // C = A . B^T in FP64: on the tensor cores where the product is large enough and the workspace can be
 // had, else on the FP64 pipe.  nsplit > 1: split along K, at most nsplit_most partials.  Returns the
-// partials written, or a negative status.
+// partials written: none if a launch was refused (the context is then poisoned).
 int gemm64(hotrg_ctx* c, const double* A, long long lda, const double* B, long long ldb, double* C, long long ldc,
            long long split_stride, int M, int N, long long K, int nsplit, int upper_only, cudaStream_t s,
            int nsplit_most = 1) {
@@ -380,7 +381,7 @@ int gemm64(hotrg_ctx* c, const double* A, long long lda, const double* B, long l
       const int r = launch_gemm_nt_f64_tc(A, lda, B, ldb, C, ldc, split_stride, M, N, K, std::max(nsplit, nsplit_most),
                                           upper_only, c->Wd.p, c->Wd.bytes, &((DevState*)c->state.p)->status, s);
       if (r > 0) return r;
-      if (r < 0) return launch_failed(c, "FP64 product on the tensor cores", M, N, K);
+      if (r < 0) return partials_written(launch_failed(c, "FP64 product on the tensor cores", M, N, K));
     }
   }
   return launch_gemm_nt_f64(A, lda, B, ldb, C, ldc, split_stride, M, N, K, nsplit, upper_only, s);

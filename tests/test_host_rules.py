@@ -1,0 +1,33 @@
+"""Rules of the library that are plain host C++: compiled with the system compiler and run here."""
+
+import os
+import subprocess
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+CSRC = os.path.join(ROOT, "paper_2110_03607_gb300", "csrc")
+
+
+def _run(tmp_path, headers, body):
+    src = tmp_path / "rule.cpp"
+    inc = "".join('#include "%s"\n' % os.path.join(CSRC, h) for h in headers)
+    src.write_text("#include <cstdio>\n" + inc + "using namespace hotrg;\n"
+                   "#define CHECK(x) do { if (!(x)) { std::printf(\"line %d: %s\\n\", __LINE__, #x); return 1; } } while (0)\n"
+                   "int main() {\n" + body + "\nreturn 0;\n}\n")
+    exe = tmp_path / "rule"
+    subprocess.run(["g++", "-std=c++17", "-O1", "-o", str(exe), str(src)], check=True)
+    r = subprocess.run([str(exe)], capture_output=True, text=True)
+    assert r.returncode == 0, r.stdout
+
+
+def test_a_refused_product_moves_no_offset(tmp_path):
+    """Two parity blocks share a buffer of partials: the second one's place follows from what the first
+    wrote.  A refused first product (each status of the library) leaves the second at the start."""
+    _run(tmp_path, ["partials.h"], """
+      const long long mb = 128;
+      for (int status = -7; status <= 0; ++status) {
+        const int n = partials_written(status);
+        CHECK(n == 0);
+        CHECK((long long)n * mb * mb == 0);
+      }
+      CHECK(partials_written(1) == 1 && partials_written(256) == 256);
+    """)
