@@ -34,6 +34,7 @@
 
 #include <algorithm>
 
+#include "eig_class.h"
 #include "hotrg_internal.cuh"
 #include "../../include/hotrg.h"
 
@@ -97,7 +98,8 @@ struct EigWs {
   int* okc;          // [nmat][n] by label: the exchange holds in the component
   int* sym;          // [nmat][n] by index: it does in this one's
   int* cls;          // [nmat][n] by eigenvector: (label + 1) even, -(label + 1) odd, 0 without the exchange
-  int* icl;          // [nmat][n] the same by index of the turned basis
+  int* lost;         // [nmat][n] by eigenvector: bits of the passes that ended its class
+  int* icl;          // [nmat][n] the same as cls by index of the turned basis
   int* idx;          // [nmat][n] columns of the secular equation
   int* defl;         // [nmat][n] deflated columns
   int* rp;           // [nmat][n] rotation columns
@@ -1469,10 +1471,10 @@ __global__ void __launch_bounds__(256) jacobi_onesided_kernel(const double* __re
 // W = A V is formed and its columns are made orthogonal to 4 n eps (one-sided Jacobi's test): groups
 // of close eigenvalues by plane rotations, the others, whose angles are tiny, all at once.
 // ---------------------------------------------------------------------------
-// two vectors are turned against each other: an even and an odd one lose their classes
-__device__ __forceinline__ void unclass(int* cls, int p, int q) {
-  if (cls[p] == -cls[q]) cls[p] = cls[q] = 0;
-}
+// The classes stay as they were until the last pass; what ends them is collected in `lost`, a bit for
+// each pass: the polish (which reads its own, turn by turn), then each pass over the tiny angles, which
+// turns all columns at once from where the passes before left them, and so reads the bits of those alone.
+constexpr int kLostPolish = 1;
 
 // out = X Y / unscale, or with the angles as X, out = Y + X Y where the matrix has any; 32 x 32
 // tiles, 2 x 2 per thread
@@ -1520,7 +1522,7 @@ __global__ void __launch_bounds__(256) eig_nn_kernel(const double* __restrict__ 
     }
 }
 
-// squared norms of W's columns (into dk); LAST: the eigenvalues
+// squared norms of W's columns (into dk); LAST: the eigenvalues, and no class where a pass ended it
 template <bool LAST>
 __global__ void __launch_bounds__(256) eig_norm_kernel(const double* __restrict__ W, EigWs ws, double* lam) {
   const int mat = blockIdx.y, n = ws.na[mat], ld = ws.n;
@@ -1533,8 +1535,12 @@ __global__ void __launch_bounds__(256) eig_norm_kernel(const double* __restrict_
   for (int i = lane; i < n; i += 32) a = fma(w[i], w[i], a);
   a = warp_sum(a);
   if (lane == 0) {
-    if (LAST) lam[mat * ld + c] = sqrt(a) * ctl.unscale;
-    else ws.dk[mat * ld + c] = a;
+    if (LAST) {
+      lam[mat * ld + c] = sqrt(a) * ctl.unscale;
+      if (ws.lost[mat * ld + c]) ws.cls[mat * ld + c] = 0;
+    } else {
+      ws.dk[mat * ld + c] = a;
+    }
   }
 }
 
@@ -1542,7 +1548,8 @@ __global__ void __launch_bounds__(256) eig_norm_kernel(const double* __restrict_
 // orthogonal to 4 n eps the tangent t of its plane rotation, w_p -= t w_q, w_q += t w_p, in M.
 // Angles above 2^-24 are left (first order does not hold): between kept vectors, or across the cut,
 // the groups have taken them.
-__global__ void __launch_bounds__(256) eig_gram_kernel(const double* __restrict__ W, EigWs ws, double* __restrict__ M) {
+__global__ void __launch_bounds__(256) eig_gram_kernel(const double* __restrict__ W, EigWs ws, double* __restrict__ M,
+                                                       int pass_bit) {
   constexpr int BK = 16;
   __shared__ double As[BK][33], Bs[BK][33];
   const int mat = blockIdx.z, n = ws.na[mat], ld = ws.n, q0 = blockIdx.x * 32, p0 = blockIdx.y * 32;
@@ -1588,7 +1595,14 @@ __global__ void __launch_bounds__(256) eig_gram_kernel(const double* __restrict_
           if (fabs(t) > 5.9604644775390625e-8) t = 0.0;
           if (t != 0.0) {
             any = true;
-            unclass(ws.cls + mat * ld, p, q);
+            int* lost = ws.lost + mat * ld;
+            const int* cl = ws.cls + mat * ld;
+            const int before = pass_bit - 1;   // other CTAs set this pass's bit meanwhile: it is not read
+            const bool lp = (__ldcg(lost + p) & before) != 0, lq = (__ldcg(lost + q) & before) != 0;
+            if (turn_ends_class(cl[p], lp, cl[q], lq)) {
+              atomicOr(lost + p, pass_bit);
+              atomicOr(lost + q, pass_bit);
+            }
           }
         }
       }
@@ -1673,7 +1687,10 @@ __global__ void __launch_bounds__(256) eig_polish_kernel(EigWs ws, double* V, do
           }
           if (lane == 0) {
             s_rot = 1;
-            unclass(ws.cls + mat * ld, lo + p, lo + q);
+            // the pairs of a round are disjoint, and a barrier ends the round
+            int *lp = ws.lost + mat * ld + lo + p, *lq = ws.lost + mat * ld + lo + q;
+            const int* cl = ws.cls + mat * ld + lo;
+            if (turn_ends_class(cl[p], *lp != 0, cl[q], *lq != 0)) *lp = *lq = kLostPolish;
           }
         }
         __syncthreads();
@@ -1721,7 +1738,7 @@ size_t eig_layout(char* base, int n, int nmat, EigWs* w, int** pos) {
   w->tf = dbl((size_t)((n + kRb - 1) / kRb) * kRb * kRb * nmat);
   for (double** p : {&w->d, &w->e, &w->tau, &w->ev0, &w->ev1, &w->dk, &w->zk, &w->zh, &w->val, &w->rc, &w->rs})
     *p = dbl(nv);
-  for (int** p : {&w->perm, &w->comp, &w->sgn, &w->okc, &w->sym, &w->icl, &w->idx, &w->defl, &w->rp, &w->rq, &w->top, &w->bot, pos}) *p = i32(nv);
+  for (int** p : {&w->perm, &w->comp, &w->sgn, &w->okc, &w->sym, &w->lost, &w->icl, &w->idx, &w->defl, &w->rp, &w->rq, &w->top, &w->bot, pos}) *p = i32(nv);
   w->ctl = (EigCtl*)(base + L.take(sizeof(EigCtl) * nmat));
   w->mc = (MergeCtl*)(base + L.take(sizeof(MergeCtl) * nmat * eig_leaves(n)));
   return L.bytes;
@@ -1813,7 +1830,9 @@ int launch_eig(const double* A, int n, int nmat, const int* na, const int* keep,
     return e == cudaSuccess ? 0 : -1;
   }
   w.swp = swp;
-  if (cudaMemsetAsync(w.ctl, 0, sizeof(EigCtl) * nmat, s) != cudaSuccess) return -1;
+  if (cudaMemsetAsync(w.ctl, 0, sizeof(EigCtl) * nmat, s) != cudaSuccess ||
+      cudaMemsetAsync(w.lost, 0, sizeof(int) * n * nmat, s) != cudaSuccess)
+    return -1;
   const dim3 rows((n + 7) / 8, nmat);
   double* m = w.q0;   // A scaled: the vectors' buffer is not needed yet
   eig_check_kernel<<<rows, 256, 0, s>>>(A, w);
@@ -1870,7 +1889,7 @@ int launch_eig(const double* A, int n, int nmat, const int* na, const int* keep,
   eig_polish_kernel<<<nmat, 256, 0, s>>>(w, V, W, lam);
   for (int it = 0; it < 2; ++it) {
     eig_norm_kernel<false><<<rows, 256, 0, s>>>(W, w, lam);
-    eig_gram_kernel<<<tiles, 256, 0, s>>>(W, w, M);
+    eig_gram_kernel<<<tiles, 256, 0, s>>>(W, w, M, kLostPolish << (it + 1));
     eig_nn_kernel<true><<<tiles, 256, 0, s>>>(M, V, w, Vn);
     eig_nn_kernel<true><<<tiles, 256, 0, s>>>(M, W, w, Wn);
     eig_take_kernel<<<rows, 256, 0, s>>>(w, Vn, Wn, V, W);

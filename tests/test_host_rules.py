@@ -31,3 +31,24 @@ def test_a_refused_product_moves_no_offset(tmp_path):
       }
       CHECK(partials_written(1) == 1 && partials_written(256) == 256);
     """)
+
+
+def test_a_class_is_lost_with_every_turn_that_mixes_it(tmp_path):
+    """An even vector p turned against two odd ones q, r, in any order and with q against r: all three
+    are mixtures afterwards.  Vectors of one class keep it, those of two components do not."""
+    _run(tmp_path, ["eig_class.h"], """
+      const int cls[3] = {+5, -5, -5};
+      const int pairs[3][2] = {{0, 1}, {0, 2}, {1, 2}};
+      const int order[4][3] = {{0, 1, -1}, {1, 0, -1}, {0, 2, -1}, {2, 1, 0}};
+      for (auto& o : order) {
+        bool lost[3] = {false, false, false};
+        for (int step = 0; step < 3 && o[step] >= 0; ++step) {
+          const int p = pairs[o[step]][0], q = pairs[o[step]][1];
+          if (turn_ends_class(cls[p], lost[p], cls[q], lost[q])) lost[p] = lost[q] = true;
+          CHECK(turn_ends_class(cls[p], lost[p], cls[q], lost[q]) == turn_ends_class(cls[q], lost[q], cls[p], lost[p]));
+        }
+        CHECK(lost[0] && lost[1] && lost[2]);
+      }
+      CHECK(!turn_ends_class(5, false, 5, false) && !turn_ends_class(0, false, 0, false));
+      CHECK(turn_ends_class(5, false, 7, false) && turn_ends_class(5, false, -7, false) && turn_ends_class(5, false, 0, false));
+    """)
