@@ -99,6 +99,14 @@ inline int split_terms(int npieces, int* ta, int* tb) {
 }
 
 #ifdef __CUDACC__
+// The limit of a kernel's dynamic shared memory belongs to the function, and so to every host thread that
+// launches it: each call sets it to the same `most`, the largest any size needs, never to its own size,
+// which another thread could lower before the launch.
+template <typename K>
+inline bool raise_smem_limit(K kernel, int most) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, most) == cudaSuccess;
+}
+
 // sum of n split-K partials in eight chains: the loads overlap, and the rounding error grows with the
 // square root of n / 8, not of n
 template <typename F>

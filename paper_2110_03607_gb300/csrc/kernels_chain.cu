@@ -272,9 +272,7 @@ template <typename TIn, typename TAcc, int NN, int OUT, bool ZIN = false, bool Z
 static void launch_one(const ChainDesc& d, const TIn* in, const TAcc* U, void* out, cudaStream_t s,
                        const Z2In& zi = Z2In{}, const Z2Out& zo = Z2Out{}) {
   size_t smem = (size_t)d.chi * d.chi * URow<TAcc, NN>::ld * sizeof(TAcc);
-  if (smem > 48 * 1024)
-    cudaFuncSetAttribute(chain_kernel<TIn, TAcc, NN, OUT, ZIN, ZW>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)smem);
+  if (smem > 48 * 1024) raise_smem_limit(chain_kernel<TIn, TAcc, NN, OUT, ZIN, ZW>, 227 * 1024);
   long long blocks = (d.total + 255) / 256;
   const long long cap = (long long)(d.ctas_per_sm > 0 ? d.ctas_per_sm : 16) * sm_count();
   if (blocks > cap) blocks = cap;

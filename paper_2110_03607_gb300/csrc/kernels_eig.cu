@@ -2052,8 +2052,7 @@ void launch_select(const double* lam, const double* V, int n, int nnew, double* 
                    LegResult* res, const int* sweeps, int* scratch, cudaStream_t s, const int* cls, int* rank_out,
                    int* cls_out) {
   const size_t smem = (size_t)4 * n * sizeof(double) + (size_t)6 * n * sizeof(int);
-  if (smem > 48 * 1024)
-    cudaFuncSetAttribute(select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (smem > 47 * 1024) raise_smem_limit(select_kernel, 56 * kEigMaxN);
   int *piv = scratch, *sgn = scratch + 2 * n, *order = scratch + 4 * n;
   select_pivot_kernel<<<(2 * n + 7) / 8, 256, 0, s>>>(V, n, piv, sgn);
   select_kernel<<<1, 1024, smem, s>>>(lam, piv, n, nnew, lam_sorted, order, res, sweeps, cls, rank_out, cls_out);

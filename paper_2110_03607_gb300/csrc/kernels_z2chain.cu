@@ -395,6 +395,8 @@ __global__ void __launch_bounds__(256, NH <= 8 ? 3 : (NH <= 16 ? 2 : 1)) z2_nonp
 
 namespace {
 
+constexpr int kChainDynSmem = 224 * 1024;   // the kernels' lists take 2 KB of an SM's 227
+
 int half_width(const Z2Chain& p) {   // columns of the larger parity class
   const int n1 = __builtin_popcount(p.mask_n);
   return n1 > p.nn - n1 ? n1 : p.nn - n1;
@@ -403,9 +405,7 @@ int half_width(const Z2Chain& p) {   // columns of the larger parity class
 // the kernel's shared-memory limit, raised where U~ needs more than the default; false: it does not fit
 template <typename K>
 bool room(K kernel, size_t smem) {
-  if (smem > 226 * 1024) return false;
-  return smem <= 40 * 1024 ||
-         cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) == cudaSuccess;
+  return smem <= kChainDynSmem && (smem <= 40 * 1024 || raise_smem_limit(kernel, kChainDynSmem));
 }
 
 template <int PF, int NP, int NH>
