@@ -98,7 +98,7 @@ struct EigWs {
   int* okc;          // [nmat][n] by label: the exchange holds in the component
   int* sym;          // [nmat][n] by index: it does in this one's
   int* cls;          // [nmat][n] by eigenvector: (label + 1) even, -(label + 1) odd, 0 without the exchange
-  int* lost;         // [nmat][n] by eigenvector: bits of the passes that ended its class
+  int* lost;         // [nmat][n] by eigenvector: 1 where a turn ended its class
   int* icl;          // [nmat][n] the same as cls by index of the turned basis
   int* idx;          // [nmat][n] columns of the secular equation
   int* defl;         // [nmat][n] deflated columns
@@ -1471,10 +1471,8 @@ __global__ void __launch_bounds__(256) jacobi_onesided_kernel(const double* __re
 // W = A V is formed and its columns are made orthogonal to 4 n eps (one-sided Jacobi's test): groups
 // of close eigenvalues by plane rotations, the others, whose angles are tiny, all at once.
 // ---------------------------------------------------------------------------
-// The classes stay as they were until the last pass; what ends them is collected in `lost`, a bit for
-// each pass: the polish (which reads its own, turn by turn), then each pass over the tiny angles, which
-// turns all columns at once from where the passes before left them, and so reads the bits of those alone.
-constexpr int kLostPolish = 1;
+// Vectors of opposite classes are left as they are (turn_forbidden); what else ends a class is noted in
+// `lost` by the polish alone, whose turns are ordered by barriers, and applied by the last pass.
 
 // out = X Y / unscale, or with the angles as X, out = Y + X Y where the matrix has any; 32 x 32
 // tiles, 2 x 2 per thread
@@ -1522,7 +1520,7 @@ __global__ void __launch_bounds__(256) eig_nn_kernel(const double* __restrict__ 
     }
 }
 
-// squared norms of W's columns (into dk); LAST: the eigenvalues, and no class where a pass ended it
+// squared norms of W's columns (into dk); LAST: the eigenvalues, and no class where the polish ended it
 template <bool LAST>
 __global__ void __launch_bounds__(256) eig_norm_kernel(const double* __restrict__ W, EigWs ws, double* lam) {
   const int mat = blockIdx.y, n = ws.na[mat], ld = ws.n;
@@ -1548,8 +1546,7 @@ __global__ void __launch_bounds__(256) eig_norm_kernel(const double* __restrict_
 // orthogonal to 4 n eps the tangent t of its plane rotation, w_p -= t w_q, w_q += t w_p, in M.
 // Angles above 2^-24 are left (first order does not hold): between kept vectors, or across the cut,
 // the groups have taken them.
-__global__ void __launch_bounds__(256) eig_gram_kernel(const double* __restrict__ W, EigWs ws, double* __restrict__ M,
-                                                       int pass_bit) {
+__global__ void __launch_bounds__(256) eig_gram_kernel(const double* __restrict__ W, EigWs ws, double* __restrict__ M) {
   constexpr int BK = 16;
   __shared__ double As[BK][33], Bs[BK][33];
   const int mat = blockIdx.z, n = ws.na[mat], ld = ws.n, q0 = blockIdx.x * 32, p0 = blockIdx.y * 32;
@@ -1578,6 +1575,7 @@ __global__ void __launch_bounds__(256) eig_gram_kernel(const double* __restrict_
   const double* nrm = ws.dk + mat * ld;
   const double tol = 4.0 * n * kEps;
   const int first = n - ws.keep[mat];   // pairs of two vectors behind the kept ones stay
+  const int *cls = ws.cls + mat * ld, *lost = ws.lost + mat * ld;
   bool any = false;
 #pragma unroll
   for (int u = 0; u < 2; ++u)
@@ -1589,20 +1587,13 @@ __global__ void __launch_bounds__(256) eig_gram_kernel(const double* __restrict_
       if (p < q) {
         const double a = nrm[p], b = nrm[q], g = acc[u][v], big = fmax(a, b);
         // squares below 1e-30 lie under any floor: the scaled matrix has lambda_1 of order 1
-        if (q >= first && big > 1e-30 && fabs(g) > tol * big) {
+        if (q >= first && big > 1e-30 && fabs(g) > tol * big &&
+            !turn_forbidden(cls[p], lost[p] != 0, cls[q], lost[q] != 0)) {
           const double zeta = (b - a) / (2.0 * g);
           t = copysign(1.0, zeta) / (fabs(zeta) + sqrt(fma(zeta, zeta, 1.0)));
           if (fabs(t) > 5.9604644775390625e-8) t = 0.0;
           if (t != 0.0) {
             any = true;
-            int* lost = ws.lost + mat * ld;
-            const int* cl = ws.cls + mat * ld;
-            const int before = pass_bit - 1;   // other CTAs set this pass's bit meanwhile: it is not read
-            const bool lp = (__ldcg(lost + p) & before) != 0, lq = (__ldcg(lost + q) & before) != 0;
-            if (turn_ends_class(cl[p], lp, cl[q], lq)) {
-              atomicOr(lost + p, pass_bit);
-              atomicOr(lost + q, pass_bit);
-            }
           }
         }
       }
@@ -1654,6 +1645,8 @@ __global__ void __launch_bounds__(256) eig_polish_kernel(EigWs ws, double* V, do
       continue;
     }
     const int mp = m + (m & 1);
+    const int* cls = ws.cls + mat * ld + lo;
+    volatile int* lost = ws.lost + mat * ld + lo;
     for (int sweep = 0; sweep < 30; ++sweep) {
       __syncthreads();
       if (threadIdx.x == 0) s_rot = 0;
@@ -1662,6 +1655,10 @@ __global__ void __launch_bounds__(256) eig_polish_kernel(EigWs ws, double* V, do
         for (int k = warp; k < mp / 2; k += nw) {
           const int p = rr_slot(k, r, mp), q = rr_slot(mp - 1 - k, r, mp);
           if (p >= m || q >= m) continue;
+          // the pairs of a round are disjoint, and a barrier ends the round
+          const int cp = cls[p], cq = cls[q];
+          const bool lp = lost[p] != 0, lq = lost[q] != 0;
+          if (turn_forbidden(cp, lp, cq, lq)) continue;
           double *wp = Wm + (long long)(lo + p) * ld, *wq = Wm + (long long)(lo + q) * ld;
           double a = 0.0, b = 0.0, g = 0.0;
           for (int i = lane; i < n; i += 32) {
@@ -1687,11 +1684,9 @@ __global__ void __launch_bounds__(256) eig_polish_kernel(EigWs ws, double* V, do
           }
           if (lane == 0) {
             s_rot = 1;
-            // the pairs of a round are disjoint, and a barrier ends the round
-            int *lp = ws.lost + mat * ld + lo + p, *lq = ws.lost + mat * ld + lo + q;
-            const int* cl = ws.cls + mat * ld + lo;
-            if (turn_ends_class(cl[p], *lp != 0, cl[q], *lq != 0)) *lp = *lq = kLostPolish;
+            if (turn_ends_class(cp, lp, cq, lq, t)) lost[p] = lost[q] = 1;
           }
+          __syncwarp();
         }
         __syncthreads();
       }
@@ -1889,7 +1884,7 @@ int launch_eig(const double* A, int n, int nmat, const int* na, const int* keep,
   eig_polish_kernel<<<nmat, 256, 0, s>>>(w, V, W, lam);
   for (int it = 0; it < 2; ++it) {
     eig_norm_kernel<false><<<rows, 256, 0, s>>>(W, w, lam);
-    eig_gram_kernel<<<tiles, 256, 0, s>>>(W, w, M, kLostPolish << (it + 1));
+    eig_gram_kernel<<<tiles, 256, 0, s>>>(W, w, M);
     eig_nn_kernel<true><<<tiles, 256, 0, s>>>(M, V, w, Vn);
     eig_nn_kernel<true><<<tiles, 256, 0, s>>>(M, W, w, Wn);
     eig_take_kernel<<<rows, 256, 0, s>>>(w, Vn, Wn, V, W);

@@ -33,22 +33,30 @@ def test_a_refused_product_moves_no_offset(tmp_path):
     """)
 
 
-def test_a_class_is_lost_with_every_turn_that_mixes_it(tmp_path):
-    """An even vector p turned against two odd ones q, r, in any order and with q against r: all three
-    are mixtures afterwards.  Vectors of one class keep it, those of two components do not."""
+def test_classes_of_turned_vectors(tmp_path):
+    """Even and odd vectors of a component are not turned against each other.  A vector without a class (0,
+    or of another component) turned against an even one, that against an odd one, in any order that the
+    rules allow: whatever took part in a mixture has no class left, and none is handed on by tiny angles."""
     _run(tmp_path, ["eig_class.h"], """
-      const int cls[3] = {+5, -5, -5};
-      const int pairs[3][2] = {{0, 1}, {0, 2}, {1, 2}};
-      const int order[4][3] = {{0, 1, -1}, {1, 0, -1}, {0, 2, -1}, {2, 1, 0}};
-      for (auto& o : order) {
-        bool lost[3] = {false, false, false};
-        for (int step = 0; step < 3 && o[step] >= 0; ++step) {
-          const int p = pairs[o[step]][0], q = pairs[o[step]][1];
-          if (turn_ends_class(cls[p], lost[p], cls[q], lost[q])) lost[p] = lost[q] = true;
-          CHECK(turn_ends_class(cls[p], lost[p], cls[q], lost[q]) == turn_ends_class(cls[q], lost[q], cls[p], lost[p]));
+      CHECK(turn_forbidden(5, false, -5, false) && !turn_forbidden(0, false, 0, false));
+      CHECK(!turn_forbidden(5, true, -5, false) && !turn_forbidden(5, false, -5, true));
+      CHECK(!turn_forbidden(5, false, 5, false) && !turn_forbidden(5, false, -7, false));
+      for (int other = -7; other <= 0; other += 7) {
+        const int cls[4] = {+5, -5, -5, other};
+        const int order[3][3][2] = {{{0, 3}, {0, 1}, {1, 2}}, {{3, 1}, {0, 1}, {0, 2}}, {{2, 3}, {0, 2}, {1, 0}}};
+        for (auto& o : order) {
+          bool lost[4] = {false, false, false, false}, mixed[4] = {false, false, false, false};
+          for (auto& pq : o) {
+            const int p = pq[0], q = pq[1];
+            if (turn_forbidden(cls[p], lost[p], cls[q], lost[q])) continue;
+            CHECK(!turn_ends_class(cls[p], lost[p], cls[q], lost[q], 1e-9));
+            if (cls[p] != cls[q] || mixed[p] || mixed[q]) mixed[p] = mixed[q] = true;
+            const bool ends = turn_ends_class(cls[p], lost[p], cls[q], lost[q], 0.7);
+            CHECK(ends == turn_ends_class(cls[q], lost[q], cls[p], lost[p], -0.7));
+            if (ends) lost[p] = lost[q] = true;
+          }
+          for (int i = 0; i < 4; ++i) CHECK(lost[i] == mixed[i]);
         }
-        CHECK(lost[0] && lost[1] && lost[2]);
       }
-      CHECK(!turn_ends_class(5, false, 5, false) && !turn_ends_class(0, false, 0, false));
-      CHECK(turn_ends_class(5, false, 7, false) && turn_ends_class(5, false, -7, false) && turn_ends_class(5, false, 0, false));
+      CHECK(!turn_ends_class(5, false, 5, false, 1.0) && !turn_ends_class(0, false, 0, false, 1.0));
     """)
