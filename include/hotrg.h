@@ -119,10 +119,11 @@ int hotrg_set_precision(hotrg_ctx* ctx, int mode);
 int hotrg_set_fp64_threshold(hotrg_ctx* ctx, double flops);
 
 /* Cap, in bytes, on the device memory of the per-slice contraction operands
- * (bottleneck operand pieces, its FP32 product, chain intermediates).  Each
- * c'-slice of the new-tensor contraction (Sec. 4.2.9) is further cut into
- * sub-ranges of n'_1 so that one sub-range fits the smaller of this cap and
- * 60 % of the free device memory.  Default 160e9. */
+ * (bottleneck operand pieces, in the FP64 form their digits, its product, chain
+ * intermediates).  Small c'-slices of the new-tensor contraction (Sec. 4.2.9)
+ * share a pass, and large ones are cut into sub-ranges of n'_1, so that a pass
+ * fits the smaller of this cap and 60 % of the free device memory (one n'_1
+ * value of one slice at the least).  Default 160e9. */
 int hotrg_set_slice_budget(hotrg_ctx* ctx, double bytes);
 
 /* Z2 (spin-flip) block form of the new-tensor contraction; enable = 1 is the

@@ -374,9 +374,11 @@ int gemm64(hotrg_ctx* c, const double* A, long long lda, const double* B, long l
            int nsplit_most = 1) {
   const size_t want = f64_tc_bytes(M, N, K, A == B && lda == ldb && M == N, upper_only);
   if (want > 0) {
-    // sizes in powers of two: a run's bond dimensions grow, its workspace seldom
-    size_t size = (size_t)4 << 20;
-    while (size < want) size <<= 1;
+    // in eighths of a power of two: a run's bond dimensions grow, its workspace seldom, and an eighth is
+    // the most that it takes beyond its need
+    size_t step = (size_t)4 << 20;
+    while (step * 16 <= want) step <<= 1;
+    const size_t size = (want + step - 1) / step * step;
     if (c->Wd.bytes >= want || dev_alloc(c, c->Wd, size) == HOTRG_OK) {
       const int r = launch_gemm_nt_f64_tc(A, lda, B, ldb, C, ldc, split_stride, M, N, K, std::max(nsplit, nsplit_most),
                                           upper_only, c->Wd.p, c->Wd.bytes, &((DevState*)c->state.p)->status, s);
@@ -1487,6 +1489,7 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
   const int nnew1 = nnew[1];
   int n1_chunk = nnew1;
   double per_unit = 1.0;   // operand bytes of one n'_1 value of a slice
+  double budget = 0.0, digits_unit = 0.0;
   {
     // the Z2 blocks of B and C hold about half of B and C again; the derivative
     // adds two more of B and C (and FP64 staging of dB in the split form) and three
@@ -1497,18 +1500,21 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
         (tan2 ? 7.0 : (tangent ? 5.0 : 2.0)) * (double)elt * (double)chain_max / nnew1;
     size_t free_b = 0, total_b = 0;
     cudaMemGetInfo(&free_b, &total_b);
-    double budget = std::min(0.6 * (double)free_b + (double)(c->Bp.bytes + c->Cb.bytes + c->chA.bytes +
-                                                             c->chB.bytes + c->Zb.bytes + c->Zc.bytes),
-                             c->slice_budget_bytes);
-    n1_chunk = (int)std::max(1.0, std::min((double)nnew1, std::floor(budget / per_unit)));
+    budget = std::min(0.6 * (double)free_b + (double)(c->Bp.bytes + c->Cb.bytes + c->chA.bytes + c->chB.bytes +
+                                                      c->Zb.bytes + c->Zc.bytes + c->Wd.bytes),
+                      c->slice_budget_bytes);
+    // the digits of B in an FP64 product on the tensor cores (their workspace grows in steps of an eighth)
+    if (fp64) digits_unit = 1.125 * f64_tc_column_bytes(R, R) * (double)(Ns / nnew1);
+    n1_chunk = (int)std::max(1.0, std::min((double)nnew1, std::floor(budget / (per_unit + digits_unit))));
   }
   // Small slices share a pass: c' becomes one more index of the columns (c', n', n~), so that a step
   // is a few launches with enough work for every SM instead of chi_c times as many small ones (2D
   // chi = 24: one slice's non-prime stage has 576 threads).  As many as keep a pass's operands under
-  // 256 MB (a slice of that size fills the chip by itself), each output below 2^31 elements.
+  // 256 MB (a slice of that size fills the chip by itself) and within the budget, each output below 2^31
+  // elements.
   int sl_chunk = 1;
   if (n1_chunk == nnew1) {
-    const double most = 268435456.0 / (per_unit * nnew1);
+    const double most = std::min(268435456.0 / (per_unit * nnew1), budget / ((per_unit + digits_unit) * nnew1));
     const double elems = 2147483648.0 / (double)std::max(Ns * R, chain_max);
     sl_chunk = (int)std::max(1.0, std::min({(double)(sl_hi - sl_lo), most, elems}));
   }

@@ -504,6 +504,11 @@ size_t f64_tc_bytes(long long M, long long N, long long K, bool same, int upper)
   return std::min(ws_of(M, same ? 0 : N, K), (size_t)kWsCap);
 }
 
+double f64_tc_column_bytes(long long M, long long K) {
+  (void)M;
+  return 16.0 * padded(K) + 4.0;
+}
+
 // Partial products written (at most max_split); 0: not done (the caller takes the FP64 pipe),
 // negative: an error
 int launch_gemm_nt_f64_tc(const double* A, long long lda, const double* B, long long ldb, double* C, long long ldc,
