@@ -64,8 +64,11 @@ enum hotrg_status {
  * products, FP32 accumulation.  BF16X6: 3 pieces, 6 products.  TF32: one TF32
  * piece (10 stored mantissa bits, rounded to nearest), one product.  TF32X3: 2
  * TF32 pieces, 3 products.  The tensor cores take TF32 at half the BF16 rate,
- * so TF32X3 issues as much tensor time as BF16X6.  FP64: plain FP64
- * everywhere. */
+ * so TF32X3 issues as much tensor time as BF16X6.  FP64: FP64
+ * operands, sums and results everywhere.  Large FP64 products (the Grams of every mode
+ * too) run on the tensor cores as exact products of BF16 digits where that gives an
+ * entry at least as well as an FP64 sum of its terms does, and on the FP64 pipe where
+ * it does not (rows whose large elements do not meet, infinities, NaN). */
 enum hotrg_precision {
   HOTRG_PREC_FP64 = 0,
   HOTRG_PREC_BF16X3 = 1,
@@ -376,8 +379,8 @@ int hotrg_tensor(hotrg_ctx* ctx, double* T, int64_t cap, int dims[8]);
 /* The bottleneck contraction of Eq. (BottleneckPart) on its own:
  * C[M][N] = sum_k A[M][K] B[N][K] (both operands K-contiguous, row-major,
  * FP64 in and out) computed with the kernels of precision `mode` (split-BF16
- * or split-TF32 pieces on the tensor cores with FP32 accumulation, or FP64
- * DFMA tiles).
+ * or split-TF32 pieces on the tensor cores with FP32 accumulation, or FP64: see
+ * HOTRG_PREC_FP64; infinities and NaN come out as of an FP64 sum).
  * A, B, C may be host or device pointers.  Synchronous; allocates and frees
  * its own device scratch.  1 <= M, N, K <= 2^20 and M*K, N*K, M*N <= 2^31.
  * Errors: EINVAL, ENOMEM, ECUDA, ETIMEOUT. */
@@ -398,7 +401,8 @@ int hotrg_gemm_nt(int mode, int M, int N, int K, const double* A, const double* 
  * np = 2 (BF16X3) or 3 (BF16X6), Kp = K rounded up to a multiple of 64 and
  * r(x) = x rounded up to a multiple of 256; sizes whose scratch exceeds the
  * array are rejected with HOTRG_EINVAL (the FP64 mode works within the array: it holds the
- * digits of the operands, of B in passes where they do not fit).
+ * digits of the operands, of B in passes where they do not fit, and large products whose A
+ * does not fit run on the FP64 pipe).
  * mode is HOTRG_PREC_FP64, HOTRG_PREC_BF16X3 or HOTRG_PREC_BF16X6 (the TF32
  * modes give HOTRG_EINVAL here).  The
  * size limits of hotrg_gemm_nt apply in every mode.  The first call on a device looks up the

@@ -372,7 +372,8 @@ int launch_failed(hotrg_ctx* c, const char* what, long long a, long long b, long
 int gemm64(hotrg_ctx* c, const double* A, long long lda, const double* B, long long ldb, double* C, long long ldc,
            long long split_stride, int M, int N, long long K, int nsplit, int upper_only, cudaStream_t s,
            int nsplit_most = 1) {
-  const size_t want = f64_tc_bytes(M, N, K, A == B && lda == ldb && M == N, upper_only);
+  const int most = std::max(nsplit, nsplit_most);
+  const size_t want = f64_tc_bytes(M, N, K, A == B && lda == ldb && M == N, upper_only, most);
   if (want > 0) {
     // in eighths of a power of two: a run's bond dimensions grow, its workspace seldom, and an eighth is
     // the most that it takes beyond its need
@@ -380,8 +381,7 @@ int gemm64(hotrg_ctx* c, const double* A, long long lda, const double* B, long l
     while (step * 16 <= want) step <<= 1;
     const size_t size = (want + step - 1) / step * step;
     if (c->Wd.bytes >= want || dev_alloc(c, c->Wd, size) == HOTRG_OK) {
-      const int r = launch_gemm_nt_f64_tc(A, lda, B, ldb, C, ldc, split_stride, M, N, K, std::max(nsplit, nsplit_most),
-                                          upper_only, c->Wd.p, c->Wd.bytes, &((DevState*)c->state.p)->status, s);
+      const int r = launch_gemm_nt_f64_tc(A, lda, B, ldb, C, ldc, split_stride, M, N, K, most, upper_only, c->Wd.p, c->Wd.bytes, &((DevState*)c->state.p)->status, s);
       if (r > 0) return r;
       if (r < 0) return partials_written(launch_failed(c, "FP64 product on the tensor cores", M, N, K));
     }
@@ -2420,7 +2420,7 @@ int hotrg_gemm_nt(int mode, int M, int N, int K, const double* A, const double* 
     cudaMemcpy(dB, B, sizeof(double) * N * K, cudaMemcpyDefault);
     cudaMemset(err, 0, sizeof(int));
     if (mode == HOTRG_PREC_FP64) {
-      const size_t want = f64_tc_bytes(M, N, K, false, 0);
+      const size_t want = f64_tc_bytes(M, N, K, false, 0, 1);
       int r = 0;
       if (want > 0) {
         if (cudaMalloc(&pA, want) == cudaSuccess)

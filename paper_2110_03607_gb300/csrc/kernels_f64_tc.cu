@@ -2,23 +2,35 @@
 //
 // The FP64 pipe of this chip does 2 multiply-adds per clock and SM (1.25 TFLOP/s); its BF16 tensor
 // cores do 4096 times as many.  Following Ozaki, Ogita, Oishi and Rump (Numerical Algorithms 59, 2012),
-// every row of an operand is written as integers of a common unit 2^(e - 62), 2^e > max |x|, and each
-// integer as eight signed digits in base 256 (seven in [-128, 127], the leading one in [-65, 65]):
+// every row of an operand is written as integers of a common unit 2^(e - 62), 2^e > max |x|, rounded to
+// nearest, and each integer as eight signed digits in base 256 (seven in [-128, 127], the leading one in
+// [-65, 65]):
 //   x = sum_a v_a 2^(e - 6 - 8 a).
 // A digit is exact in BF16, a product of two is at most 2^14, and the tensor core adds into an FP32
 // accumulator without error while every partial sum stays within 2^24.  The products v_a w_b with
-// a + b = g <= 7 share one accumulator (they share the weight 2^-8g): at most 8 products times 128
-// along K, 2^14 2^3 2^7 = 2^24.  So each chunk of 128 along K gives eight exact integers P_g per
-// output; they are added, still exactly, into two 64-bit integers (hi: g = 0 .. 3, lo: g = 4 .. 7),
-// and one rounding to FP64 ends the sum.  Left out are the bits of an element below 2^-62 of its
-// row's largest and the products with a + b > 7, at most 2^-61 of the two rows' largest and of either
-// sign: less than the roundings of an FP64 sum.  Only where the two rows have the same digits, on the
-// diagonal of a Gram, do the squares among them add up (v_4^2 of every term: 2e-15 of the sum at
-// K = 32,768).  A symmetric product therefore takes a ninth accumulator, a + b = 8, in tiles of 48
-// columns; it enters lo rounded to its unit once a chunk.
+// a + b = g share one accumulator (they share the weight 2^-8g): at most 8 products times 128
+// along K, 2^14 2^3 2^7 = 2^24.  So each chunk of 128 along K gives nine exact integers P_0 .. P_8 per
+// output; they are added, P_8 rounded to P_7's unit, into two 64-bit integers (hi: g = 0 .. 3, lo: g = 4 .. 8),
+// and one rounding to FP64 ends the sum.
 //
-// Layout: tile 128 x 64 of C per CTA, its eight accumulators fill the 512 columns of TMEM.  A ring of
-// two stages holds K slabs of 32 (64-byte rows), all eight digits of both operands (96 KB a stage).
+// What this leaves out, with alpha = |a| / 2^ea and beta = |b| / 2^eb in [0, 1) and results in units of
+// 2^(ea + eb): of an element the bits below 2^-62, at most 2^-63 and of either sign, which is 2^-63.8
+// sqrt(|alpha|^2 + |beta|^2) in the mean (2-norms of the rows) and 2^-63 sum (alpha + beta) at the most; of the
+// digits' products those with a + b > 8, six of either sign at 2^-84 each: 2^-70 sqrt(K) in the mean, K 2^-67.4 at
+// the most.  (a + b = 8 is needed for rows with the same digits, the diagonal of a Gram or equal rows of two
+// operands: v_4^2 is positive, and 32,768 of them were 2e-15 of the sum of a row with one large element.)
+// An FP64 sum has errors of a few 2^-54 of s = sum alpha beta in the mean and K 2^-53 s at the most.  So the
+// digits are as good, entry by entry, where s >= 2^-9 (|alpha| + |beta|) (an error of 2^-54.8 s); where the
+// large elements of one row meet the small ones of the other, or a row holds an infinity or a NaN, they are not.
+// Therefore s is computed too, as one more product of BF16 (a ninth plane, alpha rounded down, and a tenth
+// accumulator, summed over all of K in FP32), and f64_fix_kernel forms the entries that fail the test on the
+// FP64 pipe.  Rows of coarse-grained tensors pass in general: no entry of the Grams and products of 3D steps
+// (bonds 9 x 11 x 10 and 12 to 16, zero field or 0.01 and 0.02) fails at 2^-9, 0.1 % of the worst product at 2^-8.
+// Near a trivial fixed point, where a few elements rule a tensor, or in a field of 1e-4, whose odd elements are
+// that small, a tenth to two thirds do: there the digits lost up to all of an entry's own figures.
+//
+// Layout: tile 128 x 48 of C per CTA, its ten accumulators fill 480 of the 512 columns of TMEM.  A ring of
+// two stages holds K slabs of 32 (64-byte rows), all nine planes of both operands (99 KB a stage).
 // The MMA warp goes through a slab by accumulator g, and waits for the epilogue once per g and chunk,
 // so the drain of one accumulator runs under the MMAs of the next.
 #include <stdio.h>
@@ -31,24 +43,26 @@
 namespace hotrg {
 
 namespace {
-constexpr int TM = 128, TK = 32, DIG = 8, STAGES = 2;
+constexpr int TM = 128, TN = 48, TK = 32, DIG = 8, STAGES = 2;
+constexpr int PLANES = DIG + 1;                 // the digits and alpha
+constexpr int ACCS = 9;                         // of the digits' products; the tenth sums alpha beta
 constexpr int CHUNK = 4;                        // slabs per exact sum: 128 along K
-constexpr int A_DIG = TM * TK * 2;
-// the tile width for a number of accumulators: 64 for 8, 48 for 9
-__host__ __device__ constexpr int tile_n(int accs) { return 512 / accs / 16 * 16; }
-__host__ __device__ constexpr int stage_bytes(int accs) { return DIG * (A_DIG + tile_n(accs) * TK * 2); }
-__host__ __device__ constexpr int smem_bytes(int accs) { return 1024 + STAGES * stage_bytes(accs) + 512; }
+constexpr int A_PLANE = TM * TK * 2, B_PLANE = TN * TK * 2;
+constexpr int STAGE_BYTES = PLANES * (A_PLANE + B_PLANE);
+constexpr int SMEM_BYTES = 1024 + STAGES * STAGE_BYTES + 512;
 constexpr int EPI_WARPS = 8, W_PROD = 8, W_MMA = 9, NTHREADS = 320;
 constexpr int NON_FINITE = 0x7fffffff;          // a row with an infinity or a NaN
-static_assert(smem_bytes(8) <= 227 * 1024, "shared memory of one CTA");
-static_assert(tile_n(8) == 64 && tile_n(9) == 48, "tile widths");
+static_assert(SMEM_BYTES <= 227 * 1024, "shared memory of one CTA");
+static_assert((ACCS + 1) * TN <= 512 && TN % 16 == 0, "columns of TMEM");
+constexpr float kTrust = 0.001953125f;          // 2^-9: the least s / (|alpha| + |beta|) of an entry taken from the digits
 
 struct SliceDesc {
   const double* x;
   long long ld;
   int rows;
-  __nv_bfloat16* v;    // digit a of element (r, k) at (a rows + r) kpad + k
-  int* e;              // per row: biased exponent of the largest |x|, at least 1
+  __nv_bfloat16* v;        // plane a of element (r, k) at (a rows + r) kpad + k
+  unsigned long long* q;   // per row: sum of alpha^2 in units of 2^-30
+  int* e;                  // per row: biased exponent of the largest |x|, at least 1
 };
 
 // largest |x| of a row, as the high word of its bits (0 below 2^-1042: the row's unit is then that
@@ -67,19 +81,32 @@ __device__ __forceinline__ unsigned long long digits(double x, int E) {
   if (be) m |= 0x10000000000000ULL;
   else be = 1;
   const int sh = be - E + 9;                    // x = m 2^(be - 1075), unit 2^(E - 1084); sh <= 9
-  unsigned long long f = sh >= 0 ? m << (sh & 15) : (sh > -64 ? m >> -sh : 0ULL);
+  unsigned long long f = sh >= 0 ? m << (sh & 15) : (sh > -64 ? (m + (1ULL << (-sh - 1))) >> -sh : 0ULL);
   if ((long long)bits < 0) f = 0ULL - f;
   return (f + 0x0080808080808080ULL) ^ 0x8000000000000000ULL;
 }
+// alpha = |x| 2^(1022 - E), as the bits of a BF16 number, rounded down; what is not zero is at least 2^-60, so
+// that a sum of products is zero only if every product is
+__device__ __forceinline__ unsigned alpha_bits(double x, int E) {
+  const unsigned hi = (unsigned)high_abs(x);
+  const int be = (int)(hi >> 20), ex = be - E - 1;
+  if (be == 0) return (hi | (unsigned)__double2loint(x)) != 0u ? 67u << 7 : 0u;
+  return ex < -60 ? 67u << 7 : (unsigned)(ex + 127) << 7 | ((hi >> 13) & 0x7fu);
+}
 
-// eight consecutive elements -> one 16-byte store per digit
-__device__ __forceinline__ void store_digits(const double (&x)[8], int E, __nv_bfloat16* dst, long long dstride) {
-  unsigned lo[8], hi[8];
+// eight consecutive elements -> one 16-byte store per plane; the sum of alpha^2 is returned
+__device__ __forceinline__ float store_planes(const double (&x)[8], int E, __nv_bfloat16* dst, long long dstride) {
+  unsigned lo[8], hi[8], al[4];
+  float sq = 0.0f;
 #pragma unroll
   for (int i = 0; i < 8; ++i) {
     const unsigned long long d = E == NON_FINITE ? 0x8080808080808080ULL : digits(x[i], E);
     lo[i] = (unsigned)d;
     hi[i] = (unsigned)(d >> 32);
+    const unsigned a = E == NON_FINITE ? 0u : alpha_bits(x[i], E);
+    al[i >> 1] = i & 1 ? al[i >> 1] | a << 16 : a;
+    const float f = __uint_as_float(a << 16);
+    sq = fmaf(f, f, sq);
   }
 #pragma unroll
   for (int a = 0; a < DIG; ++a) {
@@ -98,6 +125,12 @@ __device__ __forceinline__ void store_digits(const double (&x)[8], int E, __nv_b
     }
     *reinterpret_cast<uint4*>(dst + a * dstride) = make_uint4(w[0], w[1], w[2], w[3]);
   }
+  *reinterpret_cast<uint4*>(dst + DIG * dstride) = make_uint4(al[0], al[1], al[2], al[3]);
+  return sq;
+}
+// a sum of alpha^2 in units of 2^-30, rounded up: integers add up to the same in any order
+__device__ __forceinline__ unsigned long long norm_units(float sq) {
+  return (unsigned long long)ceilf(sq * 1073741824.0f);
 }
 
 __device__ __forceinline__ void load8(const double* x, int n, double (&v)[8]) {
@@ -115,7 +148,7 @@ __device__ __forceinline__ void load8(const double* x, int n, double (&v)[8]) {
 }
 
 // Short rows (K <= 2048): 2^tprl threads per row of either operand, eight elements each; exponent and
-// digits in one pass.
+// planes in one pass.
 __global__ void __launch_bounds__(256) slice_short_kernel(SliceDesc A, SliceDesc B, int K, int kpad, int tprl) {
   const int tpr = 1 << tprl;
   const long long r0 = (long long)blockIdx.x * (256 >> tprl) + (threadIdx.x >> tprl);
@@ -130,27 +163,39 @@ __global__ void __launch_bounds__(256) slice_short_kernel(SliceDesc A, SliceDesc
 #pragma unroll
   for (int i = 0; i < 8; ++i) hi = max(hi, high_abs(x[i]));
   __shared__ int wmax[8];
+  __shared__ unsigned long long wsum[8];
+  const int w = threadIdx.x >> 5, wpr = tpr >> 5;
   for (int o = min(tpr, 32) >> 1; o > 0; o >>= 1) hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
   if (tpr > 32) {
-    const int w = threadIdx.x >> 5, wpr = tpr >> 5;
     if ((threadIdx.x & 31) == 0) wmax[w] = hi;
     __syncthreads();
     for (int q = 0; q < wpr; ++q) hi = max(hi, wmax[(w & ~(wpr - 1)) + q]);
   }
   const int E = row_exponent(hi);
-  if (!live) return;
-  if (t == 0) d.e[r] = E;
-  if (k < kpad) store_digits(x, E, d.v + r * kpad + k, (long long)d.rows * kpad);
+  float sq = 0.0f;
+  if (live && k < kpad) sq = store_planes(x, E, d.v + r * kpad + k, (long long)d.rows * kpad);
+  unsigned long long n = norm_units(sq);
+  for (int o = min(tpr, 32) >> 1; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
+  if (tpr > 32) {
+    if ((threadIdx.x & 31) == 0) wsum[w] = n;
+    __syncthreads();
+    n = 0;
+    for (int q = 0; q < wpr; ++q) n += wsum[(w & ~(wpr - 1)) + q];
+  }
+  if (live && t == 0) {
+    d.e[r] = E;
+    d.q[r] = n;
+  }
 }
 
-// Long rows: the exponents first (blocks of a row meet in an atomic maximum; e zeroed before) ...
+// Long rows: the exponents first (blocks of a row meet in an atomic maximum; e and q zeroed before) ...
 __global__ void __launch_bounds__(256) slice_max_kernel(SliceDesc A, SliceDesc B, long long K) {
-  const bool second = (int)blockIdx.y >= A.rows;
+  const bool second = (int)blockIdx.x >= A.rows;
   const SliceDesc& d = second ? B : A;
-  const int r = second ? (int)blockIdx.y - A.rows : (int)blockIdx.y;
+  const int r = second ? (int)blockIdx.x - A.rows : (int)blockIdx.x;
   const double* x = d.x + r * d.ld;
   int hi = 0;
-  for (long long k = ((long long)blockIdx.x * 256 + threadIdx.x) * 8; k < K; k += (long long)gridDim.x * 2048) {
+  for (long long k = ((long long)blockIdx.y * 256 + threadIdx.x) * 8; k < K; k += (long long)gridDim.y * 2048) {
     double v[8];
     load8(x + k, (int)min(8LL, K - k), v);
 #pragma unroll
@@ -159,19 +204,22 @@ __global__ void __launch_bounds__(256) slice_max_kernel(SliceDesc A, SliceDesc B
   for (int o = 16; o > 0; o >>= 1) hi = max(hi, __shfl_xor_sync(0xffffffffu, hi, o));
   if ((threadIdx.x & 31) == 0) atomicMax(d.e + r, row_exponent(hi));
 }
-// ... then the digits
+// ... then the planes
 __global__ void __launch_bounds__(256) slice_long_kernel(SliceDesc A, SliceDesc B, long long K, int kpad) {
-  const bool second = (int)blockIdx.y >= A.rows;
+  const bool second = (int)blockIdx.x >= A.rows;
   const SliceDesc& d = second ? B : A;
-  const int r = second ? (int)blockIdx.y - A.rows : (int)blockIdx.y;
+  const int r = second ? (int)blockIdx.x - A.rows : (int)blockIdx.x;
   const double* x = d.x + r * d.ld;
   const int E = d.e[r];
   __nv_bfloat16* v0 = d.v + (long long)r * kpad;
-  for (long long k = ((long long)blockIdx.x * 256 + threadIdx.x) * 8; k < kpad; k += (long long)gridDim.x * 2048) {
+  unsigned long long n = 0;
+  for (long long k = ((long long)blockIdx.y * 256 + threadIdx.x) * 8; k < kpad; k += (long long)gridDim.y * 2048) {
     double v[8];
     load8(x + (k < K ? k : 0), (int)max(0LL, min(8LL, K - k)), v);
-    store_digits(v, E, v0 + k, (long long)d.rows * kpad);
+    n += norm_units(store_planes(v, E, v0 + k, (long long)d.rows * kpad));
   }
+  for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
+  if ((threadIdx.x & 31) == 0) atomicAdd(d.q + r, n);
 }
 
 // (hi 2^32 + lo) 2^e, rounded once to nearest-even (twice where the result is subnormal); in integer
@@ -221,7 +269,6 @@ struct TcItems {
 }  // namespace
 
 // item -> tile and K slabs; tiles run fastest, so the CTAs at work share their K range in L2
-template <int TN>
 __device__ __forceinline__ void item_of(const TcItems& it, long long i, int* m0, int* n0, int* z, int* s0, int* cnt) {
   int t = (int)(i % it.ntiles);
   *z = (int)(i / it.ntiles);
@@ -244,12 +291,10 @@ __device__ __forceinline__ void item_of(const TcItems& it, long long i, int* m0,
   *cnt = min(it.per, it.slabs - *s0);
 }
 
-template <int ACCS>
 __global__ void __launch_bounds__(NTHREADS, 1)
     f64_tc_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB,
                   const int* __restrict__ ea, const int* __restrict__ eb, double* __restrict__ C, long long ldc,
-                  long long split_stride, TcItems its, int* g_err) {
-  constexpr int TN = tile_n(ACCS), B_DIG = TN * TK * 2, STAGE_BYTES = stage_bytes(ACCS);
+                  long long split_stride, float* __restrict__ S, TcItems its, int* g_err) {
   extern __shared__ uint8_t smem_raw[];
   volatile int* gerr = g_err;
   uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -257,7 +302,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   uint64_t* empty = full + STAGES;
   uint64_t* tfull = empty + STAGES;      // [ACCS] MMA -> epilogue
   uint64_t* tempty = tfull + ACCS;       // [ACCS] epilogue -> MMA
-  uint64_t* drain = tempty + ACCS;
+  uint64_t* sfull = tempty + ACCS;       // the sum of alpha beta, once an item
+  uint64_t* sempty = sfull + 1;
+  uint64_t* drain = sempty + 1;
   uint32_t* tmem_slot = (uint32_t*)(drain + 1);
   volatile int* cta_abort = (volatile int*)(tmem_slot + 1);
 
@@ -271,6 +318,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       mbar_init(tfull + g, 1);
       mbar_init(tempty + g, EPI_WARPS);
     }
+    mbar_init(sfull, 1);
+    mbar_init(sempty, EPI_WARPS);
     mbar_init(drain, 1);
     *cta_abort = *gerr ? 1 : 0;   // an earlier launch or CTA gave up: do nothing
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -290,12 +339,12 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 
   if (warp == W_PROD) {
     if (lane == 0) {
-      // ---------------- TMA producer: both operands' digits of one K slab per stage
+      // ---------------- TMA producer: both operands' planes of one K slab per stage
       long long g = 0;
       bool ok = true;
       for (long long i = blockIdx.x; i < nitems && ok; i += gridDim.x) {
         int m0, n0, z, s0, cnt;
-        item_of<TN>(its, i, &m0, &n0, &z, &s0, &cnt);
+        item_of(its, i, &m0, &n0, &z, &s0, &cnt);
         for (int kb = 0; kb < cnt; ++kb, ++g) {
           const int s = (int)(g % STAGES);
           if (!mbar_wait(empty + s, (uint32_t)((g / STAGES) & 1) ^ 1u, cta_abort, gerr)) {
@@ -305,7 +354,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           uint8_t* st = smem + s * STAGE_BYTES;
           mbar_expect_tx(full + s, (uint32_t)STAGE_BYTES);
           tma_load_3d(&tmA, st, full + s, (s0 + kb) * TK, m0, 0);
-          tma_load_3d(&tmB, st + DIG * A_DIG, full + s, (s0 + kb) * TK, n0, 0);
+          tma_load_3d(&tmB, st + PLANES * A_PLANE, full + s, (s0 + kb) * TK, n0, 0);
         }
       }
       // no arrival may be in flight when the CTA exits: the last slabs are consumed, or, after an
@@ -326,10 +375,10 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       // ---------------- MMA issuer: accumulator g of a slab takes the products with a + b = g
       constexpr uint32_t idesc = idesc_bf16_f32(TM, TN);
       bool ok = true;
-      long long g = 0, ch = 0;   // slabs and chunks of this CTA so far
-      for (long long i = blockIdx.x; i < nitems && ok; i += gridDim.x) {
+      long long g = 0, ch = 0, item = 0;   // slabs, chunks and items of this CTA so far
+      for (long long i = blockIdx.x; i < nitems && ok; i += gridDim.x, ++item) {
         int m0, n0, z, s0, cnt;
-        item_of<TN>(its, i, &m0, &n0, &z, &s0, &cnt);
+        item_of(its, i, &m0, &n0, &z, &s0, &cnt);
         for (int kb = 0; kb < cnt && ok; ++kb, ++g) {
           const int s = (int)(g % STAGES);
           const bool first = kb % CHUNK == 0, last = kb % CHUNK == CHUNK - 1 || kb == cnt - 1;
@@ -338,7 +387,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             break;
           }
           const uint32_t st = su32(smem + s * STAGE_BYTES);
-          const uint64_t a0 = sdesc_sw<TK * 2>(st), b0 = sdesc_sw<TK * 2>(st + DIG * A_DIG);
+          const uint64_t a0 = sdesc_sw<TK * 2>(st), b0 = sdesc_sw<TK * 2>(st + PLANES * A_PLANE);
           for (int acc = 0; acc < ACCS; ++acc) {
             if (first && ch > 0 && !mbar_wait(tempty + acc, (uint32_t)(ch - 1) & 1u, cta_abort, gerr)) {
               ok = false;
@@ -348,7 +397,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             const uint32_t dst = tmem + (uint32_t)(acc * TN);
             const int a_lo = acc < DIG ? 0 : acc - DIG + 1;
             for (int a = a_lo; a < DIG && a <= acc; ++a) {
-              const uint64_t da = a0 + (uint64_t)(a * (A_DIG >> 4)), db = b0 + (uint64_t)((acc - a) * (B_DIG >> 4));
+              const uint64_t da = a0 + (uint64_t)(a * (A_PLANE >> 4)), db = b0 + (uint64_t)((acc - a) * (B_PLANE >> 4));
 #pragma unroll
               for (int kk = 0; kk < TK / 16; ++kk)   // 16 BF16 = 32 bytes inside the swizzled row
                 umma_bf16(dst, da + (uint64_t)(2 * kk), db + (uint64_t)(2 * kk), idesc,
@@ -357,6 +406,17 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             if (last) umma_commit(tfull + acc);
           }
           if (!ok) break;
+          // alpha beta, over all slabs of the item
+          if (kb == 0 && item > 0 && !mbar_wait(sempty, (uint32_t)(item - 1) & 1u, cta_abort, gerr)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+#pragma unroll
+          for (int kk = 0; kk < TK / 16; ++kk)
+            umma_bf16(tmem + (uint32_t)(ACCS * TN), a0 + (uint64_t)(DIG * (A_PLANE >> 4) + 2 * kk),
+                      b0 + (uint64_t)(DIG * (B_PLANE >> 4) + 2 * kk), idesc, kb == 0 && kk == 0 ? 0u : 1u);
+          if (kb == cnt - 1) umma_commit(sfull);
           umma_commit(empty + s);
           if (last) ++ch;
         }
@@ -375,11 +435,24 @@ __global__ void __launch_bounds__(NTHREADS, 1)
     constexpr int EC = TN / 2;
     const int quarter = warp & 3, part = warp >> 2;
     const uint32_t lane_base = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(part * EC);
+    auto load_acc = [&](int acc, uint32_t (&v)[EC]) {
+      uint32_t v0[16], v1[8];
+      tmem_ld_async(lane_base + (uint32_t)(acc * TN), v0);
+      tmem_ld_async(lane_base + (uint32_t)(acc * TN + 16), v1);
+      tmem_wait_ld();
+#pragma unroll
+      for (int j = 0; j < EC; ++j) v[j] = j < 16 ? v0[j & 15] : v1[j & 7];
+    };
+    auto release = [&](uint64_t* bar) {
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(bar)) : "memory");
+    };
     bool ok = true;
-    long long ch = 0;
-    for (long long i = blockIdx.x; i < nitems && ok; i += gridDim.x) {
+    long long ch = 0, item = 0;
+    for (long long i = blockIdx.x; i < nitems && ok; i += gridDim.x, ++item) {
       int m0, n0, z, s0, cnt;
-      item_of<TN>(its, i, &m0, &n0, &z, &s0, &cnt);
+      item_of(its, i, &m0, &n0, &z, &s0, &cnt);
       long long hi[EC], lo[EC];
 #pragma unroll
       for (int j = 0; j < EC; ++j) hi[j] = lo[j] = 0;
@@ -392,21 +465,8 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           if (!ok) continue;
           tc_fence_after();
           uint32_t v[EC];
-          if constexpr (EC == 32) {
-            tmem_ld_async(lane_base + (uint32_t)(acc * TN), v);
-            tmem_wait_ld();
-          } else {
-            uint32_t v0[16], v1[8];
-            tmem_ld_async(lane_base + (uint32_t)(acc * TN), v0);
-            tmem_ld_async(lane_base + (uint32_t)(acc * TN + 16), v1);
-            tmem_wait_ld();
-#pragma unroll
-            for (int j = 0; j < EC; ++j) v[j] = j < 16 ? v0[j & 15] : v1[j & 7];
-          }
-          tc_fence_before();
-          __syncwarp();
-          if (lane == 0)
-            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(su32(tempty + acc)) : "memory");
+          load_acc(acc, v);
+          release(tempty + acc);
 #pragma unroll
           for (int j = 0; j < EC; ++j) {
             const int p = __float2int_rn(__uint_as_float(v[j]));
@@ -416,19 +476,27 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           }
         }
       }
-      if (!ok || *cta_abort) break;
+      if (ok) ok = __all_sync(0xffffffffu, mbar_wait(sfull, (uint32_t)item & 1u, cta_abort, gerr)) != 0;
+      if (!ok) break;
+      tc_fence_after();
+      uint32_t sv[EC];
+      load_acc(ACCS, sv);
+      release(sempty);
+      if (*cta_abort) break;
       const int row = m0 + quarter * 32 + lane, col0 = n0 + part * EC;
       if (row < its.M) {
         const int er = ea[row];
         double* dst = C + (long long)z * split_stride + (long long)row * ldc + col0;
+        float* sdst = S + ((long long)z * its.M + row) * its.N + col0;
         // x = sum_a v_a 2^(E - 1022 - 6 - 8 a) of each operand; hi counts in units of 2^-24
         const int e0 = er - 2 * 1028 - 24 - 32;
 #pragma unroll
         for (int j = 0; j < EC; ++j)
           if (col0 + j < its.N) {
             const int ec = eb[col0 + j];
-            dst[j] = er == NON_FINITE || ec == NON_FINITE ? __longlong_as_double(0x7ff8000000000000LL)
-                                                          : fixed_to_double(hi[j], lo[j], e0 + ec);
+            // rows that are not finite are left to f64_fix_kernel
+            dst[j] = er == NON_FINITE || ec == NON_FINITE ? 0.0 : fixed_to_double(hi[j], lo[j], e0 + ec);
+            sdst[j] = __uint_as_float(sv[j]);
           }
       }
     }
@@ -441,17 +509,167 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   }
 }
 
+// S[0] += the sums of the other splits
+__global__ void __launch_bounds__(256) f64_sum_kernel(float* S, long long plane, int nsplit) {
+  for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < plane; i += (long long)gridDim.x * 256) {
+    float s = S[i];
+#pragma unroll 8
+    for (int z = 1; z < nsplit; ++z) s += S[z * plane + i];
+    S[i] = s;
+  }
+}
+
+// The entries that the digits do not give as well as an FP64 sum, from the operands themselves: a warp
+// sums up to four entries of a row at a time, in 32 chains and a tree, each by itself, so that an entry's bits
+// do not depend on which others failed.  A 64 x 64 tile and one split per CTA.  Where nothing failed this reads
+// S; where all did the FP64 pipe bounds it, as it does gemm_nt_f64_kernel.
+__global__ void __launch_bounds__(256)
+    f64_fix_kernel(const double* __restrict__ A, long long lda, const double* __restrict__ B, long long ldb,
+                   double* __restrict__ C, long long ldc, long long split_stride, int M, int N, long long K,
+                   long long per, const float* __restrict__ S, const unsigned long long* __restrict__ qa,
+                   const int* __restrict__ ea, const unsigned long long* __restrict__ qb, const int* __restrict__ eb,
+                   int upper) {
+  constexpr int T = 64;
+  __shared__ float na[T], nb[T];            // 2^-9 |alpha|; infinite for a row that is not finite
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  int bx = blockIdx.x, by = blockIdx.y;
+  if (upper) {
+    const int nt = (M + T - 1) / T;
+    int t = blockIdx.x, ti = 0;
+    while (t >= nt - ti) {
+      t -= nt - ti;
+      ++ti;
+    }
+    by = ti;
+    bx = ti + t;
+  }
+  const int m0 = by * T, n0 = bx * T;
+  if (tid < 2 * T) {
+    const bool second = tid >= T;
+    const int i = tid & (T - 1), r = (second ? n0 : m0) + i;
+    float v = 0.0f;
+    if (r < (second ? N : M))
+      v = (second ? eb : ea)[r] == NON_FINITE
+              ? __int_as_float(0x7f800000)
+              : kTrust * 3.0517578125e-5f * sqrtf((float)(second ? qb : qa)[r]);   // 2^-15 sqrt(q)
+    (second ? nb : na)[i] = v;
+  }
+  __syncthreads();
+  // this warp's 32 columns of 16 rows
+  const int j0 = (warp & 1) * 32, c = n0 + j0 + lane;
+  const float line_c = nb[j0 + lane];
+  float s[16];
+#pragma unroll
+  for (int u = 0; u < 16; ++u) {
+    const int r = m0 + (warp >> 1) + 4 * u;
+    s[u] = r < M && c < N ? S[(long long)r * N + c] : 0.0f;
+  }
+  const long long k_lo = (long long)blockIdx.z * per, k_hi = k_lo + per < K ? k_lo + per : K;
+  double* Cz = C + (long long)blockIdx.z * split_stride;
+#pragma unroll
+  for (int u = 0; u < 16; ++u) {
+    const int i = (warp >> 1) + 4 * u, r = m0 + i;
+    const float line = na[i] + line_c;
+    // a sum of exact zeros needs nothing; an infinite line is never reached
+    const bool good = s[u] >= line || (s[u] == 0.0f && line < __int_as_float(0x7f800000));
+    unsigned todo = __ballot_sync(0xffffffffu, r < M && c < N && !(upper && c < r) && !good);
+    while (todo != 0u) {
+      int col[4], cnt = 0;
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        col[q] = n0 + j0;
+        if (todo != 0u) {
+          col[q] += __ffs(todo) - 1;
+          todo &= todo - 1u;
+          cnt = q + 1;
+        }
+      }
+      const double* a = A + (long long)r * lda;
+      double acc[4] = {0.0, 0.0, 0.0, 0.0};
+      for (long long k = k_lo + lane; k < k_hi; k += 32) {
+        const double x = a[k];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          if (q < cnt) acc[q] = fma(x, B[(long long)col[q] * ldb + k], acc[q]);
+      }
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        if (q >= cnt) break;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
+        if (lane == 0) Cz[(long long)r * ldc + col[q]] = acc[q];
+      }
+    }
+  }
+}
+
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
 namespace {
-constexpr long long kWsCap = 512LL << 20;   // digits of a pass; larger products go in several passes
+constexpr size_t kWsCap = (size_t)512 << 20;    // workspace of a pass; larger products go in several passes
+constexpr size_t kSumCap = (size_t)64 << 20;    // of it, for the sums of alpha beta of all splits
+constexpr int kMostChunks = 8192;               // of one 64-bit sum
 
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 int padded(long long K) { return (int)((K + TK - 1) / TK * TK); }
-size_t ws_of(long long rows_a, long long rows_b, long long K) {
-  return align256((size_t)16 * padded(K) * rows_a) + align256((size_t)16 * padded(K) * rows_b) +
-         align256(4 * (size_t)rows_a) + align256(4 * (size_t)rows_b);
+size_t plane_bytes(long long rows, long long K) { return align256((size_t)2 * PLANES * padded(K) * rows); }
+size_t row_bytes(long long rows) { return align256((size_t)12 * rows); }
+size_t operand_bytes(long long rows, long long K) { return plane_bytes(rows, K) + row_bytes(rows); }
+
+// bytes that a row of B takes: its planes, its norm and exponent, a column of sums
+double column_bytes(long long M, long long K) { return 2.0 * PLANES * padded(K) + 12.0 + 4.0 * M; }
+// whether a product without partials is done in a workspace of `cap` bytes: room for A and 256 rows of B.  It
+// depends on M and K alone, so that the columns of a product may come in any groups.
+bool fits(long long M, long long K, size_t cap) {
+  return (double)cap - (double)operand_bytes(M, K) - 4096.0 >= 256.0 * column_bytes(M, K) &&
+         (padded(K) / TK + CHUNK - 1) / CHUNK <= kMostChunks;
+}
+
+// How a product goes through a workspace of `cap` bytes: whole, in passes along K (each leaves partials of its own;
+// where partials are allowed), or along N.
+struct Plan {
+  long long kp;      // terms of a pass
+  int pieces;        // passes along K
+  int np;            // columns of a pass
+  int nsplit;        // most splits of a pass
+  bool shared;       // B's planes are A's
+  size_t bytes;
+};
+bool make_plan(long long M, long long N, long long K, bool same, int max_split, size_t cap, Plan* p) {
+  p->kp = K;
+  p->pieces = 1;
+  p->np = (int)N;
+  p->nsplit = 1;
+  p->shared = same;
+  if (max_split > 1) {
+    const size_t plane = (size_t)4 * M * N;
+    p->nsplit = (int)std::max<size_t>(1, std::min<size_t>((size_t)max_split, kSumCap / plane));
+    const size_t sums = align256(plane * p->nsplit);
+    p->bytes = operand_bytes(M, K) + (same ? 0 : operand_bytes(N, K)) + sums;
+    if (p->bytes > cap) {
+      const double rows = (double)(M + (same ? 0 : N));
+      const double left = (double)cap - (double)sums - 12.0 * rows - 4096.0;
+      p->kp = (long long)(left / (2.0 * PLANES * rows)) / 128 * 128;
+      if (p->kp < 1024) return false;
+      p->pieces = (int)((K + p->kp - 1) / p->kp);
+      if (p->pieces > max_split) return false;
+      p->nsplit = std::min(p->nsplit, max_split / p->pieces);
+      p->bytes = operand_bytes(M, p->kp) + (same ? 0 : operand_bytes(N, p->kp)) + sums;
+      if (p->bytes > cap) return false;
+    }
+    return (padded(p->kp) / TK + CHUNK - 1) / CHUNK <= (long long)kMostChunks * p->nsplit;
+  }
+  const size_t a = operand_bytes(M, K);
+  p->bytes = a + (same ? 0 : operand_bytes(N, K)) + align256((size_t)4 * M * N);
+  if (p->bytes > cap) {
+    const double rows = ((double)cap - (double)a - 4096.0) / column_bytes(M, K);
+    if (rows < 64.0) return false;
+    p->shared = false;
+    p->np = (int)std::min((double)N, rows) / 64 * 64;
+    p->bytes = a + operand_bytes(p->np, K) + align256((size_t)4 * M * p->np);
+  }
+  return p->bytes <= cap;
 }
 
 bool smem_attr_set() {
@@ -459,10 +677,7 @@ bool smem_attr_set() {
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return false;
   if (dev >= 0 && dev < kMaxDevices && done[dev].load(std::memory_order_acquire)) return true;
-  if (cudaFuncSetAttribute(f64_tc_kernel<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(8)) !=
-          cudaSuccess ||
-      cudaFuncSetAttribute(f64_tc_kernel<9>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(9)) != cudaSuccess)
-    return false;
+  if (!raise_smem_limit(f64_tc_kernel, SMEM_BYTES)) return false;
   if (dev >= 0 && dev < kMaxDevices) done[dev].store(1, std::memory_order_release);
   return true;
 }
@@ -479,12 +694,12 @@ int launch_slices(const SliceDesc& a, const SliceDesc& b, long long K, cudaStrea
     ++g_launches;
     return 0;
   }
-  if (rows > 65535) return -1;
-  if ((a.rows && cudaMemsetAsync(a.e, 0, 4 * (size_t)a.rows, s) != cudaSuccess) ||
-      (b.rows && cudaMemsetAsync(b.e, 0, 4 * (size_t)b.rows, s) != cudaSuccess))
+  // q and e of an operand are one array
+  if ((a.rows && cudaMemsetAsync(a.q, 0, 12 * (size_t)a.rows, s) != cudaSuccess) ||
+      (b.rows && cudaMemsetAsync(b.q, 0, 12 * (size_t)b.rows, s) != cudaSuccess))
     return -1;
   const long long most = (K + 2047) / 2048, fill = (8LL * sm_count() + rows - 1) / rows;
-  const dim3 grid((unsigned)std::max(1LL, std::min(most, fill)), (unsigned)rows);
+  const dim3 grid((unsigned)rows, (unsigned)std::max(1LL, std::min({most, fill, 65535LL})));
   slice_max_kernel<<<grid, 256, 0, s>>>(a, b, K);
   slice_long_kernel<<<grid, 256, 0, s>>>(a, b, K, kpad);
   g_launches += 2;
@@ -497,17 +712,17 @@ int launch_slices(const SliceDesc& a, const SliceDesc& b, long long K, cudaStrea
 // terms (2D runs: K = chi_c chi_j) stays on the pipe too: at a degenerate cut the kept vector follows the
 // rounding of the Gram (ordered 2D phase, chi = 24, step 11: a pair 2.8e-15 lambda_1 apart), and such runs
 // go on as they did; it would save 0.1 ms of a Gram of 576 rows.
-size_t f64_tc_bytes(long long M, long long N, long long K, bool same, int upper) {
+size_t f64_tc_bytes(long long M, long long N, long long K, bool same, int upper, int max_split, size_t cap) {
+  if (cap > kWsCap) cap = kWsCap;
   if (M < 32 || N < 16 || K < 32 || M >= (1LL << 31) || N >= (1LL << 31) || K >= (1LL << 31) - TK) return 0;
   if (same && K < 1024) return 0;
   if ((double)M * (double)N * (double)K * (upper ? 0.5 : 1.0) < 16777216.0) return 0;
-  return std::min(ws_of(M, same ? 0 : N, K), (size_t)kWsCap);
+  if (max_split <= 1 && !fits(M, K, cap)) return 0;
+  Plan p;
+  return make_plan(M, N, K, same, max_split, cap, &p) ? p.bytes : 0;
 }
 
-double f64_tc_column_bytes(long long M, long long K) {
-  (void)M;
-  return 16.0 * padded(K) + 4.0;
-}
+double f64_tc_column_bytes(long long M, long long K) { return column_bytes(M, K); }
 
 // Partial products written (at most max_split); 0: not done (the caller takes the FP64 pipe),
 // negative: an error
@@ -515,61 +730,43 @@ int launch_gemm_nt_f64_tc(const double* A, long long lda, const double* B, long 
                           long long split_stride, int M, int N, long long K, int max_split, int upper_only, void* ws,
                           size_t ws_bytes, int* err_flag, cudaStream_t s) {
   const bool same = A == B && lda == ldb && M == N;
-  if (!ws || !tc_gemm_ready() || !smem_attr_set()) return 0;
-  // passes along K (more partials) or along N, so that the digits fit the workspace
-  long long kp = K;
-  int np = N;
-  if (ws_of(M, same ? 0 : N, K) > ws_bytes) {
-    if (max_split > 1) {
-      const double per = 16.0 * (M + (same ? 0 : N));
-      kp = (long long)(((double)ws_bytes - 4096.0 - 8.0 * (M + (double)N)) / per) / 128 * 128;
-      if (kp < 1024 || (K + kp - 1) / kp > max_split) return 0;
-    } else {
-      if (same) return 0;
-      const double left = (double)ws_bytes - 4096.0 - (16.0 * padded(K) + 4.0) * M;
-      const double rows = left / (16.0 * padded(K) + 4.0);
-      if (rows < 256.0) return 0;
-      np = (int)std::min((double)N, rows) / 64 * 64;
-    }
-  }
-  if (K > 2048 && (long long)M + np > 65535) {
-    if (M > 32768) return 0;
-    np = std::min(np, 32704);
-  }
-  const int pieces = (int)((K + kp - 1) / kp);
-  const int accs = same ? 9 : 8, TN = tile_n(accs);
-  if (np < N && (same || pieces > 1)) return 0;
+  Plan pl;
+  if (!ws || !tc_gemm_ready() || !smem_attr_set() || !make_plan(M, N, K, same, max_split, ws_bytes, &pl)) return 0;
+  if (upper_only && pl.np < N) return 0;
   int used = 0;
-  for (int p = 0; p < pieces; ++p) {
-    const long long k0 = p * kp, Kp = std::min(kp, K - k0);
+  for (int p = 0; p < pl.pieces; ++p) {
+    const long long k0 = p * pl.kp, Kp = std::min(pl.kp, K - k0);
     const int kpad = padded(Kp);
     char* w = (char*)ws;
-    SliceDesc a, b;
-    a.x = A + k0;
-    a.ld = lda;
-    a.rows = M;
-    a.v = (__nv_bfloat16*)w;
-    w += align256((size_t)16 * kpad * M);
-    b = a;
-    if (!same) {
-      b.v = (__nv_bfloat16*)w;
-      w += align256((size_t)16 * kpad * np);
-    }
-    a.e = (int*)w;
-    b.e = same ? a.e : (int*)(w + align256(4 * (size_t)M));
-    for (int n0 = 0; n0 < N; n0 += np) {
-      const int nc = std::min(np, N - n0);
-      SliceDesc sa = a, sb = b;
-      if (!same) {
-        sb.x = B + (long long)n0 * ldb + k0;
-        sb.ld = ldb;
+    auto operand = [&](const double* x, long long ld, int rows) {
+      SliceDesc d;
+      d.x = x + k0;
+      d.ld = ld;
+      d.rows = rows;
+      d.v = (__nv_bfloat16*)w;
+      w += plane_bytes(rows, Kp);
+      d.q = (unsigned long long*)w;
+      d.e = (int*)(d.q + rows);
+      w += row_bytes(rows);
+      return d;
+    };
+    const SliceDesc a = operand(A, lda, M), b0 = pl.shared ? a : operand(B, ldb, pl.np);
+    float* sums = (float*)w;
+    for (int n0 = 0; n0 < N; n0 += pl.np) {
+      const int nc = std::min(pl.np, N - n0);
+      SliceDesc b = b0, sa = a;
+      if (!pl.shared) {
+        b.x = B + (long long)n0 * ldb + k0;
+        b.rows = nc;
+        b.e = (int*)(b.q + nc);
       }
-      sb.rows = same ? 0 : nc;
-      if (n0 > 0) sa.rows = 0;   // the digits of A are there
+      SliceDesc sb = b;
+      if (pl.shared) sb.rows = 0;
+      if (n0 > 0) sa.rows = 0;   // the planes of A are there
       if (launch_slices(sa, sb, Kp, s) != 0) return -1;
       CUtensorMap ma, mb;
-      if (make_piece_map(&ma, a.v, M, kpad, DIG, TM, TK, false, DIG) ||
-          make_piece_map(&mb, b.v, same ? M : nc, kpad, DIG, TN, TK, false, DIG))
+      if (make_piece_map(&ma, a.v, M, kpad, PLANES, TM, TK, false, PLANES) ||
+          make_piece_map(&mb, b.v, nc, kpad, PLANES, TN, TK, false, PLANES))
         return -1;
       TcItems it;
       it.M = M;
@@ -584,14 +781,13 @@ int launch_gemm_nt_f64_tc(const double* A, long long lda, const double* B, long 
       }
       it.slabs = kpad / TK;
       const int chunks = (it.slabs + CHUNK - 1) / CHUNK;
-      if (chunks > 8192 * (long long)std::max(1, max_split / pieces)) return -1;   // 64-bit sums: 2^14 chunks
       // splits: the rounds of the items over the SMs times an item's chunks, the epilogue as two more
       const long long sms = sm_count();
       long long best = -1;
       int ns_best = 1;
-      for (int ns = 1; ns <= std::max(1, std::min(max_split / pieces, chunks)); ++ns) {
+      for (int ns = 1; ns <= std::max(1, std::min(pl.nsplit, chunks)); ++ns) {
         const int cps = (chunks + ns - 1) / ns;
-        if (cps > 8192) continue;
+        if (cps > kMostChunks) continue;
         const int real = (chunks + cps - 1) / cps;
         const long long cost = ((long long)it.ntiles * real + sms - 1) / sms * (cps + 2);
         if (best < 0 || cost < best) {
@@ -603,8 +799,19 @@ int launch_gemm_nt_f64_tc(const double* A, long long lda, const double* B, long 
       it.nsplit = (chunks + cps - 1) / cps;
       it.per = cps * CHUNK;
       const long long items = (long long)it.ntiles * it.nsplit;
-      (same ? f64_tc_kernel<9> : f64_tc_kernel<8>)<<<(unsigned)std::min(items, sms), NTHREADS, smem_bytes(accs), s>>>(
-          ma, mb, a.e, b.e, C + n0 + (long long)used * split_stride, ldc, split_stride, it, err_flag);
+      double* Cp = C + n0 + (long long)used * split_stride;
+      f64_tc_kernel<<<(unsigned)std::min(items, sms), NTHREADS, SMEM_BYTES, s>>>(ma, mb, a.e, b.e, Cp, ldc, split_stride,
+                                                                                 sums, it, err_flag);
+      ++g_launches;
+      if (it.nsplit > 1) {
+        const long long plane = (long long)M * nc;
+        f64_sum_kernel<<<(unsigned)std::min((plane + 255) / 256, 8 * sms), 256, 0, s>>>(sums, plane, it.nsplit);
+        ++g_launches;
+      }
+      const int ft = (M + 63) / 64;
+      const dim3 grid = upper_only ? dim3(ft * (ft + 1) / 2, 1, it.nsplit) : dim3((nc + 63) / 64, ft, it.nsplit);
+      f64_fix_kernel<<<grid, 256, 0, s>>>(a.x, lda, b.x, ldb, Cp, ldc, split_stride, M, nc, Kp,
+                                          (long long)it.per * TK, sums, a.q, a.e, b.q, b.e, upper_only);
       ++g_launches;
       if (n0 + nc >= N) used += it.nsplit;
     }
