@@ -126,7 +126,8 @@ int hotrg_set_fp64_threshold(hotrg_ctx* ctx, double flops);
  * intermediates).  Small c'-slices of the new-tensor contraction (Sec. 4.2.9)
  * share a pass, and large ones are cut into sub-ranges of n'_1, so that a pass
  * fits the smaller of this cap and 60 % of the free device memory (one n'_1
- * value of one slice at the least).  Default 160e9. */
+ * value of one slice at the least).  The results do not depend on it, bit for
+ * bit, while the workspaces can be had.  Default 160e9. */
 int hotrg_set_slice_budget(hotrg_ctx* ctx, double bytes);
 
 /* Z2 (spin-flip) block form of the new-tensor contraction; enable = 1 is the

@@ -22,6 +22,7 @@
 #include <map>
 #include <vector>
 
+#include "f64_rule.h"
 #include "hotrg_internal.cuh"
 #include "partials.h"
 #include "../../include/hotrg.h"
@@ -366,14 +367,14 @@ int launch_failed(hotrg_ctx* c, const char* what, long long a, long long b, long
   return HOTRG_ECUDA;
 }
 
-// C = A . B^T in FP64: on the tensor cores where the product is large enough and the workspace can be
-// had, else on the FP64 pipe.  nsplit > 1: split along K, at most nsplit_most partials.  Returns the
-// partials written: none if a launch was refused (the context is then poisoned).
-int gemm64(hotrg_ctx* c, const double* A, long long lda, const double* B, long long ldb, double* C, long long ldc,
-           long long split_stride, int M, int N, long long K, int nsplit, int upper_only, cudaStream_t s,
+// C = A . B^T in FP64: on the tensor cores if `digits` and the workspace can be had, else on the FP64 pipe.
+// nsplit > 1: split along K, at most nsplit_most partials.  Returns the partials written: none if a launch was
+// refused (the context is then poisoned).
+int gemm64(hotrg_ctx* c, bool digits, const double* A, long long lda, const double* B, long long ldb, double* C,
+           long long ldc, long long split_stride, int M, int N, long long K, int nsplit, int upper_only, cudaStream_t s,
            int nsplit_most = 1) {
   const int most = std::max(nsplit, nsplit_most);
-  const size_t want = f64_tc_bytes(M, N, K, A == B && lda == ldb && M == N, upper_only, most);
+  const size_t want = digits ? f64_tc_bytes(M, N, K, A == B && lda == ldb && M == N, most) : 0;
   if (want > 0) {
     // in eighths of a power of two: a run's bond dimensions grow, its workspace seldom, and an eighth is
     // the most that it takes beyond its need
@@ -381,7 +382,8 @@ int gemm64(hotrg_ctx* c, const double* A, long long lda, const double* B, long l
     while (step * 16 <= want) step <<= 1;
     const size_t size = (want + step - 1) / step * step;
     if (c->Wd.bytes >= want || dev_alloc(c, c->Wd, size) == HOTRG_OK) {
-      const int r = launch_gemm_nt_f64_tc(A, lda, B, ldb, C, ldc, split_stride, M, N, K, most, upper_only, c->Wd.p, c->Wd.bytes, &((DevState*)c->state.p)->status, s);
+      const int r = launch_gemm_nt_f64_tc(A, lda, B, ldb, C, ldc, split_stride, M, N, K, most, upper_only, c->Wd.p,
+                                          c->Wd.bytes, &((DevState*)c->state.p)->status, s);
       if (r > 0) return r;
       if (r < 0) return partials_written(launch_failed(c, "FP64 product on the tensor cores", M, N, K));
     }
@@ -1085,8 +1087,8 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
           if (mb == 0 || Kb == 0) continue;
           const int nsplit = gram_splits(mb, Kb);
           double* pdst = (double*)c->parts.p + poff;
-          nsb[b] = gemm64(c, X + r0 * K + k0, K, X + r0 * K + k0, K, pdst, mb, mb * mb, (int)mb,
-                                      (int)mb, Kb, nsplit, 1, s, nsplit_max);
+          nsb[b] = gemm64(c, f64_gram_digits_pay(mb, Kb, true), X + r0 * K + k0, K, X + r0 * K + k0, K, pdst, mb, mb * mb,
+                          (int)mb, (int)mb, Kb, nsplit, 1, s, nsplit_max);
           pb[b] = pdst;
           poff += (long long)nsb[b] * mb * mb;
         }
@@ -1105,8 +1107,8 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
       const int nsplit = gram_splits(m, Kp);
       // the GEMM may round nsplit down: reduce the partials it wrote
       const double* X0 = (const double*)c->Xp.p + k_lo;
-      const int used = gemm64(c, X0, K, X0, K, (double*)c->parts.p, m, m * m, (int)m, (int)m, Kp,
-                                          nsplit, 1, s, nsplit_max);
+      const int used = gemm64(c, f64_gram_digits_pay(m, Kp, true), X0, K, X0, K, (double*)c->parts.p, m, m * m, (int)m,
+                              (int)m, Kp, nsplit, 1, s, nsplit_max);
       launch_reduce_sym((const double*)c->parts.p, used, (int)m, Sdst, s);
     }
     double* S0 = (double*)c->S.p + ((long long)(j - 1) * 4) * mmax * mmax;
@@ -1354,8 +1356,8 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
             const long long r0 = b == 0 ? 0 : gz_mb[j][0], q0 = b == 0 ? 0 : gz_Kb[j][kind][0];
             const int nsplit = gram_splits(mb, Kb);
             double* pdst = (double*)c->parts.p + poff;
-            nsb[b] = gemm64(c, dX + r0 * K + q0, K, X + r0 * K + q0, K, pdst, mb, mb * mb, (int)mb,
-                                        (int)mb, Kb, nsplit, 0, s, nsplit_max);
+            nsb[b] = gemm64(c, f64_digits_pay(mb, mb, Kb, false), dX + r0 * K + q0, K, X + r0 * K + q0, K, pdst, mb, mb * mb,
+                            (int)mb, (int)mb, Kb, nsplit, 0, s, nsplit_max);
             pb[b] = pdst;
             poff += (long long)nsb[b] * mb * mb;
           }
@@ -1367,8 +1369,9 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
         launch_permute(Tc, (double*)c->Xp.p, nd, size, ist, 1.0, s);
         launch_permute((const double*)c->dT.p, (double*)c->dXp.p, nd, size, ist, 1.0, s);
         const int nsplit = gram_splits(m, K);
-        const int used = gemm64(c, (const double*)c->dXp.p, K, (const double*)c->Xp.p, K,
-                                            (double*)c->parts.p, m, m * m, (int)m, (int)m, K, nsplit, 0, s, nsplit_max);
+        const bool digits = f64_digits_pay(m, m, K, false);
+        const int used = gemm64(c, digits, (const double*)c->dXp.p, K, (const double*)c->Xp.p, K,
+                                (double*)c->parts.p, m, m * m, (int)m, (int)m, K, nsplit, 0, s, nsplit_max);
         launch_sym_sum((const double*)c->parts.p, used, (int)m, dS0 + kind * mmax * mmax, s);
         if (tan2) {
           // d2S = d2X X^T + X d2X^T + 2 dX dX^T: the partials of d2X X^T and of dX dX^T (each
@@ -1376,10 +1379,10 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
           double* d2S0 = (double*)c->d2S.p + ((long long)(j - 1) * 4) * mmax * mmax;
           launch_permute((const double*)c->d2T.p, (double*)c->d2Xp.p, nd, size, ist, 1.0, s);
           double* p2 = (double*)c->parts2.p;
-          const int u1 = gemm64(c, (const double*)c->d2Xp.p, K, (const double*)c->Xp.p, K, p2, m, m * m,
-                                            (int)m, (int)m, K, nsplit, 0, s, nsplit_max);
-          const int u2 = gemm64(c, (const double*)c->dXp.p, K, (const double*)c->dXp.p, K,
-                                            p2 + (long long)u1 * m * m, m, m * m, (int)m, (int)m, K, nsplit, 0, s, nsplit_max);
+          const int u1 = gemm64(c, digits, (const double*)c->d2Xp.p, K, (const double*)c->Xp.p, K, p2, m, m * m,
+                                (int)m, (int)m, K, nsplit, 0, s, nsplit_max);
+          const int u2 = gemm64(c, f64_gram_digits_pay(m, K, false), (const double*)c->dXp.p, K, (const double*)c->dXp.p,
+                                K, p2 + (long long)u1 * m * m, m, m * m, (int)m, (int)m, K, nsplit, 0, s, nsplit_max);
           launch_sym_sum(p2, u1 + u2, (int)m, d2S0 + kind * mmax * mmax, s);
         }
       }
@@ -1408,7 +1411,7 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
                              S0 + (k0 + 1) * mmax * mmax, dS0 + (k0 + 1) * mmax * mmax,
                              d2S0 + (k0 + 1) * mmax * mmax, chij[j], chi_c, d2As, s);
         launch_gemm_nn_f64(Vs, n, dAs, n, (double*)c->eW.p, n, n, n, n, 1, 0, 0, 0, s);       // rows dA v_a
-        gemm64(c, (const double*)c->eW.p, n, Vs, n, (double*)c->eG1.p, n, 0, n, n, n, 1, 0, s);
+        gemm64(c, f64_digits_pay(n, n, n, false), (const double*)c->eW.p, n, Vs, n, (double*)c->eG1.p, n, 0, n, n, n, 1, 0, s);
         launch_gemm_nn_f64(d2As, n, (const double*)c->U64.p + u_off[j], nn, G, nn, n, nn, n, 1, 0, 0, 0, s);
         launch_gemm_nn_f64(Vs, n, G, nn, (double*)c->eZ2.p, nn, n, nn, n, 1, 0, 0, 0, s);    // v_i . d2A u_k
         launch_eig_d2((const double*)c->eG1.p, (const double*)c->eZ.p, (const double*)c->eZ2.p,
@@ -1487,6 +1490,10 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
   // Sub-slices of n'_1 keep the per-slice operands within a device-memory budget:
   // everything below except the split T scales with the number of n'_1 values.
   const int nnew1 = nnew[1];
+  // the FP64 form's products as digits or on the pipe: by the size of the whole step, whatever groups the
+  // slices come in (with parity blocks, half of each dimension)
+  const double half = z2 ? 0.5 : 1.0;
+  const bool digits = fp64 && f64_digits_pay(half * R, half * (double)Ns * chi_c, half * R, false);
   int n1_chunk = nnew1;
   double per_unit = 1.0;   // operand bytes of one n'_1 value of a slice
   double budget = 0.0, digits_unit = 0.0;
@@ -1504,7 +1511,7 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
                                                       c->Zb.bytes + c->Zc.bytes + c->Wd.bytes),
                       c->slice_budget_bytes);
     // the digits of B in an FP64 product on the tensor cores (their workspace grows in steps of an eighth)
-    if (fp64) digits_unit = 1.125 * f64_tc_column_bytes(R, R) * (double)(Ns / nnew1);
+    if (digits) digits_unit = 1.125 * f64_tc_column_bytes(R, R) * (double)(Ns / nnew1);
     n1_chunk = (int)std::max(1.0, std::min((double)nnew1, std::floor(budget / (per_unit + digits_unit))));
   }
   // Small slices share a pass: c' becomes one more index of the columns (c', n', n~), so that a step
@@ -1999,8 +2006,8 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
             launch_z2_gather_f64((const double*)c->Bp.p, R, nmap, (int)Nb, kmap, (int)Kpb[b], zb, s);
           }
           Phase ph(c, 6);
-          gemm64(c, (const double*)c->Za.p + a_off, Kpb[b], zb, Kpb[b], zc, ldz, 0, (int)Rb[b],
-                             (int)Nb, Kpb[b], 1, 0, s);
+          gemm64(c, digits, (const double*)c->Za.p + a_off, Kpb[b], zb, Kpb[b], zc, ldz, 0, (int)Rb[b], (int)Nb, Kpb[b], 1, 0,
+                 s);
           cblk[b] = zc;
         } else {
           char* zb = (char*)c->Zb.p + pbytes * npieces * b_off;
@@ -2036,23 +2043,20 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
     bn_done += 2.0 * (double)R * (double)Nc * (double)R;
     Phase ph(c, 6);
     if (fp64) {
-      gemm64(c, Tc, R, (const double*)c->Bp.p, R, (double*)c->Cb.p, Nc, 0, (int)R, (int)Nc,
-                         R, 1, 0, s);
+      gemm64(c, digits, Tc, R, (const double*)c->Bp.p, R, (double*)c->Cb.p, Nc, 0, (int)R, (int)Nc, R, 1, 0, s);
       if (tangent) {   // dC = T^ . dB^T + dT^ . B^T
-        gemm64(c, Tc, R, (const double*)c->dBp.p, R, (double*)c->dCb.p, Nc, 0, (int)R, (int)Nc, R, 1,
-                           0, s);
-        gemm64(c, (const double*)c->dT.p, R, (const double*)c->Bp.p, R, (double*)c->tCb.p, Nc, 0,
-                           (int)R, (int)Nc, R, 1, 0, s);
+        gemm64(c, digits, Tc, R, (const double*)c->dBp.p, R, (double*)c->dCb.p, Nc, 0, (int)R, (int)Nc, R, 1, 0, s);
+        gemm64(c, digits, (const double*)c->dT.p, R, (const double*)c->Bp.p, R, (double*)c->tCb.p, Nc, 0, (int)R,
+               (int)Nc, R, 1, 0, s);
         launch_axpby(1.0, (const double*)c->tCb.p, 1.0, (double*)c->dCb.p, R * Nc, s);
       }
       if (tan2) {      // d2C = T^ . d2B^T + 2 dT^ . dB^T + d2T^ . B^T
-        gemm64(c, Tc, R, (const double*)c->d2Bp.p, R, (double*)c->d2Cb.p, Nc, 0, (int)R, (int)Nc, R, 1,
-                           0, s);
-        gemm64(c, (const double*)c->dT.p, R, (const double*)c->dBp.p, R, (double*)c->tCb.p, Nc, 0,
-                           (int)R, (int)Nc, R, 1, 0, s);
+        gemm64(c, digits, Tc, R, (const double*)c->d2Bp.p, R, (double*)c->d2Cb.p, Nc, 0, (int)R, (int)Nc, R, 1, 0, s);
+        gemm64(c, digits, (const double*)c->dT.p, R, (const double*)c->dBp.p, R, (double*)c->tCb.p, Nc, 0, (int)R,
+               (int)Nc, R, 1, 0, s);
         launch_axpby(2.0, (const double*)c->tCb.p, 1.0, (double*)c->d2Cb.p, R * Nc, s);
-        gemm64(c, (const double*)c->d2T.p, R, (const double*)c->Bp.p, R, (double*)c->tCb.p, Nc, 0,
-                           (int)R, (int)Nc, R, 1, 0, s);
+        gemm64(c, digits, (const double*)c->d2T.p, R, (const double*)c->Bp.p, R, (double*)c->tCb.p, Nc, 0, (int)R,
+               (int)Nc, R, 1, 0, s);
         launch_axpby(1.0, (const double*)c->tCb.p, 1.0, (double*)c->d2Cb.p, R * Nc, s);
       }
     } else {
@@ -2420,7 +2424,7 @@ int hotrg_gemm_nt(int mode, int M, int N, int K, const double* A, const double* 
     cudaMemcpy(dB, B, sizeof(double) * N * K, cudaMemcpyDefault);
     cudaMemset(err, 0, sizeof(int));
     if (mode == HOTRG_PREC_FP64) {
-      const size_t want = f64_tc_bytes(M, N, K, false, 0, 1);
+      const size_t want = f64_digits_pay(M, N, K, false) ? f64_tc_bytes(M, N, K, false, 1) : 0;
       int r = 0;
       if (want > 0) {
         if (cudaMalloc(&pA, want) == cudaSuccess)

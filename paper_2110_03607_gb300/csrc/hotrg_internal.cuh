@@ -384,9 +384,8 @@ int measure_tc_gemm_rate(int npieces, int M, int N, int Kpad, int iters, double*
                          int pfmt = PIECE_BF16);
 
 // ---- kernels_f64_tc.cu: the FP64 products on the tensor cores, C = A . B^T as launch_gemm_nt_f64
-// workspace wanted, at most `cap` (0: the product is left to the FP64 pipe)
-size_t f64_tc_bytes(long long M, long long N, long long K, bool same, int upper, int max_split,
-                    size_t cap = ~(size_t)0);
+// workspace wanted, at most `cap` (0: the product does not go through that much and is left to the FP64 pipe)
+size_t f64_tc_bytes(long long M, long long N, long long K, bool same, int max_split, size_t cap = ~(size_t)0);
 // of it, the bytes that one more row of B takes
 double f64_tc_column_bytes(long long M, long long K);
 // partials written (<= max_split); 0: not done; negative: an error

@@ -6,6 +6,7 @@
 
 #include <mutex>
 
+#include "f64_rule.h"
 #include "hotrg_internal.cuh"
 #include "../../include/hotrg.h"
 
@@ -84,7 +85,7 @@ extern "C" int hotrg_gemm_nt_noalloc(int mode, int M, int N, int K, const double
   if (cudaMemsetAsync(err, 0, sizeof(int), s) != cudaSuccess) status = HOTRG_ECUDA;
   if (status == HOTRG_OK && mode == HOTRG_PREC_FP64) {
     int r = 0;
-    if (f64_tc_bytes(M, N, K, false, 0, 1, kScratchBytes - off_a) > 0)   // the digits of B in passes over what the array holds
+    if (f64_digits_pay(M, N, K, false) && f64_tc_bytes(M, N, K, false, 1, kScratchBytes - off_a) > 0)   // the digits of B in passes over what the array holds
       r = launch_gemm_nt_f64_tc(A, K, B, K, C, N, 0, M, N, K, 1, 0, base + off_a, kScratchBytes - off_a, err, s);
     if (r == 0) launch_gemm_nt_f64(A, K, B, K, C, N, 0, M, N, K, 1, 0, s);
     if (r < 0) status = HOTRG_ECUDA;

@@ -707,16 +707,9 @@ int launch_slices(const SliceDesc& a, const SliceDesc& b, long long K, cudaStrea
 }
 }  // namespace
 
-// Where the digits pay: the FP64 pipe does 0.6e12 multiply-adds a second, so 2^24 of them take 28 us
-// there, about as long as the launches and the first tiles of this path.  A Gram over less than 1024
-// terms (2D runs: K = chi_c chi_j) stays on the pipe too: at a degenerate cut the kept vector follows the
-// rounding of the Gram (ordered 2D phase, chi = 24, step 11: a pair 2.8e-15 lambda_1 apart), and such runs
-// go on as they did; it would save 0.1 ms of a Gram of 576 rows.
-size_t f64_tc_bytes(long long M, long long N, long long K, bool same, int upper, int max_split, size_t cap) {
+size_t f64_tc_bytes(long long M, long long N, long long K, bool same, int max_split, size_t cap) {
+  if (M < 1 || N < 1 || K < 1 || M >= (1LL << 31) || N >= (1LL << 31) || K >= (1LL << 31) - TK) return 0;
   if (cap > kWsCap) cap = kWsCap;
-  if (M < 32 || N < 16 || K < 32 || M >= (1LL << 31) || N >= (1LL << 31) || K >= (1LL << 31) - TK) return 0;
-  if (same && K < 1024) return 0;
-  if ((double)M * (double)N * (double)K * (upper ? 0.5 : 1.0) < 16777216.0) return 0;
   if (max_split <= 1 && !fits(M, K, cap)) return 0;
   Plan p;
   return make_plan(M, N, K, same, max_split, cap, &p) ? p.bytes : 0;
