@@ -127,7 +127,7 @@ int hotrg_set_fp64_threshold(hotrg_ctx* ctx, double flops);
  * share a pass, and large ones are cut into sub-ranges of n'_1, so that a pass
  * fits the smaller of this cap and 60 % of the free device memory (one n'_1
  * value of one slice at the least).  The results do not depend on it, bit for
- * bit, while the workspaces can be had.  Default 160e9. */
+ * bit, while its workspace can be had.  Default 160e9. */
 int hotrg_set_slice_budget(hotrg_ctx* ctx, double bytes);
 
 /* Z2 (spin-flip) block form of the new-tensor contraction; enable = 1 is the
@@ -402,8 +402,8 @@ int hotrg_gemm_nt(int mode, int M, int N, int K, const double* A, const double* 
  * np = 2 (BF16X3) or 3 (BF16X6), Kp = K rounded up to a multiple of 64 and
  * r(x) = x rounded up to a multiple of 256; sizes whose scratch exceeds the
  * array are rejected with HOTRG_EINVAL (the FP64 mode works within the array: it holds the
- * digits of the operands, of B in passes where they do not fit, and large products whose A
- * does not fit run on the FP64 pipe).
+ * digits of the operands, in passes where they do not fit).  The results are those of
+ * hotrg_gemm_nt bit for bit.
  * mode is HOTRG_PREC_FP64, HOTRG_PREC_BF16X3 or HOTRG_PREC_BF16X6 (the TF32
  * modes give HOTRG_EINVAL here).  The
  * size limits of hotrg_gemm_nt apply in every mode.  The first call on a device looks up the

@@ -2424,7 +2424,9 @@ int hotrg_gemm_nt(int mode, int M, int N, int K, const double* A, const double* 
     cudaMemcpy(dB, B, sizeof(double) * N * K, cudaMemcpyDefault);
     cudaMemset(err, 0, sizeof(int));
     if (mode == HOTRG_PREC_FP64) {
-      const size_t want = f64_digits_pay(M, N, K, false) ? f64_tc_bytes(M, N, K, false, 1) : 0;
+      // digits where the entry point without allocation takes them too, so that both give the same bits
+      const bool digits = f64_digits_pay(M, N, K, false) && f64_tc_bytes(M, N, K, false, 1, kNoallocWork) > 0;
+      const size_t want = digits ? f64_tc_bytes(M, N, K, false, 1) : 0;
       int r = 0;
       if (want > 0) {
         if (cudaMalloc(&pA, want) == cudaSuccess)

@@ -386,12 +386,15 @@ int measure_tc_gemm_rate(int npieces, int M, int N, int Kpad, int iters, double*
 // ---- kernels_f64_tc.cu: the FP64 products on the tensor cores, C = A . B^T as launch_gemm_nt_f64
 // workspace wanted, at most `cap` (0: the product does not go through that much and is left to the FP64 pipe)
 size_t f64_tc_bytes(long long M, long long N, long long K, bool same, int max_split, size_t cap = ~(size_t)0);
+// what hotrg_gemm_nt_noalloc has for it: its array without the error word
+constexpr size_t kNoallocScratch = (size_t)64 << 20, kNoallocWork = kNoallocScratch - 256;
 // of it, the bytes that one more row of B takes
 double f64_tc_column_bytes(long long M, long long K);
-// partials written (<= max_split); 0: not done; negative: an error
+// partials written (<= max_split); 0: not done; negative: an error.  cap: as given to f64_tc_bytes, from which
+// `same` is A == B with one leading dimension and M == N
 int launch_gemm_nt_f64_tc(const double* A, long long lda, const double* B, long long ldb, double* C, long long ldc,
                           long long split_stride, int M, int N, long long K, int max_split, int upper_only, void* ws,
-                          size_t ws_bytes, int* err_flag, cudaStream_t s);
+                          size_t ws_bytes, int* err_flag, cudaStream_t s, size_t cap = ~(size_t)0);
 
 // ---- kernels_tensor.cu: streaming multiprocessors of the current device (cached per device)
 int sm_count();

@@ -13,10 +13,10 @@
 namespace hotrg {
 namespace {
 
-constexpr size_t kScratchBytes = size_t(64) << 20;  // HOTRG_NOALLOC_SCRATCH_BYTES
+static_assert(kNoallocScratch == HOTRG_NOALLOC_SCRATCH_BYTES, "the array's size is part of the interface");
 
 // Every GPU that loads the library holds this array until the process exits.
-__device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
+__device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocScratch];
 
 std::mutex g_mu;
 unsigned char* g_scratch_ptr[kMaxDevices] = {nullptr};
@@ -79,28 +79,26 @@ extern "C" int hotrg_gemm_nt_noalloc(int mode, int M, int N, int K, const double
   const size_t bytes_b = align256(sizeof(__nv_bfloat16) * np * (size_t)N * Kpad);
   const size_t off_c = off_b + bytes_b;
   const size_t bytes_c = align256(sizeof(float) * (size_t)M * N);
-  if (mode != HOTRG_PREC_FP64 && off_c + bytes_c > kScratchBytes) return HOTRG_EINVAL;
+  if (mode != HOTRG_PREC_FP64 && off_c + bytes_c > kNoallocScratch) return HOTRG_EINVAL;
 
   int* err = (int*)base;
   if (cudaMemsetAsync(err, 0, sizeof(int), s) != cudaSuccess) status = HOTRG_ECUDA;
   if (status == HOTRG_OK && mode == HOTRG_PREC_FP64) {
     int r = 0;
-    if (f64_digits_pay(M, N, K, false) && f64_tc_bytes(M, N, K, false, 1, kScratchBytes - off_a) > 0)   // the digits of B in passes over what the array holds
-      r = launch_gemm_nt_f64_tc(A, K, B, K, C, N, 0, M, N, K, 1, 0, base + off_a, kScratchBytes - off_a, err, s);
+    if (f64_digits_pay(M, N, K, false) && f64_tc_bytes(M, N, K, A == B && M == N, 1, kNoallocWork) > 0)
+      r = launch_gemm_nt_f64_tc(A, K, B, K, C, N, 0, M, N, K, 1, 0, base + off_a, kNoallocWork, err, s, kNoallocWork);
     if (r == 0) launch_gemm_nt_f64(A, K, B, K, C, N, 0, M, N, K, 1, 0, s);
     if (r < 0) status = HOTRG_ECUDA;
   } else if (status == HOTRG_OK) {
     __nv_bfloat16* pa = (__nv_bfloat16*)(base + off_a);
     __nv_bfloat16* pb = (__nv_bfloat16*)(base + off_b);
     float* c32 = (float*)(base + off_c);
-    if (status == HOTRG_OK) {
-      launch_split(A, M, K, K, pa, Kpad, (long long)M * Kpad, np, PIECE_BF16, s);
-      launch_split(B, N, K, K, pb, Kpad, (long long)N * Kpad, np, PIECE_BF16, s);
-      int ta[6], tb[6];
-      const int nt = split_terms(np, ta, tb);
-      if (launch_tc_gemm(pa, M, pb, N, (int)Kpad, np, nt, ta, tb, c32, N, err, s, nullptr, PIECE_BF16) != 0)
-        status = HOTRG_ECUDA;
-    }
+    launch_split(A, M, K, K, pa, Kpad, (long long)M * Kpad, np, PIECE_BF16, s);
+    launch_split(B, N, K, K, pb, Kpad, (long long)N * Kpad, np, PIECE_BF16, s);
+    int ta[6], tb[6];
+    const int nt = split_terms(np, ta, tb);
+    if (launch_tc_gemm(pa, M, pb, N, (int)Kpad, np, nt, ta, tb, c32, N, err, s, nullptr, PIECE_BF16) != 0)
+      status = HOTRG_ECUDA;
     if (status == HOTRG_OK) {
       long long n = (long long)M * N;
       long long blocks = (n + 255) / 256;

@@ -619,19 +619,21 @@ size_t operand_bytes(long long rows, long long K) { return plane_bytes(rows, K) 
 
 // bytes that a row of B takes: its planes, its norm and exponent, a column of sums
 double column_bytes(long long M, long long K) { return 2.0 * PLANES * padded(K) + 12.0 + 4.0 * M; }
-// whether a product without partials is done in a workspace of `cap` bytes: room for A and 256 rows of B.  It
-// depends on M and K alone, so that the columns of a product may come in any groups.
-bool fits(long long M, long long K, size_t cap) {
-  return (double)cap - (double)operand_bytes(M, K) - 4096.0 >= 256.0 * column_bytes(M, K) &&
-         (padded(K) / TK + CHUNK - 1) / CHUNK <= kMostChunks;
+size_t pass_bytes(long long m, long long n, long long K) {
+  return operand_bytes(m, K) + operand_bytes(n, K) + align256((size_t)4 * m * n);
+}
+// whether a product without partials is done in a workspace of `cap` bytes: room for 32 rows of A and 16 of B.  It
+// depends on K alone, so that the rows and columns of a product may come in any groups.
+bool fits(long long K, size_t cap) {
+  return pass_bytes(32, 16, K) <= cap && (padded(K) / TK + CHUNK - 1) / CHUNK <= kMostChunks;
 }
 
 // How a product goes through a workspace of `cap` bytes: whole, in passes along K (each leaves partials of its own;
-// where partials are allowed), or along N.
+// where partials are allowed), or along N, and along M where A and 256 rows of B are more than that.
 struct Plan {
   long long kp;      // terms of a pass
   int pieces;        // passes along K
-  int np;            // columns of a pass
+  int mp, np;        // rows and columns of a pass
   int nsplit;        // most splits of a pass
   bool shared;       // B's planes are A's
   size_t bytes;
@@ -639,6 +641,7 @@ struct Plan {
 bool make_plan(long long M, long long N, long long K, bool same, int max_split, size_t cap, Plan* p) {
   p->kp = K;
   p->pieces = 1;
+  p->mp = (int)M;
   p->np = (int)N;
   p->nsplit = 1;
   p->shared = same;
@@ -660,15 +663,21 @@ bool make_plan(long long M, long long N, long long K, bool same, int max_split, 
     }
     return (padded(p->kp) / TK + CHUNK - 1) / CHUNK <= (long long)kMostChunks * p->nsplit;
   }
-  const size_t a = operand_bytes(M, K);
-  p->bytes = a + (same ? 0 : operand_bytes(N, K)) + align256((size_t)4 * M * N);
-  if (p->bytes > cap) {
-    const double rows = ((double)cap - (double)a - 4096.0) / column_bytes(M, K);
-    if (rows < 64.0) return false;
-    p->shared = false;
-    p->np = (int)std::min((double)N, rows) / 64 * 64;
-    p->bytes = a + operand_bytes(p->np, K) + align256((size_t)4 * M * p->np);
+  p->bytes = same ? operand_bytes(M, K) + align256((size_t)4 * M * N) : pass_bytes(M, N, K);
+  if (p->bytes <= cap) return true;
+  p->shared = false;
+  auto columns = [&](int mp) {   // of a pass of mp rows
+    return (long long)(((double)cap - (double)operand_bytes(mp, K) - 4096.0) / column_bytes(mp, K));
+  };
+  if (columns(p->mp) < std::min(N, 256LL)) {
+    // half of the workspace each: whole tiles of rows if it holds one, else quarters of a tile
+    const long long rows = (long long)(0.5 * (double)cap / (2.0 * PLANES * padded(K) + 12.0));
+    p->mp = (int)std::min(M, std::max(32LL, rows >= TM ? rows / TM * TM : rows / 32 * 32));
   }
+  const long long n = columns(p->mp);
+  p->np = (int)std::min(N, n >= 64 ? n / 64 * 64 : n / 16 * 16);
+  if (p->np < 1) return false;
+  p->bytes = pass_bytes(p->mp, p->np, K);
   return p->bytes <= cap;
 }
 
@@ -709,8 +718,8 @@ int launch_slices(const SliceDesc& a, const SliceDesc& b, long long K, cudaStrea
 
 size_t f64_tc_bytes(long long M, long long N, long long K, bool same, int max_split, size_t cap) {
   if (M < 1 || N < 1 || K < 1 || M >= (1LL << 31) || N >= (1LL << 31) || K >= (1LL << 31) - TK) return 0;
-  if (cap > kWsCap) cap = kWsCap;
-  if (max_split <= 1 && !fits(M, K, cap)) return 0;
+  cap = std::min(cap, kWsCap);
+  if (max_split <= 1 && !fits(K, cap)) return 0;
   Plan p;
   return make_plan(M, N, K, same, max_split, cap, &p) ? p.bytes : 0;
 }
@@ -721,11 +730,13 @@ double f64_tc_column_bytes(long long M, long long K) { return column_bytes(M, K)
 // negative: an error
 int launch_gemm_nt_f64_tc(const double* A, long long lda, const double* B, long long ldb, double* C, long long ldc,
                           long long split_stride, int M, int N, long long K, int max_split, int upper_only, void* ws,
-                          size_t ws_bytes, int* err_flag, cudaStream_t s) {
+                          size_t ws_bytes, int* err_flag, cudaStream_t s, size_t cap) {
   const bool same = A == B && lda == ldb && M == N;
   Plan pl;
-  if (!ws || !tc_gemm_ready() || !smem_attr_set() || !make_plan(M, N, K, same, max_split, ws_bytes, &pl)) return 0;
-  if (upper_only && pl.np < N) return 0;
+  if (!ws || !tc_gemm_ready() || !smem_attr_set() ||
+      !make_plan(M, N, K, same, max_split, std::min(cap, kWsCap), &pl) || pl.bytes > ws_bytes)
+    return 0;
+  if (upper_only && (pl.np < N || pl.mp < M)) return 0;
   int used = 0;
   for (int p = 0; p < pl.pieces; ++p) {
     const long long k0 = p * pl.kp, Kp = std::min(pl.kp, K - k0);
@@ -743,71 +754,77 @@ int launch_gemm_nt_f64_tc(const double* A, long long lda, const double* B, long 
       w += row_bytes(rows);
       return d;
     };
-    const SliceDesc a = operand(A, lda, M), b0 = pl.shared ? a : operand(B, ldb, pl.np);
+    const SliceDesc a0 = operand(A, lda, pl.mp), b0 = pl.shared ? a0 : operand(B, ldb, pl.np);
     float* sums = (float*)w;
-    for (int n0 = 0; n0 < N; n0 += pl.np) {
-      const int nc = std::min(pl.np, N - n0);
-      SliceDesc b = b0, sa = a;
-      if (!pl.shared) {
-        b.x = B + (long long)n0 * ldb + k0;
-        b.rows = nc;
-        b.e = (int*)(b.q + nc);
-      }
-      SliceDesc sb = b;
-      if (pl.shared) sb.rows = 0;
-      if (n0 > 0) sa.rows = 0;   // the planes of A are there
-      if (launch_slices(sa, sb, Kp, s) != 0) return -1;
-      CUtensorMap ma, mb;
-      if (make_piece_map(&ma, a.v, M, kpad, PLANES, TM, TK, false, PLANES) ||
-          make_piece_map(&mb, b.v, nc, kpad, PLANES, TN, TK, false, PLANES))
-        return -1;
-      TcItems it;
-      it.M = M;
-      it.N = nc;
-      it.mt = (M + TM - 1) / TM;
-      it.nt = (nc + TN - 1) / TN;
-      it.upper = upper_only;
-      it.ntiles = it.mt * it.nt;
-      if (upper_only) {
-        it.ntiles = 0;
-        for (int t = 0; t < it.mt; ++t) it.ntiles += it.nt - t * TM / TN;
-      }
-      it.slabs = kpad / TK;
-      const int chunks = (it.slabs + CHUNK - 1) / CHUNK;
-      // splits: the rounds of the items over the SMs times an item's chunks, the epilogue as two more
-      const long long sms = sm_count();
-      long long best = -1;
-      int ns_best = 1;
-      for (int ns = 1; ns <= std::max(1, std::min(pl.nsplit, chunks)); ++ns) {
-        const int cps = (chunks + ns - 1) / ns;
-        if (cps > kMostChunks) continue;
-        const int real = (chunks + cps - 1) / cps;
-        const long long cost = ((long long)it.ntiles * real + sms - 1) / sms * (cps + 2);
-        if (best < 0 || cost < best) {
-          best = cost;
-          ns_best = real;
+    for (int m0 = 0; m0 < M; m0 += pl.mp)
+      for (int n0 = 0; n0 < N; n0 += pl.np) {
+        const int mc = std::min(pl.mp, M - m0), nc = std::min(pl.np, N - n0);
+        SliceDesc a = a0, b = b0;
+        a.x += (long long)m0 * lda;
+        a.rows = mc;
+        a.e = (int*)(a.q + mc);
+        if (pl.shared) {
+          b = a;
+        } else {
+          b.x += (long long)n0 * ldb;
+          b.rows = nc;
+          b.e = (int*)(b.q + nc);
         }
-      }
-      const int cps = (chunks + ns_best - 1) / ns_best;
-      it.nsplit = (chunks + cps - 1) / cps;
-      it.per = cps * CHUNK;
-      const long long items = (long long)it.ntiles * it.nsplit;
-      double* Cp = C + n0 + (long long)used * split_stride;
-      f64_tc_kernel<<<(unsigned)std::min(items, sms), NTHREADS, SMEM_BYTES, s>>>(ma, mb, a.e, b.e, Cp, ldc, split_stride,
-                                                                                 sums, it, err_flag);
-      ++g_launches;
-      if (it.nsplit > 1) {
-        const long long plane = (long long)M * nc;
-        f64_sum_kernel<<<(unsigned)std::min((plane + 255) / 256, 8 * sms), 256, 0, s>>>(sums, plane, it.nsplit);
+        SliceDesc sa = a, sb = b;
+        if (n0 > 0) sa.rows = 0;   // the planes of A are there
+        if (pl.shared || (m0 > 0 && pl.np >= N)) sb.rows = 0;
+        if (launch_slices(sa, sb, Kp, s) != 0) return -1;
+        CUtensorMap ma, mb;
+        if (make_piece_map(&ma, a.v, mc, kpad, PLANES, TM, TK, false, PLANES) ||
+            make_piece_map(&mb, b.v, nc, kpad, PLANES, TN, TK, false, PLANES))
+          return -1;
+        TcItems it;
+        it.M = mc;
+        it.N = nc;
+        it.mt = (mc + TM - 1) / TM;
+        it.nt = (nc + TN - 1) / TN;
+        it.upper = upper_only;
+        it.ntiles = it.mt * it.nt;
+        if (upper_only) {
+          it.ntiles = 0;
+          for (int t = 0; t < it.mt; ++t) it.ntiles += it.nt - t * TM / TN;
+        }
+        it.slabs = kpad / TK;
+        const int chunks = (it.slabs + CHUNK - 1) / CHUNK;
+        // splits: the rounds of the items over the SMs times an item's chunks, the epilogue as two more
+        const long long sms = sm_count();
+        long long best = -1;
+        int ns_best = 1;
+        for (int ns = 1; ns <= std::max(1, std::min(pl.nsplit, chunks)); ++ns) {
+          const int cps = (chunks + ns - 1) / ns;
+          if (cps > kMostChunks) continue;
+          const int real = (chunks + cps - 1) / cps;
+          const long long cost = ((long long)it.ntiles * real + sms - 1) / sms * (cps + 2);
+          if (best < 0 || cost < best) {
+            best = cost;
+            ns_best = real;
+          }
+        }
+        const int cps = (chunks + ns_best - 1) / ns_best;
+        it.nsplit = (chunks + cps - 1) / cps;
+        it.per = cps * CHUNK;
+        const long long items = (long long)it.ntiles * it.nsplit;
+        double* Cp = C + (long long)m0 * ldc + n0 + (long long)used * split_stride;
+        f64_tc_kernel<<<(unsigned)std::min(items, sms), NTHREADS, SMEM_BYTES, s>>>(ma, mb, a.e, b.e, Cp, ldc,
+                                                                                   split_stride, sums, it, err_flag);
         ++g_launches;
+        if (it.nsplit > 1) {
+          const long long plane = (long long)mc * nc;
+          f64_sum_kernel<<<(unsigned)std::min((plane + 255) / 256, 8 * sms), 256, 0, s>>>(sums, plane, it.nsplit);
+          ++g_launches;
+        }
+        const int ft = (mc + 63) / 64;
+        const dim3 grid = upper_only ? dim3(ft * (ft + 1) / 2, 1, it.nsplit) : dim3((nc + 63) / 64, ft, it.nsplit);
+        f64_fix_kernel<<<grid, 256, 0, s>>>(a.x, lda, b.x, ldb, Cp, ldc, split_stride, mc, nc, Kp,
+                                            (long long)it.per * TK, sums, a.q, a.e, b.q, b.e, upper_only);
+        ++g_launches;
+        if (m0 + mc >= M && n0 + nc >= N) used += it.nsplit;
       }
-      const int ft = (M + 63) / 64;
-      const dim3 grid = upper_only ? dim3(ft * (ft + 1) / 2, 1, it.nsplit) : dim3((nc + 63) / 64, ft, it.nsplit);
-      f64_fix_kernel<<<grid, 256, 0, s>>>(a.x, lda, b.x, ldb, Cp, ldc, split_stride, M, nc, Kp,
-                                          (long long)it.per * TK, sums, a.q, a.e, b.q, b.e, upper_only);
-      ++g_launches;
-      if (n0 + nc >= N) used += it.nsplit;
-    }
   }
   if (cudaPeekAtLastError() != cudaSuccess) {
     fprintf(stderr, "hotrg: FP64 product on the tensor cores: launch error (M %d, N %d, K %lld)\n", M, N, K);

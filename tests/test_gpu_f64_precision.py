@@ -115,6 +115,25 @@ def test_a_sum_is_not_short_of_an_accumulator(pkg):
     assert np.all(err <= 2.0 ** -53 * np.abs(got) + 2.0 ** -56)
 
 
+# one pass; several passes of B's rows with a ragged last one (K up to 2048 and above); A == B; A alone beyond
+# the array (passes of its rows too, whole tiles or parts of one)
+@pytest.mark.parametrize("m,n,k,same", [(200, 700, 160, False), (600, 1800, 1800, False), (300, 1900, 3000, False),
+                                        (600, 600, 1024, True), (1700, 1700, 1700, True), (2600, 96, 2100, False),
+                                        (31, 5000, 400, False), (72, 96, 32768, False), (48, 64, 120000, False)])
+def test_caller_owned_memory_gives_the_same_bits(pkg, m, n, k, same):
+    import torch
+
+    gen = torch.Generator(device="cuda").manual_seed(m + n + k)
+    fall = torch.exp(-1.5 * torch.rand(k, generator=gen, device="cuda", dtype=torch.float64))
+    a = torch.randn(m, k, generator=gen, device="cuda", dtype=torch.float64) * fall
+    b = a if same else torch.randn(n, k, generator=gen, device="cuda", dtype=torch.float64) * fall
+    c = torch.full((m, n), float("nan"), dtype=torch.float64, device="cuda")
+    pkg.hotrg_gemm_nt_noalloc(pkg.PREC_FP64, a, b, c, torch.cuda.current_stream().cuda_stream)
+    ref = a @ b.T
+    assert ((c - ref).abs() / (a.abs() @ b.abs().T)).max().item() <= 2 * k * 2.0 ** -53
+    np.testing.assert_array_equal(c.cpu().numpy(), pkg.hotrg_gemm_nt(pkg.PREC_FP64, a.cpu().numpy(), b.cpu().numpy()))
+
+
 def test_grams_in_several_passes_along_k(pkg):
     """400 rows of 160,000 terms: the digits do not fit the workspace at once."""
     import torch
