@@ -10,11 +10,11 @@ inline bool f64_digits_pay(double M, double N, double K, bool upper_only) {
   return M >= 32.0 && N >= 16.0 && K >= 32.0 && M * N * K * (upper_only ? 0.5 : 1.0) >= 16777216.0;
 }
 
-// A Gram over less than 1024 terms (2D runs: K = chi_c chi_j) stays on the pipe: at a degenerate cut the kept vector
-// follows the rounding of the Gram (ordered 2D phase, chi = 24, step 11: a pair 2.8e-15 lambda_1 apart), and such runs
-// go on as they did; it would save 0.1 ms of a Gram of 576 rows.
+// Grams of 2D steps, K = chi_c chi_j <= 32 x 32 terms, stay on the pipe: at a degenerate cut the kept vector follows
+// the rounding of the Gram (ordered 2D phase, chi = 24, step 11: a pair 2.8e-15 lambda_1 apart), and such runs go on
+// as they did; digits would save 0.1 ms of a Gram of 576 rows.
 inline bool f64_gram_digits_pay(double M, double K, bool upper_only) {
-  return K >= 1024.0 && f64_digits_pay(M, M, K, upper_only);
+  return K > 1024.0 && f64_digits_pay(M, M, K, upper_only);
 }
 
 }  // namespace hotrg

@@ -60,3 +60,14 @@ def test_classes_of_turned_vectors(tmp_path):
       }
       CHECK(!turn_ends_class(5, false, 5, false, 1.0) && !turn_ends_class(0, false, 0, false, 1.0));
     """)
+
+
+def test_grams_of_2d_steps_stay_on_the_fp64_pipe(tmp_path):
+    """Up to the largest bonds (32 x 32 terms): the kept vectors of a degenerate cut follow their rounding."""
+    _run(tmp_path, ["f64_rule.h"], """
+      for (int c = 2; c <= 32; ++c)
+        for (int j = 2; j <= 32; ++j) CHECK(!f64_gram_digits_pay(c * j, c * j, true));
+      CHECK(f64_gram_digits_pay(256, 4096, true) && !f64_gram_digits_pay(24, 1 << 20, true));
+      CHECK(!f64_digits_pay(256, 256, 255, false) && f64_digits_pay(256, 256, 256, false));
+      CHECK(f64_digits_pay(256, 256, 512, true) && !f64_digits_pay(256, 256, 511, true));
+    """)
