@@ -1161,49 +1161,87 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
         eig_nb[j][0] = chij[j] * chij[j];
         eig_nb[j][1] = 0;
       }
-    int ld = 1, nblk = 0, na[4 * kMaxD], keep[4 * kMaxD], bidx[kMaxD][2][2];
+    // two batches: the small matrices and the others, each with its own leading dimension
+    struct Batch {
+      int ld = 1, n = 0, na[4 * kMaxD], keep[4 * kMaxD];
+      double *A = nullptr, *V = nullptr, *lam = nullptr;
+      int *swp = nullptr, *cls = nullptr;
+    } bat[2];
+    struct Place {
+      int batch = 0, i = -1;
+    } at[kMaxD][2][2];
     for (int j = 1; j < d; ++j)
       for (int k = 0; k < 2; ++k)
         for (int b = 0; b < 2; ++b) {
-          bidx[j][k][b] = -1;
-          if (eig_nb[j][b] == 0) continue;
-          bidx[j][k][b] = nblk;
-          keep[nblk] = nnew[j];
-          na[nblk++] = eig_nb[j][b];
-          ld = std::max(ld, eig_nb[j][b]);
+          const int n = eig_nb[j][b];
+          if (n == 0) continue;
+          Place& p = at[j][k][b];
+          p.batch = n <= kEigSmall ? 0 : 1;
+          Batch& t = bat[p.batch];
+          p.i = t.n;
+          t.keep[t.n] = nnew[j];
+          t.na[t.n++] = n;
+          t.ld = std::max(t.ld, n);
         }
-    const long long bb = (long long)ld * ld;
-    CHECK_ALLOC(dev_alloc(c, c->Eb, (sizeof(double) * (2 * bb + ld) + sizeof(int) * 2 * ld) * nblk));
-    CHECK_ALLOC(dev_alloc(c, c->Ew, eig_workspace_bytes(ld, nblk)));
-    double* Ab = (double*)c->Eb.p;
-    double* Vb = Ab + bb * nblk;
-    double* lb = Vb + bb * nblk;
-    int* swp = (int*)(lb + (long long)ld * nblk);
-    int* cb = swp + (long long)ld * nblk;
+    auto batch_bytes = [](const Batch& t) {
+      return (sizeof(double) * (2 * (size_t)t.ld + 1) + sizeof(int) * 2) * t.ld * t.n;
+    };
+    CHECK_ALLOC(dev_alloc(c, c->Eb, batch_bytes(bat[0]) + batch_bytes(bat[1])));
+    size_t work = 0;   // the batches run one after the other
+    for (const Batch& t : bat)
+      if (t.n > 0) work = std::max(work, eig_workspace_bytes(t.ld, t.n));
+    CHECK_ALLOC(dev_alloc(c, c->Ew, work));
+    char* ep = (char*)c->Eb.p;
+    for (Batch& t : bat) {   // the doubles of both first: all stay aligned
+      const size_t nn = (size_t)t.ld * t.ld * t.n, nv = (size_t)t.ld * t.n;
+      t.A = (double*)ep;
+      t.V = t.A + nn;
+      t.lam = t.V + nn;
+      ep = (char*)(t.lam + nv);
+    }
+    for (Batch& t : bat) {
+      t.swp = (int*)ep;
+      t.cls = t.swp + (size_t)t.ld * t.n;
+      ep = (char*)(t.cls + (size_t)t.ld * t.n);
+    }
     int* swb = (int*)c->sweeps.p + 2 * kMaxD;
     for (int j = 1; j < d; ++j)
       for (int k = 0; k < 2; ++k)
-        for (int b = 0; b < 2; ++b)
-          if (bidx[j][k][b] >= 0)
-            launch_z2_gather_sym((const double*)c->Amat.p + mat_elem_off[2 * j + k], chij[j],
-                                 z2g ? zi + gz_eig[j] + (b == 0 ? 0 : eig_nb[j][0]) : nullptr,
-                                 z2g ? zi + gz_eig[j] + 2 * chij[j] * chij[j] : nullptr, eig_nb[j][b], ld,
-                                 Ab + bb * bidx[j][k][b], swp + ld * bidx[j][k][b], s);
-    if (launch_eig(Ab, ld, nblk, na, keep, swp, c->Ew.p, Vb, lb, cb, swb, (DevState*)c->state.p, s) != 0)
-      return launch_failed(c, "eigen-solver", ld, nblk, 0);
+        for (int b = 0; b < 2; ++b) {
+          const Place& p = at[j][k][b];
+          if (p.i < 0) continue;
+          Batch& t = bat[p.batch];
+          launch_z2_gather_sym((const double*)c->Amat.p + mat_elem_off[2 * j + k], chij[j],
+                               z2g ? zi + gz_eig[j] + (b == 0 ? 0 : eig_nb[j][0]) : nullptr,
+                               z2g ? zi + gz_eig[j] + 2 * chij[j] * chij[j] : nullptr, eig_nb[j][b], t.ld,
+                               t.A + (long long)t.ld * t.ld * p.i, t.swp + (long long)t.ld * p.i, s);
+        }
+    int first = 0;
+    for (Batch& t : bat) {
+      if (t.n > 0 && launch_eig(t.A, t.ld, t.n, t.na, t.keep, t.swp, c->Ew.p, t.V, t.lam, t.cls, swb + first,
+                                (DevState*)c->state.p, s) != 0)
+        return launch_failed(c, "eigen-solver", t.ld, t.n, 0);
+      first += t.n;
+    }
     SweepMerge sm;
     sm.n = 2 * (d - 1);
     for (int j = 1; j < d; ++j) {
       const int n = chij[j] * chij[j];
       const int* eb = z2g ? zi + gz_eig[j] + n : nullptr;
       for (int k = 0; k < 2; ++k) {
-        const int mat = 2 * (j - 1) + k, i0 = bidx[j][k][0], i1 = bidx[j][k][1];
-        sm.a[mat] = i0;
-        sm.b[mat] = i1;
-        launch_z2_scatter_eig(i0 >= 0 ? Vb + bb * i0 : nullptr, i1 >= 0 ? Vb + bb * i1 : nullptr,
-                              i0 >= 0 ? lb + (long long)ld * i0 : nullptr, i1 >= 0 ? lb + (long long)ld * i1 : nullptr,
-                              i0 >= 0 ? cb + (long long)ld * i0 : nullptr, i1 >= 0 ? cb + (long long)ld * i1 : nullptr,
-                              ld, eb, eb ? eb + n : nullptr, n, (double*)c->V.p + mat_elem_off[2 * j + k],
+        const int mat = 2 * (j - 1) + k;
+        EigBlock blk[2];
+        int where[2];
+        for (int b = 0; b < 2; ++b) {
+          const Place& p = at[j][k][b];
+          where[b] = p.i < 0 ? -1 : p.i + (p.batch ? bat[0].n : 0);
+          if (p.i < 0) continue;
+          const Batch& t = bat[p.batch];
+          blk[b] = {t.V + (long long)t.ld * t.ld * p.i, t.lam + (long long)t.ld * p.i, t.cls + (long long)t.ld * p.i, t.ld};
+        }
+        sm.a[mat] = where[0];
+        sm.b[mat] = where[1];
+        launch_z2_scatter_eig(blk[0], blk[1], eb, eb ? eb + n : nullptr, n, (double*)c->V.p + mat_elem_off[2 * j + k],
                               (double*)c->lraw.p + lraw_off[j] + (long long)k * n, craw + lraw_off[j] + (long long)k * n,
                               s);
       }

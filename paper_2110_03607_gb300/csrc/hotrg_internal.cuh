@@ -228,6 +228,9 @@ void launch_assemble_a(const double* s_hat, const double* s_chk, int chi_j, int 
 // keep[]: the leading eigenvectors that may be kept; swp [nmat][n]: the partner of every index
 // under the exchange of hat and check; cls [nmat][n]: vectors that are even and odd under it have
 // opposite nonzero values
+// One batch's matrices all go the same way, by n: up to kEigSmall rows Jacobi sweeps, above reduction and divide
+// and conquer.
+constexpr int kEigSmall = 20;
 size_t eig_workspace_bytes(int n, int nmat);
 int launch_eig(const double* A, int n, int nmat, const int* na, const int* keep, const int* swp, void* work, double* V,
                double* lam, int* cls, int* iters, DevState* st, cudaStream_t s);
@@ -327,8 +330,13 @@ struct SweepMerge {
 };
 void launch_z2_gather_sym(const double* A, int chi, const int* rows, const int* pos, int nb, int npad, double* Ab,
                           int* swp, cudaStream_t s);
-void launch_z2_scatter_eig(const double* m0, const double* m1, const double* l0, const double* l1,
-                           const int* c0, const int* c1, int ld, const int* blk, const int* pos, int n, double* M,
+struct EigBlock {
+  const double* v = nullptr;   // eigenvectors, a row each, of leading dimension ld
+  const double* lam = nullptr;
+  const int* cls = nullptr;
+  int ld = 0;
+};
+void launch_z2_scatter_eig(const EigBlock& b0, const EigBlock& b1, const int* blk, const int* pos, int n, double* M,
                            double* lam, int* cls, cudaStream_t s);
 void launch_z2_merge_sweeps(const int* src, const SweepMerge& m, int* dst, cudaStream_t s);
 void launch_z2_gather_rc(const double* T, const long long* roff, int m, const long long* koff,

@@ -27,7 +27,8 @@
 //    rounding, elements between components count as zero, and a reflector never mixes two
 //    components.  Exact zeros between parities stay exact.
 //
-// Up to kJacobiMax rows the one-sided Jacobi sweeps stay (jacobi_onesided_kernel): they cost no
+// A batch of up to kJacobiMax rows (the caller gives the matrices up to there and those above as
+// two batches) goes through one-sided Jacobi sweeps (jacobi_onesided_kernel): they cost no
 // more there (n = 16: 0.2 ms), and they move nearly degenerate pairs, which the first steps of a
 // split run have at the 1e-8 of its rounding, less than the reduction's few eps.
 #include <cooperative_groups.h>
@@ -46,7 +47,7 @@ namespace {
 constexpr double kEps = 2.220446049250313e-16;
 constexpr int kRb = 16;          // reflectors per block of the back-transformation
 constexpr int kLeaf = 9;         // largest tridiagonal leaf solved by implicit QR in one warp
-constexpr int kJacobiMax = 20;   // largest order left to the Jacobi sweeps
+constexpr int kJacobiMax = kEigSmall;   // largest order left to the Jacobi sweeps
 constexpr int kPolish = 96;      // columns of a group of close eigenvalues
 constexpr int kEigMaxN = 1024;   // chi_j^2 <= 32^2
 constexpr int kTriThreads = 256;
@@ -1374,8 +1375,11 @@ __global__ void __launch_bounds__(256) eig_back_kernel(EigWs ws, const double* _
 // exceeds (4 n eps)^2 times the largest squared column norm at the start: the near-null columns
 // (rounding noise of order n eps lambda_1) are rotated too, but do not keep the sweeps going.
 // ---------------------------------------------------------------------------
+struct JacobiOrders {
+  int n[kEigMaxMat];
+};
 __global__ void __launch_bounds__(256) jacobi_onesided_kernel(const double* __restrict__ A, double* W, double* V,
-                                                              double* lam, int n, int nmat, int max_sweeps,
+                                                              double* lam, int n, JacobiOrders na, int nmat, int max_sweeps,
                                                               int* counters, unsigned long long* colmax,
                                                               int* sweeps_out, DevState* st) {
   cg::grid_group grid = cg::this_grid();
@@ -1391,7 +1395,7 @@ __global__ void __launch_bounds__(256) jacobi_onesided_kernel(const double* __re
   if (gtid < nmat) colmax[gtid] = 0ull;
   grid.sync();
 
-  const int mp = n + (n & 1), npairs = mp / 2, rounds = mp - 1;
+  const int npairs = (n + 1) / 2, rounds = 2 * npairs - 1;
   const int lane = threadIdx.x & 31;
   // consecutive tasks go to different blocks (SMs), spreading the FP64 work
   const int gw = (int)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
@@ -1411,18 +1415,19 @@ __global__ void __launch_bounds__(256) jacobi_onesided_kernel(const double* __re
   // way, but a column at rounding level carries noise of order eps times the large column it was
   // last rotated against, and the relative test would rotate that pair forever.  Columns with a
   // squared norm below 1e-280 are left alone: tol max(a, b) underflows to 0 there.
-  const double tol = 4.0 * (double)n * kEps;
-
   int sweep = 1;
+  unsigned settled = 0u;   // matrices that have had their last sweep
   bool converged = false;
   for (; sweep <= max_sweeps; ++sweep) {
-    int* cur = counters + (sweep % 3) * nmat;
+    int *cur = counters + (sweep % 3) * nmat, *prev = counters + ((sweep + 2) % 3) * nmat;
     if (blockIdx.x == 0 && (int)threadIdx.x < nmat) counters[((sweep + 1) % 3) * nmat + threadIdx.x] = 0;
     for (int r = 0; r < rounds; ++r) {
       for (int task = gw; task < ntasks; task += nw) {
-        const int mat = task / npairs, k = task % npairs;
+        // a matrix takes the turns of its own order, and none after its last sweep, whatever its batch
+        const int mat = task / npairs, k = task % npairs, nm = na.n[mat], mp = nm + (nm & 1);
+        if (k >= mp / 2 || r >= mp - 1 || (sweep > 1 && __ldcg(prev + mat) == 0)) continue;
         int p = rr_slot(k, r, mp), q = rr_slot(mp - 1 - k, r, mp);
-        if (p >= n || q >= n) continue;
+        if (p >= nm || q >= nm) continue;
         if (p > q) { const int t = p; p = q; q = t; }
         const bool in = lane < n;
         const int ip = mat * nn + p * n + lane, iq = mat * nn + q * n + lane;
@@ -1431,6 +1436,7 @@ __global__ void __launch_bounds__(256) jacobi_onesided_kernel(const double* __re
         const double vx = in ? __ldcg(V + ip) : 0.0, vy = in ? __ldcg(V + iq) : 0.0;
         const double a = warp_sum(x * x), b = warp_sum(y * y), g = warp_sum(x * y);
         const double big = fmax(a, b);
+        const double tol = 4.0 * (double)nm * kEps;
         if (!((g != 0.0) && big > 1e-280 && (fabs(g) > tol * big))) continue;
         const bool counts = big > tol * tol * __longlong_as_double((long long)__ldcg(colmax + mat));
         const double zeta = (b - a) / (2.0 * g);
@@ -1448,7 +1454,14 @@ __global__ void __launch_bounds__(256) jacobi_onesided_kernel(const double* __re
       grid.sync();
     }
     int total = 0;
-    for (int m = 0; m < nmat; ++m) total += __ldcg(cur + m);
+    for (int m = 0; m < nmat; ++m) {
+      const int rotated = __ldcg(cur + m);
+      if (gtid == 0 && !(settled >> m & 1u)) {
+        sweeps_out[m] = sweep;
+        if (rotated == 0) settled |= 1u << m;
+      }
+      total += rotated;
+    }
     if (total == 0) {
       converged = true;
       break;
@@ -1459,10 +1472,7 @@ __global__ void __launch_bounds__(256) jacobi_onesided_kernel(const double* __re
     const double a = warp_sum(x * x);
     if (lane == 0) lam[task] = sqrt(a);
   }
-  if (gtid == 0) {
-    for (int m = 0; m < nmat; ++m) sweeps_out[m] = sweep;
-    if (!converged && st->status == 0) st->status = HOTRG_ENOTCONV;
-  }
+  if (gtid == 0 && !converged && st->status == 0) st->status = HOTRG_ENOTCONV;
 }
 
 // ---------------------------------------------------------------------------
@@ -1818,7 +1828,9 @@ int launch_eig(const double* A, int n, int nmat, const int* na, const int* keep,
     int* counters = (int*)w.ctl;
     unsigned long long* colmax = (unsigned long long*)w.mc;
     const int blocks = std::max(1, std::min(nmat * npairs, sm_count()));
-    void* args[] = {&A, &W, &V, &lam, &n, &nmat, &max_sweeps, &counters, &colmax, &iters, &st};
+    JacobiOrders orders;
+    for (int m = 0; m < kEigMaxMat; ++m) orders.n[m] = w.na[m];
+    void* args[] = {&A, &W, &V, &lam, &n, &orders, &nmat, &max_sweeps, &counters, &colmax, &iters, &st};
     const cudaError_t e =
         cudaLaunchCooperativeKernel((void*)jacobi_onesided_kernel, dim3(blocks), dim3(256), args, 0, s);
     ++g_launches;

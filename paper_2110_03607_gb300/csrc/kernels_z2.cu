@@ -400,42 +400,37 @@ void launch_z2_gather_sym(const double* A, int chi, const int* rows, const int* 
   ++g_launches;
 }
 
-// Column-major n x n M from the blocks (leading dimension ld): M[r + c n] =
-// M_b[pos[r] + pos[c] ld] if rows r and c are both of parity b, else 0 (column c of M is
-// column pos[c] of block blk[c]; the padding columns of the blocks are dropped), and the
-// eigenvalue and the class of every column.  No blk: one block, in order.
-__global__ void z2_scatter_eig_kernel(const double* __restrict__ m0, const double* __restrict__ m1,
-                                      const double* __restrict__ l0, const double* __restrict__ l1,
-                                      const int* __restrict__ c0, const int* __restrict__ c1, int ld,
-                                      const int* __restrict__ blk, const int* __restrict__ pos, int n,
-                                      double* __restrict__ M, double* __restrict__ lam, int* __restrict__ cls) {
+// Column-major n x n M from the blocks: M[r + c n] = v_b[pos[r] + pos[c] ld_b] if rows r and c are
+// both of parity b, else 0 (column c of M is column pos[c] of block blk[c]; the padding columns of the
+// blocks are dropped), and the eigenvalue and the class of every column.  No blk: one block, in order.
+__global__ void z2_scatter_eig_kernel(EigBlock b0, EigBlock b1, const int* __restrict__ blk,
+                                      const int* __restrict__ pos, int n, double* __restrict__ M,
+                                      double* __restrict__ lam, int* __restrict__ cls) {
   const int total = n * n;
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < total; e += gridDim.x * blockDim.x) {
     const int cidx = e / n, r = e - cidx * n;
     if (!blk) {
-      M[e] = m0[r + (long long)cidx * ld];
+      M[e] = b0.v[r + (long long)cidx * b0.ld];
       if (e < n) {
-        lam[e] = l0[e];
-        cls[e] = c0[e];
+        lam[e] = b0.lam[e];
+        cls[e] = b0.cls[e];
       }
       continue;
     }
     const int b = blk[r];
     double v = 0.0;
-    if (b == blk[cidx]) v = (b == 0 ? m0 : m1)[pos[r] + (long long)pos[cidx] * ld];
+    if (b == blk[cidx]) v = (b == 0 ? b0.v : b1.v)[pos[r] + (long long)pos[cidx] * (b == 0 ? b0.ld : b1.ld)];
     M[e] = v;
     if (e < n) {
-      lam[e] = (blk[e] == 0 ? l0 : l1)[pos[e]];
-      cls[e] = (blk[e] == 0 ? c0 : c1)[pos[e]];
+      lam[e] = (blk[e] == 0 ? b0.lam : b1.lam)[pos[e]];
+      cls[e] = (blk[e] == 0 ? b0.cls : b1.cls)[pos[e]];
     }
   }
 }
 
-void launch_z2_scatter_eig(const double* m0, const double* m1, const double* l0, const double* l1,
-                           const int* c0, const int* c1, int ld, const int* blk, const int* pos, int n, double* M,
+void launch_z2_scatter_eig(const EigBlock& b0, const EigBlock& b1, const int* blk, const int* pos, int n, double* M,
                            double* lam, int* cls, cudaStream_t s) {
-  z2_scatter_eig_kernel<<<grid_for((long long)n * n), 256, 0, s>>>(m0, m1, l0, l1, c0, c1, ld, blk, pos, n, M, lam,
-                                                                   cls);
+  z2_scatter_eig_kernel<<<grid_for((long long)n * n), 256, 0, s>>>(b0, b1, blk, pos, n, M, lam, cls);
   ++g_launches;
 }
 
