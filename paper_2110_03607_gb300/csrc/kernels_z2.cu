@@ -193,19 +193,22 @@ void launch_z2_columns(int* map, long long rx, long long ry, int nx, int P, int 
   ++g_launches;
 }
 
-// Maps of the dense form as one block: list position o holds index (o % rest) last + o / rest (rest = n /
-// last: the fastest index goes slowest); blk and pos per index, list (twice: kcat, and kpad padded with
+// Maps of the dense form as one block: list position o holds index (o % rest) last + last - 1 - o / rest (rest = n /
+// last: the fastest index goes slowest, and down); blk and pos per index, list (twice: kcat, and kpad padded with
 // -1) per position.  last = 1 and no lists: the identity.
+// Down, because the elements of a coarse-grained tensor fall off along every leg: the product's FP32 sums take the
+// small terms first.  3D chi = 12 with a field, six tensors: error of the new tensor against 64 bits (2-norm) 2.2e-7,
+// with the index going up 3.2e-7, in the tensor's own order 3.3e-7.
 __global__ void z2_one_block_kernel(int* blk, int* pos, int* kcat, int* kpad, int n, int np, int last) {
   const int rest = n / last;
   for (int o = blockIdx.x * blockDim.x + threadIdx.x; o < n || o < np; o += gridDim.x * blockDim.x) {
     if (o < n) {
-      const int r = (o % rest) * last + o / rest;
+      const int r = (o % rest) * last + last - 1 - o / rest;
       blk[r] = 0;
       pos[r] = o;
       if (kcat) kcat[o] = r;
     }
-    if (o < np) kpad[o] = o < n ? (o % rest) * last + o / rest : -1;
+    if (o < np) kpad[o] = o < n ? (o % rest) * last + last - 1 - o / rest : -1;
   }
 }
 
