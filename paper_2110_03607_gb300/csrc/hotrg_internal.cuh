@@ -223,7 +223,7 @@ void launch_assemble_a(const double* s_hat, const double* s_chk, int chi_j, int 
                        double* A, cudaStream_t s);
 
 // ---- kernels_eig.cu
-// Eigen-decomposition of nmat (<= 16) symmetric matrices of orders na[] <= n <= 1024, leading
+// Eigen-decomposition of nmat (<= 16) symmetric matrices A (overwritten) of orders na[] <= n <= 1024, leading
 // dimension n: eigenvectors in the rows of V, eigenvalues in lam, an iteration count per matrix;
 // keep[]: the leading eigenvectors that may be kept; swp [nmat][n]: the partner of every index
 // under the exchange of hat and check; cls [nmat][n]: vectors that are even and odd under it have
@@ -232,7 +232,7 @@ void launch_assemble_a(const double* s_hat, const double* s_chk, int chi_j, int 
 // and conquer.
 constexpr int kEigSmall = 20;
 size_t eig_workspace_bytes(int n, int nmat);
-int launch_eig(const double* A, int n, int nmat, const int* na, const int* keep, const int* swp, void* work, double* V,
+int launch_eig(double* A, int n, int nmat, const int* na, const int* keep, const int* swp, void* work, double* V,
                double* lam, int* cls, int* iters, DevState* st, cudaStream_t s);
 void launch_gemm_nn_f64(const double* A, long long lda, const double* B, long long ldb, double* C,
                         long long ldc, int M, int N, int K, int batch, long long bsa,

@@ -57,7 +57,9 @@ constexpr int kVecThreads = 128;   // of them, those with the work of order n: a
 struct EigCtl {
   double unscale;    // power of two: max |A| / unscale in [0.5, 1)
   int bad;           // a non-finite element: eigenvalues and vectors are set to NaN
-  int mixed;         // a row is coupled to another label: the components need more rounds
+  int mixed;         // a row is coupled to another label: the components need more rounds; in the correction:
+                     // whether the pass has angles (1), one above 2^-24 (2) or 2^-12 (3) among them
+  int settled;       // a pass of the correction found no angle above 2^-24: it left none above 2^-48
   int iters;         // most QR iterations an eigenvalue of a leaf took
   unsigned long long amax;   // bits of max |A|
   double top;        // max |A| / unscale
@@ -91,6 +93,8 @@ struct EigWs {
   double* val;       // [nmat][n] new eigenvalues: roots, then deflated
   double* rc;        // [nmat][n] rotation cosines
   double* rs;        // [nmat][n] sines
+  double* w2;        // [nmat][n][n] turned columns of the correction
+  double* w3;        // [nmat][n][n]
   double* ap;        // [nmat][n][n] A, scaled, in the basis of the exchange's combinations
   const int* swp;    // [nmat][n] partner of every index under the exchange
   int* perm;         // [nmat][n] component order
@@ -1479,22 +1483,34 @@ __global__ void __launch_bounds__(256) jacobi_onesided_kernel(const double* __re
 // The graded part.  Backward error of a few eps ||A|| turns vectors with eigenvalues lambda, mu by eps
 // lambda_1 / |lambda - mu|, far more than A's elements leave open where lambda and mu are small.  So
 // W = A V is formed and its columns are made orthogonal to 4 n eps (one-sided Jacobi's test): groups
-// of close eigenvalues by plane rotations, the others, whose angles are tiny, all at once.
+// of close eigenvalues by plane rotations, the others, whose angles are small, all at once by 1 + M + M^2 / 2 +
+// M^3 / 8 (M skew, its elements the angles: orthogonal to M^6 / 64), as far as the angles need it.  A kept
+// vector's angles against those far below it reach 8 eps lambda_1 / lambda, 2^-9 for the least lambda that the
+// selection tells from its neighbours, 1e-12 lambda_1; a pass leaves their products, so there are three.
 // ---------------------------------------------------------------------------
 // Vectors of opposite classes are left as they are (turn_forbidden); what else ends a class is noted in
 // `lost` by the polish alone, whose turns are ordered by barriers, and applied by the last pass.
 
-// out = X Y / unscale, or with the angles as X, out = Y + X Y where the matrix has any; 32 x 32
-// tiles, 2 x 2 per thread
-template <bool ANGLES>
-__global__ void __launch_bounds__(256) eig_nn_kernel(const double* __restrict__ X, const double* __restrict__ Y,
-                                                     EigWs ws, double* __restrict__ out) {
+// EIG_AV: out[0] = X Y[0] / unscale.  With the angles as X, for V (0) and W (1): EIG_FIRST: out = Y + X Y where the
+// matrix has any; EIG_SECOND: out = Z + X (Z - Y) / 2 with Z = Y + X Y where one is above 2^-24; EIG_THIRD: the same
+// with 1 / 4, Z of second and Y of first order, where one is above 2^-12.  32 x 32 tiles, 2 x 2 per thread.
+enum EigProduct { EIG_AV, EIG_FIRST, EIG_SECOND, EIG_THIRD };
+struct EigPair {
+  double* p[2];
+};
+template <EigProduct KIND>
+__global__ void __launch_bounds__(256) eig_nn_kernel(const double* __restrict__ X, EigPair Yp, EigPair Zp, EigWs ws,
+                                                     EigPair outp) {
   constexpr int BK = 16;
   __shared__ double As[BK][33], Bs[BK][33];
-  const int mat = blockIdx.z, n = ws.na[mat], ld = ws.n, c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
+  const int mat = KIND == EIG_AV ? blockIdx.z : blockIdx.z >> 1, which = KIND == EIG_AV ? 0 : blockIdx.z & 1;
+  const int n = ws.na[mat], ld = ws.n, c0 = blockIdx.x * 32, r0 = blockIdx.y * 32;
   if (c0 >= n || r0 >= n) return;
   const EigCtl ctl = ws.ctl[mat];
-  if (ctl.bad || (ANGLES && !ctl.mixed)) return;
+  if (ctl.bad || (KIND != EIG_AV && ctl.mixed < (int)KIND)) return;
+  const double* __restrict__ Y = Yp.p[which];
+  const double* __restrict__ Z = KIND >= EIG_SECOND ? Zp.p[which] : nullptr;
+  double* __restrict__ out = outp.p[which];
   const long long o = (long long)mat * ld * ld;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
@@ -1504,7 +1520,8 @@ __global__ void __launch_bounds__(256) eig_nn_kernel(const double* __restrict__ 
       const int r = r0 + (tid >> 4) + 16 * u, k = k0 + (tid & 15);
       As[tid & 15][(tid >> 4) + 16 * u] = (r < n && k < n) ? X[o + (long long)r * ld + k] : 0.0;
       const int kb = k0 + (tid >> 5) + 8 * u, c = c0 + (tid & 31);
-      Bs[(tid >> 5) + 8 * u][tid & 31] = (kb < n && c < n) ? Y[o + (long long)kb * ld + c] : 0.0;
+      const long long eb = o + (long long)kb * ld + c;
+      Bs[(tid >> 5) + 8 * u][tid & 31] = (kb < n && c < n) ? (KIND >= EIG_SECOND ? Z[eb] - Y[eb] : Y[eb]) : 0.0;
     }
     __syncthreads();
 #pragma unroll
@@ -1517,7 +1534,7 @@ __global__ void __launch_bounds__(256) eig_nn_kernel(const double* __restrict__ 
     }
     __syncthreads();
   }
-  const double sc = ANGLES ? 1.0 : 1.0 / ctl.unscale;   // a power of two
+  const double sc = KIND == EIG_AV ? 1.0 / ctl.unscale : 1.0;   // a power of two
 #pragma unroll
   for (int u = 0; u < 2; ++u)
 #pragma unroll
@@ -1525,18 +1542,22 @@ __global__ void __launch_bounds__(256) eig_nn_kernel(const double* __restrict__ 
       const int r = r0 + ty + 16 * u, c = c0 + tx + 16 * v;
       if (r < n && c < n) {
         const long long e = o + (long long)r * ld + c;
-        out[e] = ANGLES ? Y[e] + acc[u][v] : acc[u][v] * sc;
+        out[e] = KIND == EIG_AV ? acc[u][v] * sc : KIND == EIG_FIRST ? Y[e] + acc[u][v]
+                                                                          : fma(KIND == EIG_SECOND ? 0.5 : 0.25, acc[u][v], Z[e]);
       }
     }
 }
 
 // squared norms of W's columns (into dk); LAST: the eigenvalues, and no class where the polish ended it
 template <bool LAST>
-__global__ void __launch_bounds__(256) eig_norm_kernel(const double* __restrict__ W, EigWs ws, double* lam) {
+__global__ void __launch_bounds__(256) eig_norm_kernel(const double* __restrict__ W, EigWs ws, double* lam, int pass) {
   const int mat = blockIdx.y, n = ws.na[mat], ld = ws.n;
   const int c = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   const EigCtl ctl = ws.ctl[mat];
-  if (c == 0 && lane == 0 && !LAST) ws.ctl[mat].mixed = 0;
+  if (c == 0 && lane == 0 && !LAST) {
+    if (pass > 0 && ctl.mixed < 2) ws.ctl[mat].settled = 1;
+    ws.ctl[mat].mixed = 0;
+  }
   if (c >= n || ctl.bad) return;
   const double* w = W + (long long)mat * ld * ld + (long long)c * ld;
   double a = 0.0;
@@ -1553,14 +1574,16 @@ __global__ void __launch_bounds__(256) eig_norm_kernel(const double* __restrict_
 }
 
 // Angles: the Gram matrix of W's columns (upper 32 x 32 tiles), and for every pair that is not
-// orthogonal to 4 n eps the tangent t of its plane rotation, w_p -= t w_q, w_q += t w_p, in M.
-// Angles above 2^-24 are left (first order does not hold): between kept vectors, or across the cut,
-// the groups have taken them.
+// orthogonal to 4 n eps of its norms the tangent t of its plane rotation, w_p -= t w_q, w_q += t w_p, in M.  (Of
+// the larger norm, as in the sweeps, would leave what two small columns have of a large one, and the product of
+// the two would pass for an angle between them: 3e-11 of a vector at 6e-12 lambda_1.)
+// Angles above 2^-9 are left: between kept vectors, or across the cut, the groups have taken them.  So are the
+// vectors below 1e-12 lambda_1, which are rounding: their angles would come back to the others.
 __global__ void __launch_bounds__(256) eig_gram_kernel(const double* __restrict__ W, EigWs ws, double* __restrict__ M) {
   constexpr int BK = 16;
   __shared__ double As[BK][33], Bs[BK][33];
   const int mat = blockIdx.z, n = ws.na[mat], ld = ws.n, q0 = blockIdx.x * 32, p0 = blockIdx.y * 32;
-  if (q0 >= n || p0 > q0 || ws.ctl[mat].bad) return;
+  if (q0 >= n || p0 > q0 || ws.ctl[mat].bad || ws.ctl[mat].settled) return;
   const long long o = (long long)mat * ld * ld;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
   double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
@@ -1585,8 +1608,9 @@ __global__ void __launch_bounds__(256) eig_gram_kernel(const double* __restrict_
   const double* nrm = ws.dk + mat * ld;
   const double tol = 4.0 * n * kEps;
   const int first = n - ws.keep[mat];   // pairs of two vectors behind the kept ones stay
+  const double line = 1e-24 * nrm[n - 1];
   const int *cls = ws.cls + mat * ld, *lost = ws.lost + mat * ld;
-  bool any = false;
+  int any = 0;
 #pragma unroll
   for (int u = 0; u < 2; ++u)
 #pragma unroll
@@ -1596,34 +1620,34 @@ __global__ void __launch_bounds__(256) eig_gram_kernel(const double* __restrict_
       double t = 0.0;
       if (p < q) {
         const double a = nrm[p], b = nrm[q], g = acc[u][v], big = fmax(a, b);
-        // squares below 1e-30 lie under any floor: the scaled matrix has lambda_1 of order 1
-        if (q >= first && big > 1e-30 && fabs(g) > tol * big &&
+        if (q >= first && big > line && fabs(g) > tol * sqrt(a) * sqrt(b) &&
             !turn_forbidden(cls[p], lost[p] != 0, cls[q], lost[q] != 0)) {
           const double zeta = (b - a) / (2.0 * g);
           t = copysign(1.0, zeta) / (fabs(zeta) + sqrt(fma(zeta, zeta, 1.0)));
-          if (fabs(t) > 5.9604644775390625e-8) t = 0.0;
-          if (t != 0.0) {
-            any = true;
-          }
+          if (fabs(t) > 0.001953125) t = 0.0;
+          if (t != 0.0) any = max(any, fabs(t) > 0.000244140625 ? 3 : fabs(t) > 5.9604644775390625e-8 ? 2 : 1);
         }
       }
       M[o + (long long)p * ld + q] = -t;
       M[o + (long long)q * ld + p] = t;
     }
-  if (any) ws.ctl[mat].mixed = 1;
+  if (any) atomicMax(&ws.ctl[mat].mixed, any);
 }
 
-// V and W take the turned columns
-__global__ void __launch_bounds__(256) eig_take_kernel(EigWs ws, const double* __restrict__ Vn,
-                                                       const double* __restrict__ Wn, double* V, double* W) {
+// V and W take the turned columns, of the highest order that was formed
+__global__ void __launch_bounds__(256) eig_take_kernel(EigWs ws, EigPair first, EigPair second, EigPair third, EigPair to,
+                                                       int most) {
   const int mat = blockIdx.y, n = ws.na[mat], ld = ws.n;
   const EigCtl ctl = ws.ctl[mat];
   const int c = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (c >= n || ctl.bad || !ctl.mixed) return;
   const long long o = (long long)mat * ld * ld + (long long)c * ld;
+  const int order = min(ctl.mixed, most);
+  const double* v = order > 2 ? third.p[0] : order > 1 ? second.p[0] : first.p[0];
+  const double* w = order > 2 ? third.p[1] : order > 1 ? second.p[1] : first.p[1];
   for (int i = lane; i < n; i += 32) {
-    V[o + i] = Vn[o + i];
-    W[o + i] = Wn[o + i];
+    to.p[0][o + i] = v[o + i];
+    to.p[1][o + i] = w[o + i];
   }
 }
 
@@ -1739,6 +1763,8 @@ size_t eig_layout(char* base, int n, int nmat, EigWs* w, int** pos) {
   w->q0 = dbl(nn);
   w->q1 = dbl(nn);
   w->ap = dbl(nn);
+  w->w2 = dbl(nn);
+  w->w3 = dbl(nn);
   w->s = dbl((size_t)(n + 16) * n * nmat);   // also the rows of a reduction that exceeds shared memory
   w->tf = dbl((size_t)((n + kRb - 1) / kRb) * kRb * kRb * nmat);
   for (double** p : {&w->d, &w->e, &w->tau, &w->ev0, &w->ev1, &w->dk, &w->zk, &w->zh, &w->val, &w->rc, &w->rs})
@@ -1806,9 +1832,9 @@ size_t eig_workspace_bytes(int n, int nmat) {
 }
 
 // V (rows: eigenvectors) and lam of nmat symmetric matrices of orders na[] <= n, with leading
-// dimension n; keep[]: the leading eigenvectors that may be kept; swp [nmat][n]: the partner of every index under the exchange of hat and check;
+// dimension n; A is overwritten; keep[]: the leading eigenvectors that may be kept; swp [nmat][n]: the partner of every index under the exchange of hat and check;
 // iters: one word per matrix
-int launch_eig(const double* A, int n, int nmat, const int* na, const int* keep, const int* swp, void* work, double* V,
+int launch_eig(double* A, int n, int nmat, const int* na, const int* keep, const int* swp, void* work, double* V,
                double* lam, int* cls, int* iters, DevState* st, cudaStream_t s) {
   if (n < 1 || n > kEigMaxN || nmat < 1 || nmat > kEigMaxMat) return -1;
   EigWs w;
@@ -1888,21 +1914,24 @@ int launch_eig(const double* A, int n, int nmat, const int* na, const int* keep,
   }
   eig_back_kernel<<<dim3((n + kStrip - 1) / kStrip, nmat), 256, smem, s>>>(w, q, ev, w.tf, nblk, V, lam);
   ++g_launches;
-  // W = A V, the close groups, then the tiny angles twice (they come out quadratically)
+  // W = A V, the close groups, then the small angles
   const int tn = (n + 31) / 32;
-  const dim3 tiles(tn, tn, nmat);
-  double *W = w.q0, *M = w.s, *Vn = w.q1, *Wn = w.ap;   // free by now
-  eig_nn_kernel<false><<<tiles, 256, 0, s>>>(V, A, w, W);
+  const dim3 tiles(tn, tn, nmat), both(tn, tn, 2 * nmat);
+  double *W = w.q0, *M = w.s;   // free by now, as the buffers of the turned columns are
+  const EigPair cur = {{V, W}}, one = {{w.q1, w.ap}}, two = {{w.vh, w.w2}}, three = {{A, w.w3}}, none = {{nullptr, nullptr}};
+  eig_nn_kernel<EIG_AV><<<tiles, 256, 0, s>>>(V, EigPair{{A, nullptr}}, none, w, EigPair{{W, nullptr}});
   eig_polish_kernel<<<nmat, 256, 0, s>>>(w, V, W, lam);
-  for (int it = 0; it < 2; ++it) {
-    eig_norm_kernel<false><<<rows, 256, 0, s>>>(W, w, lam);
+  for (int pass = 0; pass < 3; ++pass) {
+    eig_norm_kernel<false><<<rows, 256, 0, s>>>(W, w, lam, pass);
     eig_gram_kernel<<<tiles, 256, 0, s>>>(W, w, M);
-    eig_nn_kernel<true><<<tiles, 256, 0, s>>>(M, V, w, Vn);
-    eig_nn_kernel<true><<<tiles, 256, 0, s>>>(M, W, w, Wn);
-    eig_take_kernel<<<rows, 256, 0, s>>>(w, Vn, Wn, V, W);
+    eig_nn_kernel<EIG_FIRST><<<both, 256, 0, s>>>(M, cur, none, w, one);
+    // the second pass has angles up to 2^-18, the third up to 2^-36
+    if (pass < 2) eig_nn_kernel<EIG_SECOND><<<both, 256, 0, s>>>(M, cur, one, w, two);
+    if (pass < 1) eig_nn_kernel<EIG_THIRD><<<both, 256, 0, s>>>(M, one, two, w, three);
+    eig_take_kernel<<<rows, 256, 0, s>>>(w, one, two, three, cur, 3 - pass);
   }
-  eig_norm_kernel<true><<<rows, 256, 0, s>>>(W, w, lam);
-  g_launches += 13;
+  eig_norm_kernel<true><<<rows, 256, 0, s>>>(W, w, lam, 0);
+  g_launches += 18;
   eig_iters_kernel<<<1, 32, 0, s>>>(w, iters);
   ++g_launches;
   return cudaPeekAtLastError() == cudaSuccess ? 0 : -1;
