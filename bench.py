@@ -8,7 +8,7 @@
 Default workload: 3D Ising, d = 3, chi = 16, beta = 0.2216544, h = 0, axes cycling
 z, x, y.  The first steps grow the bonds (2 -> 4 -> 16 for the default) and are not
 timed; then W steady-state warm-up steps and K timed steps, each one full
-coarse-graining (permutation, FP64 environments, Jacobi, choice/truncation, prime
+coarse-graining (permutation, FP64 environments, eigen-solver, choice/truncation, prime
 chain, bottleneck, non-prime chain, trace/normalisation).  The local tensor (134 MB
 FP64 for the default) and the per-slice operands (GBs) exceed the 129 MB L2.
 Per-step ln Z/V is compared with the FP64 oracle's reference values in
@@ -135,7 +135,7 @@ def prec_const(pkg, name):
     return getattr(pkg, PRECISIONS[name][0])
 
 
-FP64_DIGIT_PRODUCTS = 36   # BF16 products of digits in one FP64 product on the tensor cores
+FP64_DIGIT_PRODUCTS = 44   # BF16 products in one FP64 product on the tensor cores: 43 of digits, one for its guard
 
 
 def fp64_peak(pkg):
@@ -276,7 +276,7 @@ def fp64_form_leg(pkg, args, nsteps=2):
     and the FP64 bottleneck rate as a fraction of the rate that bounds it (fp64_peak)."""
     import torch
 
-    peak, _ = fp64_peak(pkg)
+    peak, peak_src = fp64_peak(pkg)
     stream = torch.cuda.current_stream()
     f = pkg.Hotrg(D, BETA, H, precision=pkg.PREC_FP64, z2=args.z2 == "on")
     axes = axes_for(GROWTH_STEPS + nsteps)
@@ -305,8 +305,8 @@ def fp64_form_leg(pkg, args, nsteps=2):
             "steps_per_s": 1000.0 / ms,
             "rel_err_lnz_per_site_vs_oracle": abs(lnz - golden[last]) / abs(golden[last]) if last in golden else None,
             "bottleneck_flops_per_step": done / nsteps,
-            "bottleneck_tflops": achieved, "fp64_peak_tflops_measured": peak,
-            "frac_of_measured_fp64": achieved / peak if achieved else None,
+            "bottleneck_tflops": achieved, "fp64_bound_tflops": peak, "fp64_bound_source": peak_src,
+            "frac_of_fp64_bound": achieved / peak if achieved else None,
             "note": "first steady steps (balanced Z2 blocks); later steps keep more even states and cost more"}
 
 

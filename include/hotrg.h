@@ -23,8 +23,8 @@
  *    that while a derivative is carried it waits for the per-leg choices.
  *    The read-back calls (hotrg_free_energy, hotrg_observables,
  *    hotrg_isometry, hotrg_spectrum, hotrg_tensor) synchronise that stream.
- *  - Device-side failures (a non-positive or non-finite trace, a Jacobi
- *    sweep cap, a bounded wait that expired) are recorded in a device status
+ *  - Device-side failures (a non-positive or non-finite trace, the eigen-
+ *    solver's iteration cap, a bounded wait that expired) are recorded in a device status
  *    word and returned by the next read-back call.  After any failure other
  *    than HOTRG_EINVAL the context is poisoned: further calls return
  *    HOTRG_ESTATE until it is freed.
@@ -53,7 +53,7 @@ enum hotrg_status {
   HOTRG_ENOMEM = -2,    /* device allocation failed */
   HOTRG_ECUDA = -3,     /* a CUDA runtime or driver call failed */
   HOTRG_ENUMERIC = -4,  /* trace of a new tensor <= 0 or not finite */
-  HOTRG_ENOTCONV = -5,  /* Jacobi eigen-solver hit its sweep cap */
+  HOTRG_ENOTCONV = -5,  /* the eigen-solver hit its iteration cap */
   HOTRG_ETIMEOUT = -6,  /* a bounded device-side wait expired */
   HOTRG_ESTATE = -7     /* context poisoned by an earlier failure, or no step yet */
 };
@@ -185,11 +185,10 @@ int hotrg_bottleneck_flops(hotrg_ctx* ctx, double* dense, double* performed, int
  * hotrg_step_times() call (enable = 2: no per-step read-back needed), or stop
  * (0).  hotrg_step_times() then returns, after synchronising, the
  * milliseconds of the last step (enable = 1) per phase: [0] leg permutation, [1]
- * environment Grams and A assembly, [2] Jacobi, [3] choice/truncation,
+ * environment Grams and A assembly, [2] eigen-solver, [3] choice/truncation,
  * [4] BF16 split of T, [5] prime-side chain, [6] bottleneck GEMM, [7]
- * non-prime chain, [8] trace / normalisation, [9] FP32 warm start of the
- * eigen-solver (included in [2]), [10] its FP32 sweeps (included in [9]),
- * [11] gathers and scatters of the Z2 block form; *n = 12.  launches[k] =
+ * non-prime chain, [8] trace / normalisation, [9] and [10] no longer recorded
+ * (zero), [11] gathers and scatters of the Z2 block form; *n = 12.  launches[k] =
  * number of timed regions of phase k (the bottleneck: one GEMM launch per
  * c'-slice and n'_1 sub-range, two with the Z2 block form).
  * *contraction_fp64 = 1 if the last step's contraction ran in FP64. */
@@ -430,9 +429,10 @@ int hotrg_gemm_rate(int mode, int M, int N, int K, int iters, double* ms_per_lau
 
 /* FP64 fused multiply-add rate of the current device, in TFLOP/s (2 flops per
  * FMA): independent FMA chains on every SM, timed with CUDA events (best of
- * two launches after one warm-up).  The denominator of the FP64 kernels'
- * roofline (environment Grams, eigen-solver, the FP64 form of the
- * contraction); the paper has no counterpart.  Synchronous on the legacy
+ * two launches after one warm-up).  The denominator of the roofline of what
+ * runs on the FP64 pipe (eigen-solver, FP64 chains, small FP64 products; large
+ * ones are bounded by the tensor cores, HOTRG_PREC_FP64); the paper has no
+ * counterpart.  Synchronous on the legacy
  * default stream; allocates 8 bytes per CTA for its outputs.
  * Errors: EINVAL, ENOMEM, ECUDA. */
 int hotrg_fp64_rate(double* tflops);

@@ -1579,7 +1579,7 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
   // The dense split form (d >= 3) runs as one block that holds every index: the chain stages of the block
   // form serve it too, with a K order that they like (the last hat index slowest, from its end).  Per step, 3D chi = 12
   // with a field: prime 2.26 -> 1.71 ms, non-prime 1.46 -> 1.14; 3D chi = 13 split TF32, 4 slices, 8.9 -> 7.5 ms
-  const bool one_block = !z2 && !fp64 && !tangent && !c->f64_chains && d >= 3 && chij[d - 1] <= 32;
+  const bool one_block = !z2 && !fp64 && !tangent && !c->f64_chains && d >= 3;
   const bool blocks = z2 || one_block;
   // Z2 index maps.  Rows of T and the contracted index (rho, n^') run over the same
   // slots with the same parities, so one list per parity b serves as the row map
@@ -1970,7 +1970,7 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
           zo.r_magic = (unsigned)((((1ULL << l) - (unsigned long long)R) << 32) / (unsigned long long)R + 1);
         }
         tuned_chain(c, cd, 1, [&] {
-          if (d >= 3 && chij[j] <= 32 && !src_f64) {
+          if (d >= 3 && !src_f64) {
             Z2Blocks zb = {zo.cblk, zo.cpos, zo.q, {zo.blk[0], zo.blk[1]}, {zo.ld[0], zo.ld[1]},
                            {zo.pstride[0], zo.pstride[1]}, npieces};
             if (launch_z2_prime(last_leg, (const float*)src, (int)(P / chij[j]), chi_c, (int)P, Nc / nsz[j], zo.kcat,
@@ -2189,7 +2189,7 @@ int step_impl(hotrg_ctx* c, int axis, int chi, const Shard& sh) {
         zi.c[1] = (const float*)cblk_cur[1];
         zi.ld = ldz;
         tuned_chain(c, cd, 2, [&] {
-          if (d >= 3 && chij[j] <= 32 &&
+          if (d >= 3 &&
               launch_z2_nonprime(last_leg, zi, R / chij[j], Nc / chij[j], (float*)dst, cd.ctas_per_sm, s))
             return;
           launch_chain_f32_z2in(cd, zi, (const float*)c->U32.p + u_off[j], dst, last ? OUT_F64 : OUT_F32, s);

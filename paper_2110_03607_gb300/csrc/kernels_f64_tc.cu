@@ -30,7 +30,9 @@
 // that small, a tenth to two thirds do: there the digits lost up to all of an entry's own figures.
 //
 // Layout: tile 128 x 48 of C per CTA, its ten accumulators fill 480 of the 512 columns of TMEM.  A ring of
-// two stages holds K slabs of 32 (64-byte rows), all nine planes of both operands (99 KB a stage).
+// two stages holds K slabs of 32 (64-byte rows), all nine planes of both operands (99 KB a stage).  44 products of
+// 48 columns; with eight accumulators of 64 columns (36 products, entries unguarded) the FP64 products of a 3D step,
+// bonds 9 x 11 x 10, took 12.8 ms with their slicing, so 22.4.
 // The MMA warp goes through a slab by accumulator g, and waits for the epilogue once per g and chunk,
 // so the drain of one accumulator runs under the MMAs of the next.
 #include <stdio.h>
@@ -509,20 +511,35 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   }
 }
 
-// S[0] += the sums of the other splits
+// S[0] = the sum over the splits: 32 entries a block, each by eight threads (a thread per entry waits for one load
+// after another: 12.5 us for 128 x 128 in 64 splits, 4.3 so)
 __global__ void __launch_bounds__(256) f64_sum_kernel(float* S, long long plane, int nsplit) {
-  for (long long i = (long long)blockIdx.x * 256 + threadIdx.x; i < plane; i += (long long)gridDim.x * 256) {
-    float s = S[i];
-#pragma unroll 8
-    for (int z = 1; z < nsplit; ++z) s += S[z * plane + i];
-    S[i] = s;
+  __shared__ float part[8][33];
+  const int lane = threadIdx.x & 31, y = threadIdx.x >> 5;
+  for (long long i0 = (long long)blockIdx.x * 32; i0 < plane; i0 += (long long)gridDim.x * 32) {
+    const long long i = i0 + lane;
+    float s = 0.0f;
+    if (i < plane) {
+#pragma unroll 4
+      for (int z = y; z < nsplit; z += 8) s += S[z * plane + i];
+    }
+    part[y][lane] = s;
+    __syncthreads();
+    if (y == 0 && i < plane) {
+#pragma unroll
+      for (int q = 1; q < 8; ++q) s += part[q][lane];
+      S[i] = s;
+    }
+    __syncthreads();
   }
 }
 
 // The entries that the digits do not give as well as an FP64 sum, from the operands themselves: a warp
 // sums up to four entries of a row at a time, in 32 chains and a tree, each by itself, so that an entry's bits
 // do not depend on which others failed.  A 64 x 64 tile and one split per CTA.  Where nothing failed this reads
-// S; where all did the FP64 pipe bounds it, as it does gemm_nt_f64_kernel.
+// S: 30 us for 990 x 16,270, behind 2.3 ms of products, 9 us for 128 x 128 in 64 splits; where all did the FP64 pipe
+// bounds it, as it does gemm_nt_f64_kernel.  (A thread for each entry, and the whole tile where an eighth of it
+// failed: 0.8 ms more for the first, whose few entries then took a chain of 990 multiply-adds each.)
 __global__ void __launch_bounds__(256)
     f64_fix_kernel(const double* __restrict__ A, long long lda, const double* __restrict__ B, long long ldb,
                    double* __restrict__ C, long long ldc, long long split_stride, int M, int N, long long K,
@@ -815,7 +832,7 @@ int launch_gemm_nt_f64_tc(const double* A, long long lda, const double* B, long 
         ++g_launches;
         if (it.nsplit > 1) {
           const long long plane = (long long)mc * nc;
-          f64_sum_kernel<<<(unsigned)std::min((plane + 255) / 256, 8 * sms), 256, 0, s>>>(sums, plane, it.nsplit);
+          f64_sum_kernel<<<(unsigned)std::min((plane + 31) / 32, 64 * sms), 256, 0, s>>>(sums, plane, it.nsplit);
           ++g_launches;
         }
         const int ft = (mc + 63) / 64;
