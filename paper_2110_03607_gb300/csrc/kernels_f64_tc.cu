@@ -536,85 +536,82 @@ __global__ void __launch_bounds__(256) f64_sum_kernel(float* S, long long plane,
 
 // The entries that the digits do not give as well as an FP64 sum, from the operands themselves: a warp
 // sums up to four entries of a row at a time, in 32 chains and a tree, each by itself, so that an entry's bits
-// do not depend on which others failed.  A 64 x 64 tile and one split per CTA.  Where nothing failed this reads
-// S: 30 us for 990 x 16,270, behind 2.3 ms of products, 9 us for 128 x 128 in 64 splits; where all did the FP64 pipe
-// bounds it, as it does gemm_nt_f64_kernel.  (A thread for each entry, and the whole tile where an eighth of it
-// failed: 0.8 ms more for the first, whose few entries then took a chain of 990 multiply-adds each.)
+// do not depend on which others failed.  A tile of 16 x 64 and one split per CTA.  Where nothing failed this
+// reads S: 41 us for 990 x 16,270, behind 2.3 ms of products, 5 us for 128 x 128 in 64 splits.  Where all did the
+// FP64 pipe bounds it as it does gemm_nt_f64_kernel: 600 x 1800 x 1800 4.4 ms in all, 3.1 at the pipe's full rate.
+// (Tiles of 64 x 64 left SMs without one: 7.2 ms; their code unrolled over the rows, 10 us for the 128 x 128.)
+constexpr int FIX_M = 16, FIX_N = 64;
 __global__ void __launch_bounds__(256)
     f64_fix_kernel(const double* __restrict__ A, long long lda, const double* __restrict__ B, long long ldb,
                    double* __restrict__ C, long long ldc, long long split_stride, int M, int N, long long K,
                    long long per, const float* __restrict__ S, const unsigned long long* __restrict__ qa,
                    const int* __restrict__ ea, const unsigned long long* __restrict__ qb, const int* __restrict__ eb,
                    int upper) {
-  constexpr int T = 64;
-  __shared__ float na[T], nb[T];            // 2^-9 |alpha|; infinite for a row that is not finite
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  int bx = blockIdx.x, by = blockIdx.y;
-  if (upper) {
-    const int nt = (M + T - 1) / T;
-    int t = blockIdx.x, ti = 0;
-    while (t >= nt - ti) {
-      t -= nt - ti;
-      ++ti;
-    }
-    by = ti;
-    bx = ti + t;
-  }
-  const int m0 = by * T, n0 = bx * T;
-  if (tid < 2 * T) {
-    const bool second = tid >= T;
-    const int i = tid & (T - 1), r = (second ? n0 : m0) + i;
-    float v = 0.0f;
-    if (r < (second ? N : M))
-      v = (second ? eb : ea)[r] == NON_FINITE
-              ? __int_as_float(0x7f800000)
-              : kTrust * 3.0517578125e-5f * sqrtf((float)(second ? qb : qa)[r]);   // 2^-15 sqrt(q)
-    (second ? nb : na)[i] = v;
-  }
-  __syncthreads();
-  // this warp's 32 columns of 16 rows
-  const int j0 = (warp & 1) * 32, c = n0 + j0 + lane;
-  const float line_c = nb[j0 + lane];
-  float s[16];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  // this warp's 32 columns of 4 rows
+  const int r0 = blockIdx.y * FIX_M + (warp >> 1) * 4, c0 = blockIdx.x * FIX_N + (warp & 1) * 32, c = c0 + lane;
+  if (r0 >= M || c0 >= N || (upper && c0 + 31 < r0)) return;
+  // 2^-9 |alpha|; infinite for a row that is not finite
+  auto line_of = [](const unsigned long long* q, const int* e, int r) {
+    return e[r] == NON_FINITE ? __int_as_float(0x7f800000)
+                              : kTrust * 3.0517578125e-5f * sqrtf((float)q[r]);   // 2^-15 sqrt(q)
+  };
+  float s[4];
 #pragma unroll
-  for (int u = 0; u < 16; ++u) {
-    const int r = m0 + (warp >> 1) + 4 * u;
-    s[u] = r < M && c < N ? S[(long long)r * N + c] : 0.0f;
-  }
-  const long long k_lo = (long long)blockIdx.z * per, k_hi = k_lo + per < K ? k_lo + per : K;
-  double* Cz = C + (long long)blockIdx.z * split_stride;
+  for (int u = 0; u < 4; ++u) s[u] = r0 + u < M && c < N ? S[(long long)(r0 + u) * N + c] : 0.0f;
+  const float line_c = c < N ? line_of(qb, eb, c) : 0.0f;
+  unsigned mine = 0u;   // lane u: the entries of row u to form
 #pragma unroll
-  for (int u = 0; u < 16; ++u) {
-    const int i = (warp >> 1) + 4 * u, r = m0 + i;
-    const float line = na[i] + line_c;
+  for (int u = 0; u < 4; ++u) {
+    const int r = r0 + u;
+    const float line = line_c + (r < M ? line_of(qa, ea, r) : 0.0f);
     // a sum of exact zeros needs nothing; an infinite line is never reached
     const bool good = s[u] >= line || (s[u] == 0.0f && line < __int_as_float(0x7f800000));
-    unsigned todo = __ballot_sync(0xffffffffu, r < M && c < N && !(upper && c < r) && !good);
+    const unsigned todo = __ballot_sync(0xffffffffu, r < M && c < N && !(upper && c < r) && !good);
+    if (lane == u) mine = todo;
+  }
+  unsigned rows = __ballot_sync(0xffffffffu, mine != 0u);
+  const long long k_lo = (long long)blockIdx.z * per, k_hi = k_lo + per < K ? k_lo + per : K;
+  double* Cz = C + (long long)blockIdx.z * split_stride;
+#pragma unroll 1
+  for (; rows != 0u; rows &= rows - 1u) {
+    const int u = __ffs(rows) - 1;
+    unsigned todo = __shfl_sync(0xffffffffu, mine, u);
+    const double* a = A + (long long)(r0 + u) * lda;
+#pragma unroll 1
     while (todo != 0u) {
       int col[4], cnt = 0;
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
-        col[q] = n0 + j0;
+        col[q] = c0;
         if (todo != 0u) {
           col[q] += __ffs(todo) - 1;
           todo &= todo - 1u;
           cnt = q + 1;
         }
       }
-      const double* a = A + (long long)r * lda;
       double acc[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll 4
       for (long long k = k_lo + lane; k < k_hi; k += 32) {
         const double x = a[k];
 #pragma unroll
         for (int q = 0; q < 4; ++q)
           if (q < cnt) acc[q] = fma(x, B[(long long)col[q] * ldb + k], acc[q]);
       }
+      // the four sums over the lanes: halves are exchanged while there is more than one value a lane, the
+      // same tree for each; lanes 8 q end with sum q
+      const bool h4 = (lane & 16) != 0, h3 = (lane & 8) != 0;
+      double x0 = h4 ? acc[2] : acc[0], x1 = h4 ? acc[3] : acc[1];
+      x0 += __shfl_xor_sync(0xffffffffu, h4 ? acc[0] : acc[2], 16);
+      x1 += __shfl_xor_sync(0xffffffffu, h4 ? acc[1] : acc[3], 16);
+      double x = h3 ? x1 : x0;
+      x += __shfl_xor_sync(0xffffffffu, h3 ? x0 : x1, 8);
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        if (q >= cnt) break;
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc[q] += __shfl_xor_sync(0xffffffffu, acc[q], o);
-        if (lane == 0) Cz[(long long)r * ldc + col[q]] = acc[q];
+      for (int o = 4; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+      const int q = lane >> 3;
+      if ((lane & 7) == 0 && q < cnt) {
+        const int to = q == 0 ? col[0] : q == 1 ? col[1] : q == 2 ? col[2] : col[3];
+        Cz[(long long)(r0 + u) * ldc + to] = x;
       }
     }
   }
@@ -835,8 +832,7 @@ int launch_gemm_nt_f64_tc(const double* A, long long lda, const double* B, long 
           f64_sum_kernel<<<(unsigned)std::min((plane + 31) / 32, 64 * sms), 256, 0, s>>>(sums, plane, it.nsplit);
           ++g_launches;
         }
-        const int ft = (mc + 63) / 64;
-        const dim3 grid = upper_only ? dim3(ft * (ft + 1) / 2, 1, it.nsplit) : dim3((nc + 63) / 64, ft, it.nsplit);
+        const dim3 grid((nc + FIX_N - 1) / FIX_N, (mc + FIX_M - 1) / FIX_M, it.nsplit);
         f64_fix_kernel<<<grid, 256, 0, s>>>(a.x, lda, b.x, ldb, Cp, ldc, split_stride, mc, nc, Kp,
                                             (long long)it.per * TK, sums, a.q, a.e, b.q, b.e, upper_only);
         ++g_launches;
