@@ -144,10 +144,7 @@ int launch_gemm_nt_f64(const double* A, long long lda, const double* B, long lon
   return nsplit;
 }
 
-// Batched small FP64 products for the Newton-Schulz re-orthonormalisation in the
-// eigen-solver: C_b = A_b . op(B_b), op(B) = B^T (B_N = false: B rows are K-contiguous)
-// or B (B_N = true: B[k][j], j contiguous).  64 x 64 tiles, 4 x 4 per thread.
-template <bool B_N>
+// Small FP64 products C_b = A_b B_b (B[k][j], j contiguous): 64 x 64 tiles, 4 x 4 per thread.
 __global__ void __launch_bounds__(256) gemm_small_f64_kernel(
     const double* __restrict__ A, long long lda, const double* __restrict__ B, long long ldb,
     double* __restrict__ C, long long ldc, int M, int N, int K, long long bsa, long long bsb,
@@ -172,14 +169,9 @@ __global__ void __launch_bounds__(256) gemm_small_f64_kernel(
       int k = k0 + lk + u;
       int ra = m0 + lr;
       As[lk + u][lr] = (ra < M && k < K) ? A[(long long)ra * lda + k] : 0.0;
-      if (!B_N) {
-        int rb = n0 + lr;
-        Bs[lk + u][lr] = (rb < N && k < K) ? B[(long long)rb * ldb + k] : 0.0;
-      } else {
-        int kk = tid >> 4, col = (tid & 15) * 4 + u;
-        int kb = k0 + kk;
-        Bs[kk][col] = (kb < K && n0 + col < N) ? B[(long long)kb * ldb + n0 + col] : 0.0;
-      }
+      int kk = tid >> 4, col = (tid & 15) * 4 + u;
+      int kb = k0 + kk;
+      Bs[kk][col] = (kb < K && n0 + col < N) ? B[(long long)kb * ldb + n0 + col] : 0.0;
     }
     __syncthreads();
 #pragma unroll
@@ -212,15 +204,7 @@ void launch_gemm_nn_f64(const double* A, long long lda, const double* B, long lo
                         long long ldc, int M, int N, int K, int batch, long long bsa, long long bsb,
                         long long bsc, cudaStream_t s) {
   dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM, batch);
-  gemm_small_f64_kernel<true><<<grid, 256, 0, s>>>(A, lda, B, ldb, C, ldc, M, N, K, bsa, bsb, bsc);
-  ++g_launches;
-}
-
-void launch_gemm_nt_f64_batched(const double* A, long long lda, const double* B, long long ldb,
-                                double* C, long long ldc, int M, int N, int K, int batch,
-                                long long bsa, long long bsb, long long bsc, cudaStream_t s) {
-  dim3 grid((N + BN - 1) / BN, (M + BM - 1) / BM, batch);
-  gemm_small_f64_kernel<false><<<grid, 256, 0, s>>>(A, lda, B, ldb, C, ldc, M, N, K, bsa, bsb, bsc);
+  gemm_small_f64_kernel<<<grid, 256, 0, s>>>(A, lda, B, ldb, C, ldc, M, N, K, bsa, bsb, bsc);
   ++g_launches;
 }
 
